@@ -337,6 +337,14 @@ struct NoPre {
 // step 1 (thread = (c, n2)): DFT_R1 over x[R2 n1 + n2] (each value passed
 // through pre() as it is loaded), times w_L^(n2 k1), intermediate at
 // n2 (R1 + 1) + k1; step 2 (thread = (c, k1)): DFT_R2 gives X[k1 + R1 k2].
+// w1 holds w_L^(n2 k1) at w1[k1 R2 + n2] (k1 >= 1; row_twiddle<L> gives the
+// entry): consecutive lanes read consecutive entries.  Read from the table
+// exp(-2 pi i m / T) instead, at m = n2 k1 T / L, the lanes of one load sit
+// k1 T / L entries apart, up to 16 lanes on one bank pair, which took a third
+// of the shared-memory wavefronts of the row passes (ncu, 512-point rows: r2c
+// 24 per point and warp, LSU pipe 81 % busy).  At 512^3 / 1024^3 (ms): x r2c
+// 1.86 -> 1.61, screening x 3.83 -> 3.45, force x c2r 5.20 -> 4.42, LPT x
+// 1.17 -> 1.01.
 // PAIR32: for L = 16 x 32 with half as many step-2 items as threads, step 2
 // runs on thread pairs (dft32_pair), halving its registers per thread.
 // The caller synchronises before the call; returns after a barrier.
@@ -348,9 +356,16 @@ struct RowStore {
   __device__ __forceinline__ float2 operator()(float2 v, int, int) const { return v; }
 };
 
-template <int L, int TW, int CW, int NT, bool INV, int TWS = 1, class Pre = NoPre, bool PAIR32 = false,
+// Index m (of exp(-2 pi i m / L)) of entry i = k1 R2 + n2 of a row transform's
+// first-step twiddles.
+template <int L>
+__host__ __device__ constexpr int row_twiddle(int i) {
+  return (i / Split<L>::R2) * (i % Split<L>::R2);
+}
+
+template <int L, int TW, int CW, int NT, bool INV, class Pre = NoPre, bool PAIR32 = false,
           class Store = RowStore>
-__device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const float2* __restrict__ tw,
+__device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const float2* __restrict__ w1,
                                             Pre pre = Pre(), Store st = Store()) {
   constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;
   constexpr int U1 = TW * R2, P1 = (U1 + NT - 1) / NT;
@@ -371,7 +386,7 @@ __device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const floa
         if (n2 > 0) {
 #pragma unroll
           for (int k1 = 1; k1 < R1; ++k1) {
-            float2 w = tw[n2 * k1 * TWS];
+            float2 w = w1[k1 * R2 + n2];
             if (INV) w.y = -w.y;
             v[i][k1] = cmul(v[i][k1], w);
           }
@@ -439,11 +454,11 @@ __device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const floa
   __syncthreads();
 }
 
-template <int L, int TW, int CW, int NT, bool INV, int TWS = 1, class Pre = NoPre, bool PAIR32 = false,
+template <int L, int TW, int CW, int NT, bool INV, class Pre = NoPre, bool PAIR32 = false,
           class Store = RowStore>
-__device__ __noinline__ void fft_rowtile_call(float2* buf, const float2* tw, Pre pre = Pre(),
+__device__ __noinline__ void fft_rowtile_call(float2* buf, const float2* w1, Pre pre = Pre(),
                                               Store st = Store()) {
-  fft_rowtile<L, TW, CW, NT, INV, TWS, Pre, PAIR32, Store>(buf, tw, pre, st);
+  fft_rowtile<L, TW, CW, NT, INV, Pre, PAIR32, Store>(buf, w1, pre, st);
 }
 
 // Out-of-line copy for kernels that run several transforms per tile: each

@@ -134,6 +134,19 @@ __device__ __forceinline__ void load_tw(float2* tw, const float2* __restrict__ t
   for (int i = threadIdx.x; i < n; i += NT) tw[i] = twg[i];
 }
 
+// Twiddles of an x pass over rows of N reals (M = N/2 complex): entries 0..M the
+// table exp(-2 pi i k / N) of the real <-> half-spectrum split, entry M + k1 R2 + n2
+// (k1 >= 1) the row transform's first-step twiddle (fft_rowtile), which therefore
+// takes w1 = tw + M.  Together they fill the N entries of the plain table.
+template <int N>
+__device__ __forceinline__ void load_row_tw(float2* tw, const float2* __restrict__ twg) {
+  constexpr int M = N / 2;
+  for (int i = threadIdx.x; i < N; i += NT) {
+    const int j = i - M;
+    if (i <= M || j >= Split<M>::R2) tw[i] = twg[i <= M ? i : 2 * row_twiddle<M>(j)];
+  }
+}
+
 // ---------------------------------------------------------------- cp.async helpers
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool valid) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
@@ -1467,7 +1480,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xr2c(const float* 
       fence_bar_init();
       fail = 0;
     }
-    load_tw(tw, twg, N);
+    load_row_tw<N>(tw, twg);
     __syncthreads();
     uint32_t par = 0, pend = 0;
     int64_t t = blockIdx.x;
@@ -1495,7 +1508,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xr2c(const float* 
       __syncthreads();
       if (fail) break;
       float2* buf = cur ? st1 : st0;
-      fft_rowtile<M, TWX, C::CW, NT, false, 2>(buf, tw, ScaleOffset{scale, offset});
+      fft_rowtile<M, TWX, C::CW, NT, false>(buf, tw + M, ScaleOffset{scale, offset});
       row_r2c_store<N, TWX>(buf, tw, out, row_tile<N, TWX>(t, m).row0);
       __syncthreads();
       cur ^= 1;
@@ -1507,7 +1520,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xr2c(const float* 
     }
     return;
   }
-  load_tw(tw, twg, N);
+  load_row_tw<N>(tw, twg);
   int64_t t = blockIdx.x;
   if (t < ntiles) {
     const RowTile r = row_tile<N, TWX>(t, m);
@@ -1525,7 +1538,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xr2c(const float* 
     cp_async_wait<1>();
     __syncthreads();
     float2* buf = cur ? st1 : st0;
-    fft_rowtile<M, TWX, C::CW, NT, false, 2>(buf, tw, ScaleOffset{scale, offset});
+    fft_rowtile<M, TWX, C::CW, NT, false>(buf, tw + M, ScaleOffset{scale, offset});
     const RowTile r = row_tile<N, TWX>(t, m);
     row_r2c_store<N, TWX>(buf, tw, moved(out, r.by), r.row0);
     __syncthreads();
@@ -1628,7 +1641,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r(const __grid_
   float2* tw = sm;
   float2* st0 = sm + N;
   float2* st1 = st0 + C::stage;
-  load_tw(tw, twg, N);
+  load_row_tw<N>(tw, twg);
   const int64_t ntiles = tiles_per_job * jobs.njobs * m.nb;
   int64_t t = blockIdx.x;
   if (t < ntiles) {
@@ -1663,7 +1676,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r(const __grid_
       float* out = moved(static_cast<float*>(jobs.out[j.job]), j.by);
       const RealRowOut<M> o{reinterpret_cast<float2*>(out + real_row_q(j.row0, N) * N),
                             reinterpret_cast<float2*>(out + real_row_q(j.row0 + 1, N) * N)};
-      fft_rowtile<M, TWX, C::CW, NT, true, 2, Pre, false, RealRowOut<M>>(buf, tw, pre, o);
+      fft_rowtile<M, TWX, C::CW, NT, true, Pre, false, RealRowOut<M>>(buf, tw + M, pre, o);
     } else {
       const SimHeader* h = moved(jobs.hdr, j.by);
       if (j.q != run_q) {  // the same for every thread of the CTA
@@ -1677,7 +1690,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r(const __grid_
       float tile_max = 0.f;
       const RealRowOut16<M, OUT> o{out + real_row_q(j.row0, N) * M, out + real_row_q(j.row0 + 1, N) * M,
                                    1.f / h->lq_scale[j.job], &tile_max};
-      fft_rowtile<M, TWX, C::CW, NT, true, 2, Pre, false, RealRowOut16<M, OUT>>(buf, tw, pre, o);
+      fft_rowtile<M, TWX, C::CW, NT, true, Pre, false, RealRowOut16<M, OUT>>(buf, tw + M, pre, o);
       run_max = fmaxf(run_max, tile_max);
     }
     __syncthreads();
@@ -1733,7 +1746,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r_pair(
   float2* tw = sm;
   float2* st0 = sm + N;
   float2* st1 = st0 + C::stage;
-  load_tw(tw, twg, N);
+  load_row_tw<N>(tw, twg);
   const int64_t ntiles = tiles_per_sim * m.nb;
   auto tile = [&](int64_t t, int64_t& q0, int64_t& by) {
     const int64_t s = t / tiles_per_sim;
@@ -1763,8 +1776,8 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r_pair(
     float2* buf = cur ? st1 : st0;
     float2* o = moved(out, by);
     const PairRowOut<N, R1> st{o + real_row_q(q0, N) * N, o + real_row_q(q0 + 1, N) * N};
-    fft_rowtile<M, TWX, C::CW, NT, true, 2, C2rCombine2<N, C::CW>, false, PairRowOut<N, R1>>(
-        buf, tw, C2rCombine2<N, C::CW>{buf, tw, kfs, 0.f}, st);
+    fft_rowtile<M, TWX, C::CW, NT, true, C2rCombine2<N, C::CW>, false, PairRowOut<N, R1>>(
+        buf, tw + M, C2rCombine2<N, C::CW>{buf, tw, kfs, 0.f}, st);
     __syncthreads();
     cur ^= 1;
   }
@@ -1837,7 +1850,7 @@ __global__ void __launch_bounds__(NT, 2) k_x_screen(const float2* __restrict__ w
   float2* tw = sm;
   float2* st0 = sm + N;
   float2* st1 = st0 + C::stage;
-  load_tw(tw, twg, N);
+  load_row_tw<N>(tw, twg);
   int64_t t = blockIdx.x;
   if (t < ntiles) {
     const RowTile r = row_tile<N, TWX>(t, m);
@@ -1860,14 +1873,14 @@ __global__ void __launch_bounds__(NT, 2) k_x_screen(const float2* __restrict__ w
       stage_complex_rows<N, TWX>(cur ? st0 : st1, moved(w_in, rn.by), rn.row0);
     }
     cp_async_commit();
-    fft_rowtile_call<M, TWX, C::CW, NT, true, 2, C2rCombine<N, C::CW>, true>(buf, tw,
+    fft_rowtile_call<M, TWX, C::CW, NT, true, C2rCombine<N, C::CW>, true>(buf, tw + M,
                                                                            C2rCombine<N, C::CW>{buf, tw, 0.f});
     // S = delta eps(w) is formed as the forward transform loads it
     const float* rho_t = moved(rho, r.by);
     const ScreenSourceRows<M, MODEL> src{reinterpret_cast<const float2*>(rho_t + real_row_q(row0, N) * N),
                                          reinterpret_cast<const float2*>(rho_t + real_row_q(row0 + 1, N) * N),
                                          fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef};
-    fft_rowtile_call<M, TWX, C::CW, NT, false, 2, ScreenSourceRows<M, MODEL>, true>(buf, tw, src);
+    fft_rowtile_call<M, TWX, C::CW, NT, false, ScreenSourceRows<M, MODEL>, true>(buf, tw + M, src);
     row_r2c_store<N, TWX>(buf, tw, moved(s_out, r.by), row0);
     __syncthreads();
     cur ^= 1;
@@ -1892,9 +1905,18 @@ struct PlaneCfg {
   static constexpr int ROWS = fft_rows<N>();
   static constexpr int TWCOL = N == 128 ? 24 : CW;  // column chunk (a multiple of 8, CW = 3 x 24 at N = 128)
   static constexpr size_t buf = (size_t)ROWS * CW;   // float2
-  static constexpr size_t smem = ((size_t)N + buf) * sizeof(float2);
+  static constexpr size_t smem = ((size_t)N + M + buf) * sizeof(float2);  // twiddles (load_plane_tw), plane
   static_assert(CW >= M + 1 && CW % 8 == 0 && CW % TWCOL == 0 && TWCOL % 8 == 0, "plane pitch");
 };
+
+// Twiddles of a plane pass: the N-entry table (columns, real split), then M entries of
+// row transform first-step twiddles (fft_rowtile's w1 = tw + N).
+template <int N>
+__device__ __forceinline__ void load_plane_tw(float2* tw, const float2* __restrict__ twg) {
+  constexpr int M = N / 2;
+  load_tw(tw, twg, N);
+  for (int i = threadIdx.x; i < M; i += NT) tw[N + i] = twg[2 * row_twiddle<M>(i)];
+}
 
 // The N real rows of a plane (N floats each) as M complex values per row at pitch CW.
 template <int N>
@@ -1937,15 +1959,15 @@ __global__ void __launch_bounds__(NT) k_plane_r2c(const float* __restrict__ in, 
   using C = PlaneCfg<N>;
   extern __shared__ __align__(128) float2 sm[];
   float2* tw = sm;
-  float2* buf = sm + N;
+  float2* buf = sm + N + C::M;
   const int z = blockIdx.x;
   const int64_t by = shift_of(m, blockIdx.y);
-  load_tw(tw, twg, N);
+  load_plane_tw<N>(tw, twg);
   stage_real_plane<N>(buf, moved(in, by) + (int64_t)z * N * N);
   cp_async_commit();
   cp_async_wait<0>();
   __syncthreads();
-  fft_rowtile<C::M, N, C::CW, NT, false, 2>(buf, tw, ScaleOffset{scale, offset});
+  fft_rowtile<C::M, N, C::CW, NT, false>(buf, tw + N, ScaleOffset{scale, offset});
   plane_r2c_split<N>(buf, tw);
   constexpr int64_t P = half_pitch(N);
   float2* g = moved(out, by) + hrow(z, 0, N, P);
@@ -1992,8 +2014,8 @@ __device__ __forceinline__ void plane_yinv(float2* a, const float2* tw) {
 template <int N>
 __device__ __forceinline__ void plane_xc2r(float2* a, const float2* tw, float kfs, float* g) {
   using C = PlaneCfg<N>;
-  fft_rowtile<C::M, N, C::CW, NT, true, 2, C2rCombine<N, C::CW>, false, PlaneRowOut<C::M>>(
-      a, tw, C2rCombine<N, C::CW>{a, tw, kfs}, PlaneRowOut<C::M>{reinterpret_cast<float2*>(g)});
+  fft_rowtile<C::M, N, C::CW, NT, true, C2rCombine<N, C::CW>, false, PlaneRowOut<C::M>>(
+      a, tw + N, C2rCombine<N, C::CW>{a, tw, kfs}, PlaneRowOut<C::M>{reinterpret_cast<float2*>(g)});
 }
 
 // i kfs f_y times every value of plane buffer a (f_y the signed frequency of row y;
@@ -2029,7 +2051,7 @@ __global__ void __launch_bounds__(NT) k_plane_grad(PlaneJobs jobs, const float2*
   using C = PlaneCfg<N>;
   extern __shared__ __align__(128) float2 sm[];
   float2* tw = sm;
-  float2* a = sm + N;
+  float2* a = sm + N + C::M;
   const int z = blockIdx.x / jobs.n, q = blockIdx.x - z * jobs.n;
   const int64_t by = shift_of(m, blockIdx.y), off = (int64_t)z * N * N;
   const float2* in = jobs.in[0];
@@ -2040,7 +2062,7 @@ __global__ void __launch_bounds__(NT) k_plane_grad(PlaneJobs jobs, const float2*
       in = jobs.in[i];
       out = jobs.out[i];
     }
-  load_tw(tw, twg, N);
+  load_plane_tw<N>(tw, twg);
   stage_complex_plane<N>(a, moved(in, by), z);
   cp_async_commit();
   if (jobs.zdst) {  // this CTA's share of the zero fill while its plane lands
@@ -2069,20 +2091,20 @@ __global__ void __launch_bounds__(NT) k_plane_screen(const float2* __restrict__ 
   constexpr int M = C::M;
   extern __shared__ __align__(128) float2 sm[];
   float2* tw = sm;
-  float2* a = sm + N;
+  float2* a = sm + N + C::M;
   const int z = blockIdx.x;
   const int64_t by = shift_of(m, blockIdx.y);
   resolve(fp, by);
-  load_tw(tw, twg, N);
+  load_plane_tw<N>(tw, twg);
   stage_complex_plane<N>(a, moved(w_in, by), z);
   cp_async_commit();
   cp_async_wait<0>();
   __syncthreads();
   plane_yinv<N>(a, tw);
-  fft_rowtile<M, N, C::CW, NT, true, 2, C2rCombine<N, C::CW>>(a, tw, C2rCombine<N, C::CW>{a, tw, 0.f});
+  fft_rowtile<M, N, C::CW, NT, true, C2rCombine<N, C::CW>>(a, tw + N, C2rCombine<N, C::CW>{a, tw, 0.f});
   const ScreenSource<M, MODEL> src{reinterpret_cast<const float2*>(moved(rho, by) + (int64_t)z * N * N),
                                          fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef};
-  fft_rowtile<M, N, C::CW, NT, false, 2, ScreenSource<M, MODEL>>(a, tw, src);
+  fft_rowtile<M, N, C::CW, NT, false, ScreenSource<M, MODEL>>(a, tw + N, src);
   plane_r2c_split<N>(a, tw);
   constexpr int64_t P = half_pitch(N);
   float2* g = moved(s_out, by) + hrow(z, 0, N, P);
