@@ -363,13 +363,11 @@ __host__ __device__ constexpr int row_twiddle(int i) {
   return (i / Split<L>::R2) * (i % Split<L>::R2);
 }
 
-template <int L, int TW, int CW, int NT, bool INV, class Pre = NoPre, bool PAIR32 = false,
-          class Store = RowStore>
-__device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const float2* __restrict__ w1,
-                                            Pre pre = Pre(), Store st = Store()) {
+// Step 1 of the row transforms, with the barriers that separate it from step 2.
+template <int L, int TW, int CW, int NT, bool INV, class Pre>
+__device__ __forceinline__ void row_step1(float2* __restrict__ buf, const float2* __restrict__ w1, Pre pre) {
   constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;
   constexpr int U1 = TW * R2, P1 = (U1 + NT - 1) / NT;
-  constexpr int U2 = TW * R1, P2 = (U2 + NT - 1) / NT;
   static_assert(CW >= L + R2 - 1, "row pitch too small for the intermediate");
   const int tid = threadIdx.x;
   {
@@ -406,6 +404,16 @@ __device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const floa
     }
   }
   __syncthreads();
+}
+
+template <int L, int TW, int CW, int NT, bool INV, class Pre = NoPre, bool PAIR32 = false,
+          class Store = RowStore>
+__device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const float2* __restrict__ w1,
+                                            Pre pre = Pre(), Store st = Store()) {
+  constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;
+  constexpr int U2 = TW * R1, P2 = (U2 + NT - 1) / NT;
+  const int tid = threadIdx.x;
+  row_step1<L, TW, CW, NT, INV, Pre>(buf, w1, pre);
   if constexpr (PAIR32 && R1 == 16 && R2 == 32 && 2 * U2 == NT) {
     // step 2 on thread pairs (dft32_pair): U2 items would leave half the threads
     // idle; half the registers per thread
@@ -454,11 +462,96 @@ __device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const floa
   __syncthreads();
 }
 
+// Forward row transform of real rows packed as z[n] = x[2n] + i x[2n+1] (L
+// complex values), with the split into the half spectrum of the 2L reals
+//   X[k] = (Z[k] + conj Z[L-k])/2 - i/2 w^k (Z[k] - conj Z[L-k]),  k = 0..L,
+// w = exp(-2 pi i / 2L) from twr, done in the registers of step 2: thread (c,
+// k1) holds Z[k1 + R1 k2], and Z[L - k] of k1 > 0 is entry R2 - 1 - k2 of lane
+// R1 - k1 of the same row, one shuffle away (k1 = 0: the thread's own entry
+// (R2 - k2) mod R2).  X leaves through st(X[k], c, k), where consecutive lanes
+// hold consecutive k.  Writing Z back to the tile and reading the pairs from
+// there costs 8 shared-memory wavefronts per point and warp, this 3 (two
+// shuffles, one broadcast twiddle read), and one barrier less: x r2c 1.61 ->
+// 1.30 ms and screening x 3.45 -> 3.14 ms at 1024^3, x r2c plane pass 1.21 ->
+// 1.06 ms over 256 meshes of 128^3.  PAIR32 as in fft_rowtile.
+template <int L, int TW, int CW, int NT, class Pre, bool PAIR32, class Store>
+__device__ __forceinline__ void fft_rowtile_r2c(float2* __restrict__ buf, const float2* __restrict__ w1,
+                                                const float2* __restrict__ twr, Pre pre, Store st) {
+  constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;
+  constexpr int U2 = TW * R1, P2 = (U2 + NT - 1) / NT;
+  static_assert(R1 <= 32 && U2 % 32 == 0, "whole warps take part in the shuffles");
+  const int tid = threadIdx.x, lane = tid & 31;
+  row_step1<L, TW, CW, NT, false, Pre>(buf, w1, pre);
+  auto emit = [&](float2 zk, float2 zm, int c, int k) {
+    const float2 b = cconj(zm), E = cscale(cadd(zk, b), 0.5f), D = csub(zk, b);
+    const float2 X = cadd(E, cmul(twr[k], make_float2(0.5f * D.y, -0.5f * D.x)));  // O = (-i/2) D
+    const float2 o = st(X, c, k);
+    if constexpr (Store::kSmem) buf[c * CW + k] = o;
+  };
+  if constexpr (PAIR32 && R1 == 16 && R2 == 32 && 2 * U2 == NT) {
+    // a row per warp; half h of lane (k1, h) holds Z[k1 + 16 (2k + h)] at y[k]
+    const int half = lane >> 4, c = tid >> 5, k1 = lane & 15;
+    float2 y[16];
+    const float2* yr = buf + c * CW + k1 + 16 * half * (R1 + 1);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) y[j] = yr[j * (R1 + 1)];
+    dft32_pair<false>(y, half);
+    if constexpr (Store::kSmem) __syncthreads();
+    const int partner = k1 ? ((1 - half) << 4) | (16 - k1) : lane;
+    const bool own = k1 == 0 && half == 0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      float2 zm = make_float2(__shfl_sync(0xffffffffu, y[15 - k].x, partner),
+                              __shfl_sync(0xffffffffu, y[15 - k].y, partner));
+      if (own) zm = y[(16 - k) & 15];
+      emit(y[k], zm, c, k1 + 16 * (2 * k + half));
+    }
+    if (own) emit(y[0], y[0], c, L);
+  } else {
+    float2 y[P2][R2];
+#pragma unroll
+    for (int i = 0; i < P2; ++i) {
+      const int u = tid + i * NT;
+      if ((U2 % NT) == 0 || u < U2) {
+        const int c = u / R1, k1 = u % R1;
+        const float2* yr = buf + c * CW + k1;
+#pragma unroll
+        for (int n2 = 0; n2 < R2; ++n2) y[i][pos_of<R2>(n2)] = yr[n2 * (R1 + 1)];
+        dftR<R2, false>(y[i]);
+      }
+    }
+    if constexpr (Store::kSmem) __syncthreads();
+#pragma unroll
+    for (int i = 0; i < P2; ++i) {
+      const int u = tid + i * NT;
+      if ((U2 % NT) == 0 || u < U2) {
+        const int c = u / R1, k1 = u % R1;
+        const int partner = (lane & ~(R1 - 1)) | ((R1 - k1) & (R1 - 1));
+#pragma unroll
+        for (int k2 = 0; k2 < R2; ++k2) {
+          float2 zm = make_float2(__shfl_sync(0xffffffffu, y[i][R2 - 1 - k2].x, partner),
+                                  __shfl_sync(0xffffffffu, y[i][R2 - 1 - k2].y, partner));
+          if (k1 == 0) zm = y[i][(R2 - k2) % R2];
+          emit(y[i][k2], zm, c, k1 + R1 * k2);
+        }
+        if (k1 == 0) emit(y[i][0], y[i][0], c, L);
+      }
+    }
+  }
+  __syncthreads();
+}
+
 template <int L, int TW, int CW, int NT, bool INV, class Pre = NoPre, bool PAIR32 = false,
           class Store = RowStore>
 __device__ __noinline__ void fft_rowtile_call(float2* buf, const float2* w1, Pre pre = Pre(),
                                               Store st = Store()) {
   fft_rowtile<L, TW, CW, NT, INV, Pre, PAIR32, Store>(buf, w1, pre, st);
+}
+
+template <int L, int TW, int CW, int NT, class Pre, bool PAIR32, class Store>
+__device__ __noinline__ void fft_rowtile_r2c_call(float2* buf, const float2* w1, const float2* twr, Pre pre,
+                                                  Store st) {
+  fft_rowtile_r2c<L, TW, CW, NT, Pre, PAIR32, Store>(buf, w1, twr, pre, st);
 }
 
 // Out-of-line copy for kernels that run several transforms per tile: each

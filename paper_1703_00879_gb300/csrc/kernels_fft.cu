@@ -1360,33 +1360,19 @@ __device__ __forceinline__ void stage_real_rows(float* st, const float* __restri
   }
 }
 
-// r2c post-processing: X[k] = (Z[k] + conj Z[M-k])/2 - i/2 w^k (Z[k] - conj Z[M-k]),
-// written in memory order; position w of a row pair is row (w >> 3) & 1,
-// column k = (w >> 4) 8 + (w & 7); w + 32 is the same row, k + 16.  Padding
-// columns k > M are not written.
-template <int N, int TWX>
-__device__ __forceinline__ void row_r2c_store(const float2* buf, const float2* tw,
-                                              float2* __restrict__ out, int64_t q0) {
-  using C = RowCfg<N, TWX>;
-  constexpr int M = N / 2;
-  constexpr int P = (int)half_pitch(N);
-  float2* dst = out + hrow_q(q0, P);
-  for_pairs<TWX / 2, 2 * P>([&](int pr, int w0, int w1) {
-    int k = (w0 >> 4) * 8 + (w0 & 7);
-    const float2* z = buf + (2 * pr + ((w0 >> 3) & 1)) * C::CW;
-    float2* o = dst + (int64_t)pr * 2 * P + w0;
-#pragma unroll 2
-    for (int w = w0; w < w1; w += 32, k += 16, o += 32) {
-      if (k > M) continue;
-      const float2 a = z[k & (M - 1)];
-      const float2 b = cconj(z[(M - k) & (M - 1)]);
-      const float2 E = cscale(cadd(a, b), 0.5f);
-      const float2 D = csub(a, b);
-      const float2 O = make_float2(0.5f * D.y, -0.5f * D.x);  // (-i/2) D
-      *o = cadd(E, cmul(tw[k], O));
-    }
-  });
-}
+// Store hook of the forward row transforms (fft_rowtile_r2c): X[k] of tile row r into
+// the interleaved half spectrum, g = the tile's first row pair.  A warp holds 16 (or
+// fewer) consecutive k of an even and an odd tile row, the two halves of whole
+// 128-byte chunk pairs.
+template <int P>
+struct HalfRowOut {
+  static constexpr bool kSmem = false;
+  float2* g;
+  __device__ __forceinline__ float2 operator()(float2 v, int r, int k) const {
+    g[(r >> 1) * 2 * P + (r & 1) * 8 + (k >> 3) * 16 + (k & 7)] = v;
+    return v;
+  }
+};
 
 // The c2r input convention on a staged spectrum value X[k] (k = 0..M): the
 // optional derivative i kfs k (zero at the Nyquist k = M), and the imaginary
@@ -1464,7 +1450,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xr2c(const float* 
                                                 const float2* __restrict__ twg, int64_t ntiles,
                                                 Multi m) {
   using C = RowCfg<N, TWX>;
-  constexpr int M = N / 2;
+  constexpr int M = N / 2, P = (int)half_pitch(N);
   extern __shared__ __align__(128) float2 sm[];
   float2* tw = sm;
   float2* st0 = sm + N;
@@ -1507,10 +1493,9 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xr2c(const float* 
       }
       __syncthreads();
       if (fail) break;
-      float2* buf = cur ? st1 : st0;
-      fft_rowtile<M, TWX, C::CW, NT, false>(buf, tw + M, ScaleOffset{scale, offset});
-      row_r2c_store<N, TWX>(buf, tw, out, row_tile<N, TWX>(t, m).row0);
-      __syncthreads();
+      const HalfRowOut<P> o{out + hrow_q(row_tile<N, TWX>(t, m).row0, P)};
+      fft_rowtile_r2c<M, TWX, C::CW, NT, ScaleOffset, false, HalfRowOut<P>>(cur ? st1 : st0, tw + M, tw,
+                                                                           ScaleOffset{scale, offset}, o);
       cur ^= 1;
     }
     if (lead && fail) {
@@ -1537,11 +1522,10 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xr2c(const float* 
     cp_async_commit();
     cp_async_wait<1>();
     __syncthreads();
-    float2* buf = cur ? st1 : st0;
-    fft_rowtile<M, TWX, C::CW, NT, false>(buf, tw + M, ScaleOffset{scale, offset});
     const RowTile r = row_tile<N, TWX>(t, m);
-    row_r2c_store<N, TWX>(buf, tw, moved(out, r.by), r.row0);
-    __syncthreads();
+    const HalfRowOut<P> o{moved(out, r.by) + hrow_q(r.row0, P)};
+    fft_rowtile_r2c<M, TWX, C::CW, NT, ScaleOffset, false, HalfRowOut<P>>(cur ? st1 : st0, tw + M, tw,
+                                                                         ScaleOffset{scale, offset}, o);
     cur ^= 1;
   }
   cp_async_wait<0>();
@@ -1880,9 +1864,9 @@ __global__ void __launch_bounds__(NT, 2) k_x_screen(const float2* __restrict__ w
     const ScreenSourceRows<M, MODEL> src{reinterpret_cast<const float2*>(rho_t + real_row_q(row0, N) * N),
                                          reinterpret_cast<const float2*>(rho_t + real_row_q(row0 + 1, N) * N),
                                          fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef};
-    fft_rowtile_call<M, TWX, C::CW, NT, false, ScreenSourceRows<M, MODEL>, true>(buf, tw + M, src);
-    row_r2c_store<N, TWX>(buf, tw, moved(s_out, r.by), row0);
-    __syncthreads();
+    constexpr int P = (int)half_pitch(N);
+    fft_rowtile_r2c_call<M, TWX, C::CW, NT, ScreenSourceRows<M, MODEL>, true, HalfRowOut<P>>(
+        buf, tw + M, tw, src, HalfRowOut<P>{moved(s_out, r.by) + hrow_q(row0, P)});
     cur ^= 1;
   }
   cp_async_wait<0>();
@@ -1928,28 +1912,6 @@ __device__ __forceinline__ void stage_real_plane(float2* buf, const float* __res
   }
 }
 
-// r2c split of every plane row in place (the split of row_r2c_store): from the
-// packed transform Z of row r, X[k] = (Z[k] + conj Z[M-k])/2 - i/2 w^k (Z[k] - conj Z[M-k])
-// for k = 0..M; a thread takes the pair (k, M - k) (k = 0: X[0] and X[M] from Z[0]).
-template <int N>
-__device__ __forceinline__ void plane_r2c_split(float2* buf, const float2* tw) {
-  constexpr int M = N / 2, CW = PlaneCfg<N>::CW, H = M / 2 + 1;
-  auto X = [&](float2 a, float2 bz, float2 w) {
-    const float2 b = cconj(bz);
-    const float2 E = cscale(cadd(a, b), 0.5f), D = csub(a, b);
-    return cadd(E, cmul(w, make_float2(0.5f * D.y, -0.5f * D.x)));
-  };
-  for (int e = threadIdx.x; e < N * H; e += NT) {
-    const int r = e / H, k = e - r * H;
-    float2* z = buf + r * CW;
-    const float2 zk = z[k], zm = z[(M - k) & (M - 1)];
-    const float2 xk = X(zk, zm, tw[k]), xm = X(zm, zk, tw[M - k]);
-    z[k] = xk;
-    if (k != M - k) z[M - k] = xm;
-  }
-  __syncthreads();
-}
-
 // Forward x (r2c, input scaled then offset) and y transforms of plane blockIdx.x of a
 // real N^3 field into the interleaved half spectrum (the z pass follows separately).
 template <int N>
@@ -1967,8 +1929,8 @@ __global__ void __launch_bounds__(NT) k_plane_r2c(const float* __restrict__ in, 
   cp_async_commit();
   cp_async_wait<0>();
   __syncthreads();
-  fft_rowtile<C::M, N, C::CW, NT, false>(buf, tw + N, ScaleOffset{scale, offset});
-  plane_r2c_split<N>(buf, tw);
+  fft_rowtile_r2c<C::M, N, C::CW, NT, ScaleOffset, false, RowStore>(buf, tw + N, tw, ScaleOffset{scale, offset},
+                                                                   RowStore{});
   constexpr int64_t P = half_pitch(N);
   float2* g = moved(out, by) + hrow(z, 0, N, P);
 #pragma unroll 1
@@ -2104,8 +2066,7 @@ __global__ void __launch_bounds__(NT) k_plane_screen(const float2* __restrict__ 
   fft_rowtile<M, N, C::CW, NT, true, C2rCombine<N, C::CW>>(a, tw + N, C2rCombine<N, C::CW>{a, tw, 0.f});
   const ScreenSource<M, MODEL> src{reinterpret_cast<const float2*>(moved(rho, by) + (int64_t)z * N * N),
                                          fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef};
-  fft_rowtile<M, N, C::CW, NT, false, ScreenSource<M, MODEL>>(a, tw + N, src);
-  plane_r2c_split<N>(a, tw);
+  fft_rowtile_r2c<M, N, C::CW, NT, ScreenSource<M, MODEL>, false, RowStore>(a, tw + N, tw, src, RowStore{});
   constexpr int64_t P = half_pitch(N);
   float2* g = moved(s_out, by) + hrow(z, 0, N, P);
 #pragma unroll 1
