@@ -770,7 +770,7 @@ ForceParams force_params(const cola_ctx* c, double a) {
   return fp;
 }
 
-// 3-D transforms on the internal half-spectrum layout (plane pairs interleaved
+// 3-D transforms on the internal half-spectrum layout (planes interleaved
 // in 64-byte chunks, cola_internal.h).
 int r2c3(cola_ctx* ctx, int N, const float* in, float2* out, const float2* tw, float scale,
          float offset, Multi m = {}) {

@@ -9,7 +9,7 @@
 // Every pass is a persistent kernel (grid = SMs x resident CTAs) that walks
 // its tiles in a software pipeline: the next tile is staged with cp.async into
 // a second shared-memory buffer while the current tile is transformed.  The
-// half spectra use the plane-pair interleaved layout of cola_internal.h.
+// half spectra use the plane-interleaved layout of cola_internal.h.
 //
 // Most k-space operations and output stores run inside the tile transforms,
 // through their load hook (first step) and store hook (last step), so a tile
@@ -162,24 +162,24 @@ __device__ __forceinline__ void cp_async_wait() {
 
 // ---------------------------------------------------------------- column tiles
 // Tile element (n, c) of sub-block `sub` lives at buf[n * TP + sub * TW + c];
-// global element at g[base + row(n) + hcol(c)] with row(n) = (n >> 1) ra +
-// (n & 1) rb (the half-spectrum layout of cola_internal.h); only columns
+// global element at g[base + row(n) + hcol(c)] with row(n) = (n / HQ) ra +
+// (n mod HQ) rb (the half-spectrum layout of cola_internal.h); only columns
 // c0 + c < N/2 + 1 exist.  Each thread keeps one 16-byte piece (or one column)
-// and walks rows n0, n0 + step, ... (step even, so n & 1 stays fixed).
+// and walks rows n0, n0 + step, ... (HQ | step, so n mod HQ stays fixed).
 template <int N, int TW, int TP>
 __device__ __forceinline__ void col_issue(float2* buf, int sub, const float2* __restrict__ g,
                                           int64_t base, int64_t ra, int64_t rb, int c0) {
   constexpr int CH = TW / 2;  // 16-byte pieces per row segment
   constexpr int STEP = NT / CH;
-  static_assert(STEP % 2 == 0, "row step must be even");
+  static_assert(STEP % HQ == 0, "row step: whole plane groups");
   const int j = threadIdx.x % CH, n0 = threadIdx.x / CH;
   const bool v = c0 + 2 * j < N / 2 + 1;
-  const float2* src = g + base + (n0 >> 1) * ra + (n0 & 1) * rb + hcol(2 * j);
+  const float2* src = g + base + (n0 / HQ) * ra + (n0 % HQ) * rb + hcol(2 * j);
   float2* dst = buf + n0 * TP + sub * TW + 2 * j;
 #pragma unroll 4
   for (int n = n0; n < N; n += STEP) {
     cp_async16(dst, v ? (const void*)src : (const void*)g, v);
-    src += (STEP / 2) * ra;
+    src += (STEP / HQ) * ra;
     dst += STEP * TP;
   }
 }
@@ -192,15 +192,15 @@ __device__ __forceinline__ void col_issue_raw(uint32_t* rb_, int f, const uint32
                                               int64_t base, int64_t ra, int64_t rb, int c0) {
   constexpr int CH = TW / 4;
   constexpr int STEP = NT / CH;
-  static_assert(STEP % 2 == 0, "row step must be even");
+  static_assert(STEP % HQ == 0, "row step: whole plane groups");
   const int j = threadIdx.x % CH, n0 = threadIdx.x / CH;
   const bool v = c0 + 4 * j < N / 2 + 1;
-  const uint32_t* src = g + base + (n0 >> 1) * ra + (n0 & 1) * rb + hcol(4 * j);
+  const uint32_t* src = g + base + (n0 / HQ) * ra + (n0 % HQ) * rb + hcol(4 * j);
   uint32_t* dst = rb_ + 8 * n0 * TW + 4 * TW + f * TW + 4 * j;
 #pragma unroll 4
   for (int n = n0; n < N; n += STEP) {
     cp_async16(dst, v ? (const void*)src : (const void*)g, v);
-    src += (STEP / 2) * ra;
+    src += (STEP / HQ) * ra;
     dst += 8 * STEP * TW;
   }
 }
@@ -209,15 +209,15 @@ template <int N, int TW, int TP>
 __device__ __forceinline__ void col_store(const float2* buf, int sub, float2* __restrict__ g,
                                           int64_t base, int64_t ra, int64_t rb, int c0) {
   constexpr int STEP = NT / TW;
-  static_assert(STEP % 2 == 0, "row step must be even");
+  static_assert(STEP % HQ == 0, "row step: whole plane groups");
   const int c = threadIdx.x % TW, n0 = threadIdx.x / TW;
   if (c0 + c >= N / 2 + 1) return;
-  float2* dst = g + base + (n0 >> 1) * ra + (n0 & 1) * rb + hcol(c);
+  float2* dst = g + base + (n0 / HQ) * ra + (n0 % HQ) * rb + hcol(c);
   const float2* src = buf + n0 * TP + sub * TW + c;
 #pragma unroll 4
   for (int n = n0; n < N; n += STEP) {
     *dst = *src;
-    dst += (STEP / 2) * ra;
+    dst += (STEP / HQ) * ra;
     src += STEP * TP;
   }
 }
@@ -244,16 +244,16 @@ struct TileLane {
 };
 
 // Store hook of a column transform that writes element (n, c) straight to
-// g[(n >> 1) ra + (n & 1) rb + hcol(c)] (g = the tile's base, columns c < live
+// g[(n / HQ) ra + (n mod HQ) rb + hcol(c)] (g = the tile's base, columns c < live
 // exist) instead of through the tile and col_store: a warp's stores cover whole
-// 128-byte chunk pairs.
+// 64-byte chunks.
 struct ColOut {
   static constexpr bool kSmem = false;
   float2* g;
   int64_t ra, rb;
   int live;
   __device__ __forceinline__ float2 operator()(float2 v, int n, int c, int) const {
-    if (c < live) g[(n >> 1) * ra + (n & 1) * rb + hcol(c)] = v;
+    if (c < live) g[(n / HQ) * ra + (n % HQ) * rb + hcol(c)] = v;
     return v;
   }
   __device__ __forceinline__ void ready() const {}
@@ -261,16 +261,15 @@ struct ColOut {
 
 // Column geometry: tile t -> (simulation b, outer index o, column block c0);
 // base = the element offset of (o, row 0, c0) and `by` = the byte shift of
-// simulation b's buffers.  Outer index o sits at (o >> 1) oa + (o & 1) ob and
-// tile row n at (n >> 1) ra + (n & 1) rb.  With pair_tiles, consecutive tiles
-// take o = 2i and 2i + 1 of the same column block (the two halves of each
-// 128-byte chunk pair of the y pass are read by neighbouring CTAs together).
+// simulation b's buffers.  Outer index o sits at (o / HQ) oa + (o mod HQ) ob and
+// tile row n at (n / HQ) ra + (n mod HQ) rb.  Along y, consecutive tiles take the
+// HQ planes o of one group at the same column block (the parts of each chunk
+// group are read by neighbouring CTAs together).
 template <int N, int TW>
 struct ColGeo {
   static constexpr int ntx = (N / 2) / TW + 1;
   static constexpr int64_t tps = (int64_t)N * ntx;  // tiles per simulation
   int64_t oa, ob, ra, rb;
-  int pair_tiles;
   int zaxis;  // 1: tiles run along z (o = y), 0: along y (o = z)
   Multi m;
   // t < 2^31 (prep checks the tile count); divisions by compile-time constants
@@ -279,16 +278,16 @@ struct ColGeo {
     const uint32_t b = t / (uint32_t)tps;
     t -= b * (uint32_t)tps;
     by = shift_of(m, (int)b);
-    if (pair_tiles) {
-      const uint32_t q = t / (2 * ntx), r = t - q * (2 * ntx);
-      o = (int)(q * 2 + (r & 1));
-      c0 = (int)(r >> 1) * TW;
+    if (!zaxis) {
+      const uint32_t q = t / (HQ * ntx), r = t - q * (HQ * ntx);
+      o = (int)(q * HQ + r % HQ);
+      c0 = (int)(r / HQ) * TW;
     } else {
       const uint32_t q = t / ntx;
       o = (int)q;
       c0 = (int)(t - q * ntx) * TW;
     }
-    base = (o >> 1) * oa + (o & 1) * ob + hcol(c0);
+    base = (o / HQ) * oa + (o % HQ) * ob + hcol(c0);
   }
 };
 
@@ -332,11 +331,11 @@ __device__ __forceinline__ void col_pipeline(Op op, const float2* __restrict__ t
 // the tensor-memory accelerator: thread 0 issues a few cp.async.bulk.tensor
 // copies per tile, completion is tracked by an mbarrier per stage buffer, and
 // the transform warps issue no load instructions.  The half spectrum is seen
-// as a 5-D array of 8-byte elements (column within a 64-byte half chunk, plane
-// parity, chunk, y, plane pair), byte strides 8, 64, 128, 2P*8, 2NP*8: the
-// interleaved layout of cola_internal.h.  A z tile (TW <= 8 columns of one y)
-// is boxes of {TW, 2, 1, 1, <= 256 pairs}, landing as rows n = 2j + parity of
-// TW values; a y tile (one z) boxes of {TW, 1, 1, <= 256 rows, 1}.
+// as a 5-D array of 8-byte elements (column within a 64-byte chunk, plane
+// within its group, chunk, y, plane group), byte strides 8, 64, 64 HQ, 8 HQ P,
+// 8 HQ N P: the interleaved layout of cola_internal.h.  A z tile (TW <= 8 columns
+// of one y) is boxes of {TW, HQ, 1, 1, <= 256 groups}, landing as rows n = HQ j +
+// plane of TW values; a y tile (one z) boxes of {TW, 1, 1, <= 256 rows, 1}.
 __device__ unsigned int g_tile_load_failures;  // waits that ran out (host: tile_load_failures)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -419,19 +418,19 @@ __device__ __forceinline__ void bulk_store_drain() { asm volatile("cp.async.bulk
 template <int N, int TW>
 __device__ __forceinline__ void tma_tile(const ColGeo<N, TW>& geo, const CUtensorMap* map, float2* buf,
                                          int64_t t, uint64_t* bar) {
-  static_assert(TW <= 8 && TW % 2 == 0, "TMA tiles: at most one 64-byte half chunk");
+  static_assert(TW <= 8 && TW % 2 == 0, "TMA tiles: at most one 64-byte chunk");
   int o, c0;
   int64_t base, by;
   geo.tile(t, o, c0, base, by);
   bar_expect(bar, (uint32_t)(N * TW * sizeof(float2)));
   if (geo.zaxis) {
-    constexpr int B = N / 2 < 256 ? N / 2 : 256;
+    constexpr int B = N / HQ < 256 ? N / HQ : 256;
 #pragma unroll
-    for (int k = 0; k < N / 2; k += B) tma_load5(buf + 2 * k * TW, map, c0 & 7, 0, c0 >> 3, o, k, bar);
+    for (int k = 0; k < N / HQ; k += B) tma_load5(buf + HQ * k * TW, map, c0 & 7, 0, c0 >> 3, o, k, bar);
   } else {
     constexpr int B = N < 256 ? N : 256;
 #pragma unroll
-    for (int k = 0; k < N; k += B) tma_load5(buf + k * TW, map, c0 & 7, o & 1, c0 >> 3, k, o >> 1, bar);
+    for (int k = 0; k < N; k += B) tma_load5(buf + k * TW, map, c0 & 7, o % HQ, c0 >> 3, k, o / HQ, bar);
   }
 }
 
@@ -602,7 +601,7 @@ struct OpYinv2 {
     __device__ __forceinline__ float2 operator()(float2 v, int n, int c, int) const {
       const bool d = c >= TW;
       const int cc = d ? c - TW : c;
-      if (cc < live) (d ? gd : gp)[(n >> 1) * ra + (n & 1) * rb + hcol(cc)] = v;
+      if (cc < live) (d ? gd : gp)[(n / HQ) * ra + (n % HQ) * rb + hcol(cc)] = v;
       return v;
     }
     __device__ __forceinline__ void ready() const {}
@@ -813,13 +812,13 @@ struct OpZScreenField {
   // multiplier (-kappa/k^2, or the smoothing window) applied in place.
   struct Field {
     static constexpr bool kSmem = true;
-    float2* dk;  // delta(k) of the tile: element (n, c) at dk[(n >> 1) ra + (n & 1) rb + hcol(c)]
+    float2* dk;  // delta(k) of the tile: element (n, c) at dk[(n / HQ) ra + (n mod HQ) rb + hcol(c)]
     int64_t ra, rb;
     int c0, fy2;
     float kf2, kappa_norm, R2half, norm;
     int filter;
     __device__ __forceinline__ float2 operator()(float2 v, int n, int c, int) const {
-      if (c0 + c < N / 2 + 1) dk[(n >> 1) * ra + (n & 1) * rb + hcol(c)] = v;
+      if (c0 + c < N / 2 + 1) dk[(n / HQ) * ra + (n % HQ) * rb + hcol(c)] = v;
       const int fx = c0 + c, fz = freq_index(n, N);
       const float k2 = kf2 * (float)(fx * fx + fy2 + fz * fz);
       float m = 0.f;
@@ -1129,7 +1128,7 @@ __global__ void __launch_bounds__(NT, blocks_for_smem(col_smem_c(N, 4), N)) k_lp
 
 // The LPT z pass with 8-column tiles (N = 256, 512), where four 4-column
 // output arrays would otherwise fill shared memory: an 8-column tile reads and
-// writes whole 128-byte plane-pair pieces of the interleaved layout (4-column
+// writes whole 64-byte chunks of the interleaved layout (4-column
 // tiles move 32-byte halves of them).  Shared memory: two input buffers
 // (phi1 in columns 0..7, phi2 in 8..15; double-buffered) and one work buffer
 // that first holds (d, i kz d) and then (A, i kz A), each pair inverse
@@ -1152,7 +1151,7 @@ struct PairColOut {
   __device__ __forceinline__ float2 operator()(float2 v, int n, int c, int) const {
     const bool b = c >= 8;
     const int cc = b ? c - 8 : c;
-    if (cc < live) (b ? gb : ga)[(n >> 1) * ra + (n & 1) * rb + hcol(cc)] = v;
+    if (cc < live) (b ? gb : ga)[(n / HQ) * ra + (n % HQ) * rb + hcol(cc)] = v;
     return v;
   }
   __device__ __forceinline__ void ready() const {}
@@ -1165,12 +1164,12 @@ __device__ __forceinline__ void col_issue_raw8(uint32_t* sb, int f, const uint32
   constexpr int STEP = NT / 2;  // two 16-byte pieces (8 words) per row and field
   const int j = threadIdx.x & 1, n0 = threadIdx.x >> 1;
   const bool v = c0 + 4 * j < N / 2 + 1;
-  const uint32_t* src = g + base + (n0 >> 1) * ra + (n0 & 1) * rb + hcol(4 * j);
+  const uint32_t* src = g + base + (n0 / HQ) * ra + (n0 % HQ) * rb + hcol(4 * j);
   uint32_t* dst = sb + n0 * 32 + f * 8 + 4 * j;
 #pragma unroll 4
   for (int n = n0; n < N; n += STEP) {
     cp_async16(dst, v ? (const void*)src : (const void*)g, v);
-    src += (STEP / 2) * ra;
+    src += (STEP / HQ) * ra;
     dst += STEP * 32;
   }
 }
@@ -1277,67 +1276,72 @@ struct RowCfg {
   static constexpr size_t smem = (N + 2 * stage) * sizeof(float2);
 };
 
-// The rows of a row tile (first pair-major row q0, TWX even) are the pairs
-// (z, y) and (z + 1, y) of TWX/2 consecutive y: in the half spectrum one
-// contiguous block of TWX/2 interleaved row pairs (2P complex values each), in
-// real space two blocks of TWX/2 consecutive rows (even tile rows from real row
-// real_row_q(q0), odd ones from real_row_q(q0 + 1)).  Tile row r is staged at
+// The rows of a row tile (first group-major row q0, HQ | TWX) are the rows (z, y) ..
+// (z + HQ - 1, y) of TWX/HQ consecutive y: in the half spectrum one contiguous block
+// of TWX/HQ interleaved row groups (HQ P complex values each), in real space HQ
+// blocks of TWX/HQ consecutive rows, one per plane, N rows apart (the first from
+// real row real_row_q(q0)).  Tile row r (plane r mod HQ, y r / HQ) is staged at
 // st[r * CW ...].
 //
-// Walk over the NPAIR row pairs of a tile in memory order, LEN positions per
-// pair: warps take whole pairs, or split each pair into NW / NPAIR segments
-// when there are fewer pairs than warps; f(pair, p0, p1) visits p = p0, p0 +
+// Walk over the NG row groups of a tile in memory order, LEN positions per
+// group: warps take whole groups, or split each group into NW / NG segments
+// when there are fewer groups than warps; f(group, p0, p1) visits p = p0, p0 +
 // 32, ... < p1 with p0 = segment start + lane (segment starts are multiples of
 // 32, so each warp reads or writes whole lines).
-template <int NPAIR, int LEN, class F>
-__device__ __forceinline__ void for_pairs(F f) {
+template <int NG, int LEN, class F>
+__device__ __forceinline__ void for_groups(F f) {
   constexpr int NW = NT / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if constexpr (NPAIR >= NW) {
-    for (int pr = warp; pr < NPAIR; pr += NW) f(pr, lane, LEN);
+  if constexpr (NG >= NW) {
+    for (int g = warp; g < NG; g += NW) f(g, lane, LEN);
   } else {
-    constexpr int S = NW / NPAIR;
+    constexpr int S = NW / NG;
     constexpr int SEG = (LEN + 32 * S - 1) / (32 * S) * 32;
     const int s = warp % S;
     f(warp / S, s * SEG + lane, (s + 1) * SEG < LEN ? (s + 1) * SEG : LEN);
   }
 }
 
+// 16-byte piece p of a row group holds values 2 (p mod 4), + 1 of chunk p / (4 HQ) of
+// row (p / 4) mod HQ; piece p + 32 is the same row, columns + KSTEP.
+constexpr int KSTEP = 64 / HQ;
+static_assert(32 % (4 * HQ) == 0 && KSTEP * HQ == 64, "32 pieces are whole chunk groups");
+__device__ __forceinline__ int piece_col(int p) { return p / (4 * HQ) * 8 + 2 * (p & 3); }
+__device__ __forceinline__ int piece_row(int p) { return (p >> 2) % HQ; }
+
 // Complex half rows (M + 1 values, staged as M + 2 to keep 16-byte pieces).
-// Piece p of a row pair holds values 2p, 2p + 1 of the pair: row (p >> 2) & 1,
-// columns k = (p >> 3) 8 + 2 (p & 3), k + 1; p + 32 is the same row, k + 32.
 template <int N, int TWX>
 __device__ __forceinline__ void stage_complex_rows(float2* st, const float2* __restrict__ in,
                                                    int64_t q0) {
   using C = RowCfg<N, TWX>;
-  constexpr int P = (int)half_pitch(N);  // 16-byte pieces per row pair
+  constexpr int P = (int)half_pitch(N), LEN = HQ * P / 2;  // 16-byte pieces per row group
   const float2* src = in + hrow_q(q0, P);
-  for_pairs<TWX / 2, P>([&](int pr, int p0, int p1) {
-    int k = (p0 >> 3) * 8 + 2 * (p0 & 3);
-    float2* d = st + (2 * pr + ((p0 >> 2) & 1)) * C::CW + k;
-    const float2* g = src + (int64_t)pr * 2 * P + 2 * p0;
-    for (int p = p0; p < p1; p += 32, k += 32, d += 32, g += 64)
+  for_groups<TWX / HQ, LEN>([&](int gr, int p0, int p1) {
+    int k = piece_col(p0);
+    float2* d = st + (HQ * gr + piece_row(p0)) * C::CW + k;
+    const float2* g = src + (int64_t)gr * HQ * P + 2 * p0;
+    for (int p = p0; p < p1; p += 32, k += KSTEP, d += KSTEP, g += 64)
       if (k < C::M + 2) cp_async16(d, g, true);
   });
 }
 
-// A pair tile: TWX/4 row pairs of a and the same row pairs of b (first pair-major
-// row q0), row pair i of a at tile rows 4i (plane z) and 4i + 2 (plane z + 1), of b
-// at 4i + 1 and 4i + 3, so that tile rows 2w and 2w + 1 are the same real row of a
-// and of b.
+// A pair tile: TWX/2 rows of a and the same rows of b (first group-major row q0), row
+// group i of a at tile rows 2 HQ i + 2 j (plane j), of b at 2 HQ i + 2 j + 1, so that
+// tile rows 2w and 2w + 1 are the same real row of a and of b.
 template <int N, int TWX>
 __device__ __forceinline__ void stage_complex_rows_pair(float2* st, const float2* __restrict__ a,
                                                         const float2* __restrict__ b, int64_t q0) {
   using C = RowCfg<N, TWX>;
-  constexpr int P = (int)half_pitch(N);
+  static_assert(TWX % (2 * HQ) == 0, "whole row groups of a and b");
+  constexpr int P = (int)half_pitch(N), LEN = HQ * P / 2;
   const float2* srca = a + hrow_q(q0, P);
   const float2* srcb = b + hrow_q(q0, P);
-  for_pairs<TWX / 2, P>([&](int pr, int p0, int p1) {
-    const int job = pr & 1, i = pr >> 1;
-    int k = (p0 >> 3) * 8 + 2 * (p0 & 3);
-    float2* d = st + (4 * i + 2 * ((p0 >> 2) & 1) + job) * C::CW + k;
-    const float2* g = (job ? srcb : srca) + (int64_t)i * 2 * P + 2 * p0;
-    for (int p = p0; p < p1; p += 32, k += 32, d += 32, g += 64)
+  for_groups<TWX / HQ, LEN>([&](int gr, int p0, int p1) {
+    const int job = gr & 1, i = gr >> 1;
+    int k = piece_col(p0);
+    float2* d = st + (2 * HQ * i + 2 * piece_row(p0) + job) * C::CW + k;
+    const float2* g = (job ? srcb : srca) + (int64_t)i * HQ * P + 2 * p0;
+    for (int p = p0; p < p1; p += 32, k += KSTEP, d += KSTEP, g += 64)
       if (k < C::M + 2) cp_async16(d, g, true);
   });
 }
@@ -1347,29 +1351,33 @@ __device__ __forceinline__ void stage_complex_rows_pair(float2* st, const float2
 template <int N, int TWX>
 __device__ __forceinline__ void stage_real_rows(float* st, const float* __restrict__ in, int64_t q0,
                                                 int pitch_floats) {
-  constexpr int CH = N / 4;           // 16-byte pieces per row
-  constexpr int HALF = TWX / 2 * CH;  // pieces per block of one parity
-  static_assert(HALF % NT == 0, "a parity block is whole iterations");
-  const float* src0 = in + real_row_q(q0, N) * N;
-  const float* src1 = in + real_row_q(q0 + 1, N) * N;
+  constexpr int CH = N / 4;             // 16-byte pieces per row
+  constexpr int BLK = TWX / HQ * CH;    // pieces per plane
+  const float* src = in + real_row_q(q0, N) * N;
+  if constexpr (BLK % NT == 0) {
 #pragma unroll
-  for (int i = 0; i < 2 * HALF / NT; ++i) {
-    const int h = i * NT / HALF;  // constant per iteration
-    const int e2 = threadIdx.x + i * NT - h * HALF;
-    cp_async16(st + (2 * (e2 / CH) + h) * pitch_floats + 4 * (e2 % CH), (h ? src1 : src0) + 4 * e2, true);
+    for (int i = 0; i < HQ * BLK / NT; ++i) {
+      const int h = i * NT / BLK;  // plane, constant per iteration
+      const int e = threadIdx.x + i * NT - h * BLK;
+      cp_async16(st + (HQ * (e / CH) + h) * pitch_floats + 4 * (e % CH), src + (int64_t)h * N * N + 4 * e, true);
+    }
+  } else {
+    for (int i = threadIdx.x; i < HQ * BLK; i += NT) {
+      const int h = i / BLK, e = i - h * BLK;
+      cp_async16(st + (HQ * (e / CH) + h) * pitch_floats + 4 * (e % CH), src + (int64_t)h * N * N + 4 * e, true);
+    }
   }
 }
 
 // Store hook of the forward row transforms (fft_rowtile_r2c): X[k] of tile row r into
-// the interleaved half spectrum, g = the tile's first row pair.  A warp holds 16 (or
-// fewer) consecutive k of an even and an odd tile row, the two halves of whole
-// 128-byte chunk pairs.
+// the interleaved half spectrum, g = the tile's first row group.  A warp holds 16 (or
+// fewer) consecutive k of adjacent tile rows: whole 64-byte chunks of adjacent planes.
 template <int P>
 struct HalfRowOut {
   static constexpr bool kSmem = false;
   float2* g;
   __device__ __forceinline__ float2 operator()(float2 v, int r, int k) const {
-    g[(r >> 1) * 2 * P + (r & 1) * 8 + (k >> 3) * 16 + (k & 7)] = v;
+    g[(r / HQ) * HQ * P + (r % HQ) * 8 + (k >> 3) * (8 * HQ) + (k & 7)] = v;
     return v;
   }
 };
@@ -1420,7 +1428,7 @@ struct ScaleOffset {
 };
 
 // Row tile t of a multi-simulation launch: simulation t / tps, first row (t mod tps) TWX
-// in the pair-major row order q of the half-spectrum layout (TWX even).
+// in the group-major row order q of the half-spectrum layout (HQ | TWX).
 struct RowTile {
   int64_t row0, by;
 };
@@ -1431,17 +1439,16 @@ __device__ __forceinline__ RowTile row_tile(int64_t t64, const Multi& m) {
   return RowTile{(int64_t)(t - b * TPS) * TWX, shift_of(m, (int)b)};
 }
 
-// The real rows of row tile q0 into st by 1-D bulk copies (thread 0): tile row r
-// (r even from real_row_q(q0), odd from real_row_q(q0 + 1)) at st + r * pitch floats.
+// The real rows of row tile q0 into st by 1-D bulk copies (thread 0): tile row r at
+// st + r * pitch floats.
 template <int N, int TWX>
 __device__ __forceinline__ void bulk_real_rows(float* st, const float* __restrict__ in, int64_t q0,
                                                int pitch_floats, uint64_t* bar) {
   bar_expect(bar, (uint32_t)(TWX * N * sizeof(float)));
-  const float* src0 = in + real_row_q(q0, N) * N;
-  const float* src1 = in + real_row_q(q0 + 1, N) * N;
+  const float* src = in + real_row_q(q0, N) * N;
 #pragma unroll
   for (int r = 0; r < TWX; ++r)
-    bulk_load(st + r * pitch_floats, ((r & 1) ? src1 : src0) + (r >> 1) * N, N * sizeof(float), bar);
+    bulk_load(st + r * pitch_floats, src + ((int64_t)(r % HQ) * N + r / HQ) * N, N * sizeof(float), bar);
 }
 
 template <int N, int TWX, bool BULK>
@@ -1569,14 +1576,20 @@ __device__ __forceinline__ JobTile job_tile(int64_t t64, const RowJobs& jobs, co
   return JobTile{(int)(q - b * (uint32_t)jobs.njobs), (int64_t)(t - q * TPJ) * TWX, shift_of(m, (int)b), q};
 }
 
-// Store hook of the c2r row transform: tile row r's M complex outputs (2M
-// reals) to real row r / 2 of the even (o0) or odd (o1) block.
+// Real row of tile row r relative to the tile's first: plane r mod HQ, y r / HQ.
+template <int N>
+__device__ __forceinline__ int tile_real_row(int r) {
+  return (r % HQ) * N + r / HQ;
+}
+
+// Store hook of the c2r row transform: tile row r's M complex outputs (2M reals) to its
+// real row (o: the first real row of the tile).
 template <int M>
 struct RealRowOut {
   static constexpr bool kSmem = false;
-  float2 *o0, *o1;
+  float2* o;
   __device__ __forceinline__ float2 operator()(float2 v, int r, int k) const {
-    ((r & 1) ? o1 : o0)[(r >> 1) * M + k] = v;
+    o[tile_real_row<2 * M>(r) * M + k] = v;
     return v;
   }
 };
@@ -1587,7 +1600,7 @@ struct RealRowOut {
 template <int M, int OUT>
 struct RealRowOut16 {
   static constexpr bool kSmem = false;
-  uint32_t *o0, *o1;
+  uint32_t* o;
   float inv;
   float* amax;
   __device__ __forceinline__ float2 operator()(float2 v, int r, int k) const {
@@ -1603,7 +1616,7 @@ struct RealRowOut16 {
       const __half2 h = __floats2half2_rn(a, b);
       w = *reinterpret_cast<const uint32_t*>(&h);
     }
-    ((r & 1) ? o1 : o0)[(r >> 1) * M + k] = w;
+    o[tile_real_row<2 * M>(r) * M + k] = w;
     return v;
   }
 };
@@ -1654,12 +1667,10 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r(const __grid_
     // the c2r pre-processing rides on the transform's first loads
     using Pre = C2rCombine<N, C::CW>;
     const Pre pre{buf, tw, jobs.kfs[j.job]};
-    // even tile rows go to one block of consecutive real rows, odd ones to
-    // another, straight from the transform's last step
+    // the outputs leave straight from the transform's last step
     if constexpr (OUT == 0) {
       float* out = moved(static_cast<float*>(jobs.out[j.job]), j.by);
-      const RealRowOut<M> o{reinterpret_cast<float2*>(out + real_row_q(j.row0, N) * N),
-                            reinterpret_cast<float2*>(out + real_row_q(j.row0 + 1, N) * N)};
+      const RealRowOut<M> o{reinterpret_cast<float2*>(out + real_row_q(j.row0, N) * N)};
       fft_rowtile<M, TWX, C::CW, NT, true, Pre, false, RealRowOut<M>>(buf, tw + M, pre, o);
     } else {
       const SimHeader* h = moved(jobs.hdr, j.by);
@@ -1672,7 +1683,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r(const __grid_
       }
       uint32_t* out = moved(static_cast<uint32_t*>(jobs.out[j.job]), j.by);
       float tile_max = 0.f;
-      const RealRowOut16<M, OUT> o{out + real_row_q(j.row0, N) * M, out + real_row_q(j.row0 + 1, N) * M,
+      const RealRowOut16<M, OUT> o{out + real_row_q(j.row0, N) * M,
                                    1.f / h->lq_scale[j.job], &tile_max};
       fft_rowtile<M, TWX, C::CW, NT, true, Pre, false, RealRowOut16<M, OUT>>(buf, tw + M, pre, o);
       run_max = fmaxf(run_max, tile_max);
@@ -1701,15 +1712,15 @@ struct C2rCombine2 {
 // first-step radix, the outputs per row and lane group of that step); one
 // shuffle gives lane l (a) the pair (a, b) of real 2k and lane l ^ R1 (b) that
 // of real 2k + 1, and each writes one 8-byte pair, so a warp's stores cover
-// consecutive cells.  o0 / o1: cell 0 of the first real row of planes z / z + 1.
+// consecutive cells.  o: cell 0 of the tile's first real row.
 template <int N, int R1>
 struct PairRowOut {
   static constexpr bool kSmem = false;
-  float2 *o0, *o1;
+  float2* o;
   __device__ __forceinline__ float2 operator()(float2 v, int r, int k) const {
     const int isb = r & 1;
     const float recv = __shfl_xor_sync(0xffffffffu, isb ? v.x : v.y, R1);
-    float2* row = (((r >> 1) & 1) ? o1 : o0) + (int64_t)(r >> 2) * N;
+    float2* row = o + (int64_t)tile_real_row<N>(r >> 1) * N;
     // one store instruction for the warp: cell 2k (a lanes) or 2k + 1 (b lanes)
     row[2 * k + isb] = isb ? make_float2(recv, v.y) : make_float2(v.x, recv);
     return v;
@@ -1718,7 +1729,7 @@ struct PairRowOut {
 
 // c2r of the rows of a (x derivative i kfs kx on load) and of b into the (x, y)
 // pairs of one interleaved real field (App. B: F_x and F_y of the force mesh),
-// pair tiles of TWX/4 row pairs of each.
+// pair tiles of TWX/2 rows of each.
 template <int N, int TWX>
 __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r_pair(
     const float2* __restrict__ a, const float2* __restrict__ b, float2* __restrict__ out, float kfs,
@@ -1759,7 +1770,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r_pair(
     __syncthreads();
     float2* buf = cur ? st1 : st0;
     float2* o = moved(out, by);
-    const PairRowOut<N, R1> st{o + real_row_q(q0, N) * N, o + real_row_q(q0 + 1, N) * N};
+    const PairRowOut<N, R1> st{o + real_row_q(q0, N) * N};
     fft_rowtile<M, TWX, C::CW, NT, true, C2rCombine2<N, C::CW>, false, PairRowOut<N, R1>>(
         buf, tw + M, C2rCombine2<N, C::CW>{buf, tw, kfs, 0.f}, st);
     __syncthreads();
@@ -1798,16 +1809,14 @@ struct ScreenSource {
   }
 };
 
-// The same for an x-pass row tile, whose even rows are consecutive density rows
-// from `even` and odd rows from `odd`: each warp's loads of one transform step
-// cover 32 consecutive values of a row.
+// The same for an x-pass row tile (rho: the tile's first density row): each warp's
+// loads of one transform step cover 32 consecutive values of a row.
 template <int M, int MODEL>
 struct ScreenSourceRows {
-  const float2* even;
-  const float2* odd;
+  const float2* rho;
   float inv_rhobar, p;
   __device__ __forceinline__ float2 operator()(float2 w, int r, int j) const {
-    const float2 rv = __ldg((r & 1 ? odd : even) + (r >> 1) * M + j);
+    const float2 rv = __ldg(rho + tile_real_row<2 * M>(r) * M + j);
     const float d0 = rv.x * inv_rhobar - 1.f, d1 = rv.y * inv_rhobar - 1.f;
     return make_float2(d0 * screen_eps<MODEL>(w.x, p), d1 * screen_eps<MODEL>(w.y, p));
   }
@@ -1862,7 +1871,6 @@ __global__ void __launch_bounds__(NT, 2) k_x_screen(const float2* __restrict__ w
     // S = delta eps(w) is formed as the forward transform loads it
     const float* rho_t = moved(rho, r.by);
     const ScreenSourceRows<M, MODEL> src{reinterpret_cast<const float2*>(rho_t + real_row_q(row0, N) * N),
-                                         reinterpret_cast<const float2*>(rho_t + real_row_q(row0 + 1, N) * N),
                                          fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef};
     constexpr int P = (int)half_pitch(N);
     fft_rowtile_r2c_call<M, TWX, C::CW, NT, ScreenSourceRows<M, MODEL>, true, HalfRowOut<P>>(
@@ -1936,7 +1944,7 @@ __global__ void __launch_bounds__(NT) k_plane_r2c(const float* __restrict__ in, 
 #pragma unroll 1
   for (int c0 = 0; c0 < C::CW; c0 += C::TWCOL)
     fft_tile<N, C::TWCOL, C::CW, NT, false, 1, TileLoad, ColOut>(
-        buf + c0, tw, TileLoad{}, ColOut{g + hcol(c0), 4 * P, 2 * P, C::M + 1 - c0});
+        buf + c0, tw, TileLoad{}, ColOut{g + hcol(c0), HQ * HQ * P, HQ * P, C::M + 1 - c0});
 }
 
 // Store hook of a plane's row transforms: real row r (M float2 = N reals) to g + r M.
@@ -1959,7 +1967,7 @@ __device__ __forceinline__ void stage_complex_plane(float2* buf, const float2* _
   const float2* src = g + hrow(z, 0, N, P);
   for (int e = threadIdx.x; e < N * CH; e += NT) {
     const int y = e / CH, p = e - y * CH, kx = 2 * p;
-    cp_async16(buf + y * CW + kx, src + (int64_t)y * 2 * P + hcol(kx), true);
+    cp_async16(buf + y * CW + kx, src + (int64_t)y * HQ * P + hcol(kx), true);
   }
 }
 
@@ -2072,7 +2080,7 @@ __global__ void __launch_bounds__(NT) k_plane_screen(const float2* __restrict__ 
 #pragma unroll 1
   for (int c0 = 0; c0 < C::CW; c0 += C::TWCOL)
     fft_tile<N, C::TWCOL, C::CW, NT, false, 1, TileLoad, ColOut>(
-        a + c0, tw, TileLoad{}, ColOut{g + hcol(c0), 4 * P, 2 * P, C::M + 1 - c0});
+        a + c0, tw, TileLoad{}, ColOut{g + hcol(c0), HQ * HQ * P, HQ * P, C::M + 1 - c0});
 }
 
 // ---------------------------------------------------------------- launch helpers
@@ -2087,16 +2095,16 @@ constexpr size_t row_smem() {
   return RowCfg<N, row_tw(N)>::smem;
 }
 
-// Along y: o = z, n = y.  Along z: o = y, n = z (rows of a plane pair 8 elements apart).
+// Along y: o = z, n = y.  Along z: o = y, n = z (rows of a plane group 8 elements apart).
 template <int N, int TW>
 ColGeo<N, TW> geo_y(Multi m) {
   const int64_t P = half_pitch(N);
-  return ColGeo<N, TW>{2 * N * P, 8, 4 * P, 2 * P, 1, 0, m};
+  return ColGeo<N, TW>{HQ * N * P, 8, HQ * HQ * P, HQ * P, 0, m};
 }
 template <int N, int TW>
 ColGeo<N, TW> geo_z(Multi m) {
   const int64_t P = half_pitch(N);
-  return ColGeo<N, TW>{4 * P, 2 * P, 2 * N * P, 8, 0, 1, m};
+  return ColGeo<N, TW>{HQ * HQ * P, HQ * P, HQ * N * P, 8, 1, m};
 }
 template <int N, int TW>
 constexpr int64_t col_tiles() {
@@ -2263,10 +2271,10 @@ static bool spectrum_map(CUtensorMap& map, const float2* base, int N, int TW, bo
   }();
   if (!encode || (reinterpret_cast<uintptr_t>(base) & 15)) return false;
   const cuuint64_t P = (cuuint64_t)half_pitch(N), n = (cuuint64_t)N;
-  const cuuint64_t dims[5] = {8, 2, P / 8, n, n / 2};
-  const cuuint64_t strides[4] = {64, 128, 2 * P * 8, 2 * P * n * 8};
-  const cuuint32_t box[5] = {(cuuint32_t)TW, zaxis ? 2u : 1u, 1u, zaxis ? 1u : (cuuint32_t)std::min(N, 256),
-                             zaxis ? (cuuint32_t)std::min(N / 2, 256) : 1u};
+  const cuuint64_t dims[5] = {8, HQ, P / 8, n, n / HQ};
+  const cuuint64_t strides[4] = {64, 64 * HQ, HQ * P * 8, HQ * P * n * 8};
+  const cuuint32_t box[5] = {(cuuint32_t)TW, zaxis ? (cuuint32_t)HQ : 1u, 1u, zaxis ? 1u : (cuuint32_t)std::min(N, 256),
+                             zaxis ? (cuuint32_t)std::min(N / HQ, 256) : 1u};
   const cuuint32_t es[5] = {1, 1, 1, 1, 1};
   return encode(&map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 5, const_cast<float2*>(base), dims, strides, box, es,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -2274,7 +2282,7 @@ static bool spectrum_map(CUtensorMap& map, const float2* base, int N, int TW, bo
 }
 
 // TMA staging applies to single-simulation launches of 1024-point columns
-// (tiles of at most one 64-byte half chunk).  Measured on GB300 (ms per launch
+// (tiles of at most one 64-byte chunk).  Measured on GB300 (ms per launch
 // against cp.async staging): z force pass 5.09 -> 4.57, screening-field z pass
 // 3.24 -> 3.05, y passes 1-2 % faster; at N = 512 the plain y pass runs two
 // CTAs per SM at 128 registers and lost (0.187 -> 0.222).

@@ -68,10 +68,10 @@ struct Mode {
 // elements (kx > N/2) are not valid.
 __device__ __forceinline__ Mode mode_of(int64_t m, int N, int64_t P, bool& valid) {
   Mode md;
-  const int64_t pr = m / (2 * P);            // (z >> 1) N + y
-  const int w = (int)(m - pr * 2 * P);       // position in the interleaved row pair
-  const int ix = (w >> 4) * 8 + (w & 7);
-  const int iy = (int)(pr % N), iz = (int)(pr / N) * 2 + ((w >> 3) & 1);
+  const int64_t g = m / (HQ * P);            // (z / HQ) N + y
+  const int w = (int)(m - g * HQ * P);       // position in the interleaved rows
+  const int ix = w / (8 * HQ) * 8 + (w & 7);
+  const int iy = (int)(g % N), iz = (int)(g / N) * HQ + (w >> 3) % HQ;
   valid = ix <= N / 2;
   md.ix = ix;
   md.fy = iy < N / 2 ? iy : iy - N;
@@ -231,8 +231,8 @@ __global__ void k_absmax(int64_t n, int N, int64_t P, const float2* __restrict__
   float mx = 0.f;
   for (int64_t m = (int64_t)blockIdx.x * NTI + threadIdx.x; m < n;
        m += (int64_t)gridDim.x * NTI) {
-    const int w = (int)(m % (2 * P));
-    if ((w >> 4) * 8 + (w & 7) > N / 2) continue;  // padding (kx > N/2)
+    const int w = (int)(m % (HQ * P));
+    if (w / (8 * HQ) * 8 + (w & 7) > N / 2) continue;  // padding (kx > N/2)
     const float2 v = src[m];
     mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y)));
   }
