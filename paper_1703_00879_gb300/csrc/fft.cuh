@@ -317,6 +317,198 @@ __device__ __forceinline__ void fft_tile(float2* __restrict__ buf, const float2*
   __syncthreads();
 }
 
+// A forward transform whose outputs feed an inverse one (the k-space operations of
+// the z passes) stays in registers in between: after step 2 thread (c, k1) holds
+// X[k1 + R1 k2], and those are the inputs n = n2 + R2' n1 of the inverse
+// transform's first-step items n2 = k1 + R1 h, h < R2' / R1 (R1', R2' its split).
+// So the operation, the inverse's first DFTs and their twiddles follow on the
+// same registers: per point and warp 8 shared-memory wavefronts for the two
+// transforms instead of 12 (16 with the operation in a pass of its own), and 5
+// barriers instead of 8.  Screening-field pass 2.85 -> 2.35 ms at 1024^3.
+
+// Radix of the forward transform's first step: the split's own, or the larger of
+// the two where the middle would otherwise have fewer items than threads.
+template <int L, int TW, int NT>
+__host__ __device__ constexpr int fused_r1() {
+  return Split<L>::R1 < Split<L>::R2 && TW * Split<L>::R1 < NT ? Split<L>::R2 : Split<L>::R1;
+}
+
+// Step 1 of a column transform (split R1 x R2) up to its intermediate in the tile;
+// the caller synchronises before step 2.
+template <int R1, int R2, int TW, int PITCH, int NT, bool INV, class Load>
+__device__ __forceinline__ void col_step1(float2* __restrict__ buf, const float2* __restrict__ tw, Load ld) {
+  constexpr int U = TW * R2, P = (U + NT - 1) / NT;
+  float2 v[P][R1];
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    const int u = threadIdx.x + i * NT;
+    if ((U % NT) == 0 || u < U) {
+      const int c = u % TW, n2 = u / TW;
+#pragma unroll
+      for (int n1 = 0; n1 < R1; ++n1)
+        v[i][pos_of<R1>(n1)] = ld(buf, R2 * n1 + n2, c, (R2 * n1 + n2) * PITCH + c);
+      dftR<R1, INV>(v[i]);
+      if (n2 > 0) {
+#pragma unroll
+        for (int k1 = 1; k1 < R1; ++k1) {
+          float2 w = tw[n2 * k1];
+          if (INV) w.y = -w.y;
+          v[i][k1] = cmul(v[i][k1], w);
+        }
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    const int u = threadIdx.x + i * NT;
+    if ((U % NT) == 0 || u < U) {
+      const int c = u % TW, n2 = u / TW;
+      float2* y = buf + n2 * (R1 + 1) * PITCH + c;
+#pragma unroll
+      for (int k1 = 0; k1 < R1; ++k1) y[k1 * PITCH] = v[i][k1];
+    }
+  }
+}
+
+// Step 2 of the forward transform: the item's X[k1 + R1 k2] into y[k2].
+template <int R1, int R2, int PITCH>
+__device__ __forceinline__ void col_fwd2(float2 (&y)[R2], const float2* __restrict__ buf, int c, int k1) {
+  const float2* yr = buf + k1 * PITCH + c;
+#pragma unroll
+  for (int n2 = 0; n2 < R2; ++n2) y[pos_of<R2>(n2)] = yr[n2 * (R1 + 1) * PITCH];
+  dftR<R2, false>(y);
+}
+
+// First step of the inverse transform (split IR1 x IR2) on the R2 forward outputs x
+// of item (c, k1): the intermediate's values into v (items h = 0.., IR1 each).
+template <int R1, int R2, int IR1, int IR2>
+__device__ __forceinline__ void col_inv1(float2 (&v)[R2], const float2 (&x)[R2], const float2* __restrict__ tw,
+                                         int k1) {
+  constexpr int H = IR2 / R1;
+  static_assert(IR2 % R1 == 0 && H * IR1 == R2, "splits");
+#pragma unroll
+  for (int h = 0; h < H; ++h) {
+    float2 t[IR1];
+#pragma unroll
+    for (int n1 = 0; n1 < IR1; ++n1) t[pos_of<IR1>(n1)] = x[h + H * n1];
+    dftR<IR1, true>(t);
+    const int n2 = k1 + R1 * h;
+    v[h * IR1] = t[0];
+#pragma unroll
+    for (int k = 1; k < IR1; ++k) v[h * IR1 + k] = n2 > 0 ? cmul(t[k], cconj(tw[n2 * k])) : t[k];
+  }
+}
+
+// ... and from v into the tile (intermediate rows n2 (IR1 + 1) + k).
+template <int R1, int R2, int IR1, int IR2, int PITCH>
+__device__ __forceinline__ void col_inv1_store(float2* __restrict__ buf, const float2 (&v)[R2], int c, int k1) {
+#pragma unroll
+  for (int h = 0; h < IR2 / R1; ++h) {
+    float2* y = buf + (k1 + R1 * h) * (IR1 + 1) * PITCH + c;
+#pragma unroll
+    for (int k = 0; k < IR1; ++k) y[k * PITCH] = v[h * IR1 + k];
+  }
+}
+
+// Last step of an inverse transform from the tile's intermediate to the store hook
+// (one that writes the outputs itself); no barrier.
+template <int R1, int R2, int TW, int PITCH, int NT, class Store>
+__device__ __forceinline__ void col_inv2(const float2* __restrict__ buf, Store st) {
+  static_assert(!Store::kSmem, "outputs leave from registers");
+  constexpr int U = TW * R1, P = (U + NT - 1) / NT;
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    const int u = threadIdx.x + i * NT;
+    if ((U % NT) == 0 || u < U) {
+      const int c = u % TW, k1 = u / TW;
+      const float2* yr = buf + k1 * PITCH + c;
+      float2 y[R2];
+#pragma unroll
+      for (int n2 = 0; n2 < R2; ++n2) y[pos_of<R2>(n2)] = yr[n2 * (R1 + 1) * PITCH];
+      dftR<R2, true>(y);
+#pragma unroll
+      for (int k2 = 0; k2 < R2; ++k2) {
+        const int n = k1 + R1 * k2;
+        st(y[k2], n, c, n * PITCH + c);
+      }
+    }
+  }
+}
+
+// Forward transform of the tile's TW columns, x = mid(X[n], n, c, at) on every value,
+// inverse transform of x to st.  mid.ready() runs in every thread before the barrier
+// ahead of mid.  The caller synchronises before the call and before it reuses the tile.
+template <int L, int TW, int PITCH, int NT, class Mid, class Store>
+__device__ __forceinline__ void fft_tile_fwd_inv(float2* __restrict__ buf, const float2* __restrict__ tw, Mid mid,
+                                                 Store st) {
+  constexpr int R1 = fused_r1<L, TW, NT>(), R2 = L / R1, IR1 = Split<L>::R1, IR2 = Split<L>::R2;
+  constexpr int U = TW * R1, P = (U + NT - 1) / NT;
+  static_assert(PITCH % 4 == 0, "column tiles: row pitch a multiple of 4");
+  col_step1<R1, R2, TW, PITCH, NT, false>(buf, tw, TileLoad{});
+  mid.ready();
+  __syncthreads();
+  float2 v[P][R2];
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    const int u = threadIdx.x + i * NT;
+    if ((U % NT) == 0 || u < U) {
+      const int c = u % TW, k1 = u / TW;
+      float2 y[R2];
+      col_fwd2<R1, R2, PITCH>(y, buf, c, k1);
+#pragma unroll
+      for (int k2 = 0; k2 < R2; ++k2) y[k2] = mid(y[k2], k1 + R1 * k2, c, (k1 + R1 * k2) * PITCH + c);
+      col_inv1<R1, R2, IR1, IR2>(v[i], y, tw, k1);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    const int u = threadIdx.x + i * NT;
+    if ((U % NT) == 0 || u < U) col_inv1_store<R1, R2, IR1, IR2, PITCH>(buf, v[i], u % TW, u / TW);
+  }
+  __syncthreads();
+  col_inv2<IR1, IR2, TW, PITCH, NT>(buf, st);
+}
+
+// The same with two inverse transforms, of x = mid(X) to st and of grad(x, n) to st2, one
+// after the other; x stays in registers in between.  after() runs in every thread once
+// all of mid's reads are done.
+template <int L, int TW, int PITCH, int NT, class Mid, class Grad, class After, class Store>
+__device__ __forceinline__ void fft_tile_fwd_inv2(float2* __restrict__ buf, const float2* __restrict__ tw, Mid mid,
+                                                  Grad grad, After after, Store st, Store st2) {
+  constexpr int R1 = fused_r1<L, TW, NT>(), R2 = L / R1, IR1 = Split<L>::R1, IR2 = Split<L>::R2;
+  constexpr int U = TW * R1;
+  static_assert(PITCH % 4 == 0, "column tiles: row pitch a multiple of 4");
+  static_assert(U <= NT, "one middle item per thread");
+  col_step1<R1, R2, TW, PITCH, NT, false>(buf, tw, TileLoad{});
+  mid.ready();
+  __syncthreads();
+  const int c = threadIdx.x % TW, k1 = threadIdx.x / TW;
+  const bool on = U == NT || threadIdx.x < U;
+  float2 x[R2], v[R2];
+  if (on) {
+    col_fwd2<R1, R2, PITCH>(x, buf, c, k1);
+#pragma unroll
+    for (int k2 = 0; k2 < R2; ++k2) x[k2] = mid(x[k2], k1 + R1 * k2, c, (k1 + R1 * k2) * PITCH + c);
+    col_inv1<R1, R2, IR1, IR2>(v, x, tw, k1);
+  }
+  __syncthreads();
+  after();
+  if (on) col_inv1_store<R1, R2, IR1, IR2, PITCH>(buf, v, c, k1);
+  __syncthreads();
+  col_inv2<IR1, IR2, TW, PITCH, NT>(buf, st);
+  if (on) {
+#pragma unroll
+    for (int k2 = 0; k2 < R2; ++k2) x[k2] = grad(x[k2], k1 + R1 * k2);
+    col_inv1<R1, R2, IR1, IR2>(v, x, tw, k1);
+  }
+  __syncthreads();
+  if (on) col_inv1_store<R1, R2, IR1, IR2, PITCH>(buf, v, c, k1);
+  __syncthreads();
+  col_inv2<IR1, IR2, TW, PITCH, NT>(buf, st2);
+}
+
 // Row pitch (complex values) of a row-major tile transformed in place by
 // fft_rowtile<L>: at least L + R2 - 1 (room for the padded intermediate) and
 // 8 mod 16, so that the half-warps of both steps hit distinct bank pairs.

@@ -70,10 +70,21 @@ constexpr size_t col_smem_c(int N, int NBUF) {
 }
 // the same for an explicit tile width
 constexpr size_t col_smem_tw(int N, int TW) { return (N + 2 * (size_t)col_rows(N) * TW) * 8; }
-// Tile width of the fused force-side z passes: 128-byte tile rows at N = 512
-// (the z stride is N P 8 bytes; longer contiguous rows per DRAM page), the
-// column default elsewhere.
-constexpr int ztw(int N) { return N == 512 ? 16 : col_tw(N, 1); }
+// Tiles and threads of the fused force-side z passes (screening field, force).  What
+// bounds them is latency: two or three transforms per tile, each a chain of shared
+// memory, arithmetic and barriers, at about 40 % of the issue and half of the DRAM
+// rate.  Small CTAs that keep every thread busy in every step and drift apart hide it:
+// 128 threads on 8 columns (16 up to 128 points) with all the registers the items of a
+// radix-32 step take.  Per launch, against one or two CTAs of 256 threads (half of them
+// idle in the longer step below 1024 points), us, screening field / force: 512^3 mesh
+// 326 / 565 -> 271 / 498, 256^3 47 / 80 -> 42 / 59, 256 meshes of 128^3 642 / 1148 ->
+// 533 / 964.  At 1024 points two tiles of 8 columns fill shared memory (one CTA of 256
+// threads); 4-column tiles in CTAs of 128 threads lose more to their 32-byte rows
+// (2.35 / 4.17 -> 2.84 / 4.94 ms).
+constexpr int ztw(int N) { return N == 256 ? 8 : col_tw(N, 1); }
+constexpr int zt(int N) { return N <= 512 ? 128 : NT; }
+// Resident CTAs per SM they are compiled for (shared memory; 3 at 512 points: 295 us).
+constexpr int zblocks(int N) { return N <= 256 ? 4 : N <= 512 ? 2 : 1; }
 
 int sm_count() {
   static int n = 0;
@@ -98,7 +109,7 @@ std::vector<KernelInfo> g_kinfo;
 
 // Sets the shared-memory limit of a kernel once and caches its resident CTAs per SM.
 template <class K>
-cudaError_t resident_ctas(K kernel, size_t smem, int& per_sm) {
+cudaError_t resident_ctas(K kernel, size_t smem, int& per_sm, int threads) {
   std::lock_guard<std::mutex> lk(g_kinfo_mu);
   for (const KernelInfo& k : g_kinfo)
     if (k.fn == (const void*)kernel && k.smem == smem) {
@@ -109,7 +120,7 @@ cudaError_t resident_ctas(K kernel, size_t smem, int& per_sm) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, smem);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
   if (e != cudaSuccess) return e;
   g_kinfo.push_back({(const void*)kernel, smem, per_sm});
   return cudaSuccess;
@@ -118,10 +129,10 @@ cudaError_t resident_ctas(K kernel, size_t smem, int& per_sm) {
 // Persistent grid: resident CTAs x SMs, at most one CTA per tile, at most the
 // calling thread's grid cap (used when many small simulations run concurrently).
 template <class K>
-cudaError_t prep(K kernel, size_t smem, int64_t ntiles, unsigned& grid) {
+cudaError_t prep(K kernel, size_t smem, int64_t ntiles, unsigned& grid, int threads = NT) {
   if (ntiles >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;  // tile indices are 32-bit
   int per_sm = 0;
-  cudaError_t e = resident_ctas(kernel, smem, per_sm);
+  cudaError_t e = resident_ctas(kernel, smem, per_sm, threads);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   int64_t g = std::min<int64_t>(ntiles, (int64_t)per_sm * sm_count());
@@ -130,8 +141,9 @@ cudaError_t prep(K kernel, size_t smem, int64_t ntiles, unsigned& grid) {
   return cudaSuccess;
 }
 
+template <int T = NT>
 __device__ __forceinline__ void load_tw(float2* tw, const float2* __restrict__ twg, int n) {
-  for (int i = threadIdx.x; i < n; i += NT) tw[i] = twg[i];
+  for (int i = threadIdx.x; i < n; i += T) tw[i] = twg[i];
 }
 
 // Twiddles of an x pass over rows of N reals (M = N/2 complex): entries 0..M the
@@ -166,11 +178,11 @@ __device__ __forceinline__ void cp_async_wait() {
 // (n mod HQ) rb (the half-spectrum layout of cola_internal.h); only columns
 // c0 + c < N/2 + 1 exist.  Each thread keeps one 16-byte piece (or one column)
 // and walks rows n0, n0 + step, ... (HQ | step, so n mod HQ stays fixed).
-template <int N, int TW, int TP>
+template <int N, int TW, int TP, int T = NT>
 __device__ __forceinline__ void col_issue(float2* buf, int sub, const float2* __restrict__ g,
                                           int64_t base, int64_t ra, int64_t rb, int c0) {
   constexpr int CH = TW / 2;  // 16-byte pieces per row segment
-  constexpr int STEP = NT / CH;
+  constexpr int STEP = T / CH;
   static_assert(STEP % HQ == 0, "row step: whole plane groups");
   const int j = threadIdx.x % CH, n0 = threadIdx.x / CH;
   const bool v = c0 + 2 * j < N / 2 + 1;
@@ -293,12 +305,14 @@ struct ColGeo {
 
 // Software pipeline over the tiles of one launch.  Op supplies
 //   issue(buf, t): cp.async the inputs of tile t into buf (no commit)
-//   issue_side(t): cp.async of a second input of tile t into op.extra (no commit;
-//     may do nothing); its group is committed BEFORE the next tile's prefetch,
-//     so process() can wait for it with cp_async_wait<1>() while the prefetch
-//     of tile t + grid stays in flight
 //   process(buf, tw, t): transform + store (leaves buf free after a final barrier)
-template <int N, int BUFELEMS, class Op>
+// and, with kSide (a second input, landing in op.extra),
+//   issue_side(t): cp.async of tile t's second input (no commit)
+//   process(buf, tw, t, next): next() once op.extra has been read; it issues the
+//     next tile's second input and commits it, so that it lands while this tile's
+//     outputs are formed.  process() waits for its own with cp_async_wait<1>(),
+//     which leaves the prefetch of tile t + grid in flight.
+template <int N, int BUFELEMS, int T = NT, class Op>
 __device__ __forceinline__ void col_pipeline(Op op, const float2* __restrict__ twg,
                                              int64_t ntiles) {
   extern __shared__ __align__(128) float2 sm[];
@@ -306,20 +320,29 @@ __device__ __forceinline__ void col_pipeline(Op op, const float2* __restrict__ t
   float2* b0 = sm + N;
   float2* b1 = b0 + BUFELEMS;
   op.extra = b1 + BUFELEMS;  // optional per-op scratch after the two stage buffers
-  load_tw(tw, twg, N);
+  load_tw<T>(tw, twg, N);
   int64_t t = blockIdx.x;
   if (t < ntiles) op.issue(b0, t);
   cp_async_commit();
+  if constexpr (Op::kSide) {
+    if (t < ntiles) op.issue_side(t);
+    cp_async_commit();
+  }
   int cur = 0;
   for (; t < ntiles; t += gridDim.x) {
-    op.issue_side(t);  // op.extra is free: the previous tile ended with a barrier
-    cp_async_commit();
     const int64_t tn = t + gridDim.x;
     if (tn < ntiles) op.issue(cur ? b0 : b1, tn);
     cp_async_commit();
-    cp_async_wait<2>();  // tile t's main input has landed
+    cp_async_wait<Op::kSide ? 2 : 1>();  // tile t's main input has landed
     __syncthreads();
-    op.process(cur ? b1 : b0, tw, t);
+    if constexpr (Op::kSide) {
+      op.process(cur ? b1 : b0, tw, t, [&] {
+        if (tn < ntiles) op.issue_side(tn);
+        cp_async_commit();
+      });
+    } else {
+      op.process(cur ? b1 : b0, tw, t);
+    }
     __syncthreads();
     cur ^= 1;
   }
@@ -457,7 +480,7 @@ constexpr size_t tma_smem() {
   return ((size_t)N + 2 * (size_t)BUFELEMS + EXTRA) * sizeof(float2) + 4 * sizeof(uint64_t);
 }
 
-template <int N, int BUFELEMS, bool SIDE, int EXTRA, class Op>
+template <int N, int BUFELEMS, bool SIDE, int EXTRA, int T, class Op>
 __device__ __forceinline__ void col_pipeline_tma(Op op, const float2* __restrict__ twg, int64_t ntiles,
                                                  const CUtensorMap* map0, const CUtensorMap* map1) {
   static_assert((N * sizeof(float2)) % 128 == 0 && (BUFELEMS * sizeof(float2)) % 128 == 0,
@@ -477,7 +500,7 @@ __device__ __forceinline__ void col_pipeline_tma(Op op, const float2* __restrict
     fence_bar_init();
     fail = (smem_u32(sm) & 127) ? 1 : 0;  // no copy goes into a misaligned buffer
   }
-  load_tw(tw, twg, N);
+  load_tw<T>(tw, twg, N);
   __syncthreads();
   if (fail) {
     if (lead) atomicAdd(&g_tile_load_failures, 1u);
@@ -490,16 +513,16 @@ __device__ __forceinline__ void col_pipeline_tma(Op op, const float2* __restrict
   if (lead && t < ntiles) {
     tma_tile(op.geo, map0, b0, t, &bars[0]);
     pend |= 1u;
+    if (SIDE) {
+      tma_tile(op.geo, map1, op.extra, t, &bars[2]);
+      pend |= 4u;
+    }
   }
   int cur = 0;
   for (; t < ntiles; t += gridDim.x) {
+    const int64_t tn = t + gridDim.x;
     if (lead) {
-      fence_async_smem();  // the previous tile's accesses to the buffers and to extra are done
-      if (SIDE) {
-        tma_tile(op.geo, map1, op.extra, t, &bars[2]);
-        pend |= 4u;
-      }
-      const int64_t tn = t + gridDim.x;
+      fence_async_smem();  // the previous tile's accesses to the buffers are done
       if (tn < ntiles) {
         tma_tile(op.geo, map0, cur ? b0 : b1, tn, &bars[cur ^ 1]);
         pend |= 1u << (cur ^ 1);
@@ -513,14 +536,27 @@ __device__ __forceinline__ void col_pipeline_tma(Op op, const float2* __restrict
     }
     __syncthreads();
     if (fail) break;
-    if constexpr (SIDE) op.side = TmaSide{&bars[2], (par >> 2) & 1u, &fail};
-    op.process(cur ? b1 : b0, tw, t);
+    if constexpr (SIDE) {
+      op.side = TmaSide{&bars[2], (par >> 2) & 1u, &fail};
+      // after the tile's second input has been read: the next tile's (unless this one's
+      // wait ran out, in which case its copy is still pending)
+      op.process(cur ? b1 : b0, tw, t, [&] {
+        if (!lead || fail) return;
+        par ^= 4u;
+        pend &= ~4u;
+        if (tn < ntiles) {
+          fence_async_smem();
+          tma_tile(op.geo, map1, op.extra, tn, &bars[2]);
+          pend |= 4u;
+        }
+      });
+    } else if constexpr (Op::kSide) {
+      op.process(cur ? b1 : b0, tw, t, [] {});
+    } else {
+      op.process(cur ? b1 : b0, tw, t);
+    }
     __syncthreads();
     if (fail) break;
-    if (SIDE && lead) {
-      par ^= 4u;
-      pend &= ~4u;
-    }
     cur ^= 1;
   }
   if (lead && fail) {
@@ -551,7 +587,7 @@ struct OpCol {
   const float2* in;
   float2* out;
   float2* extra = nullptr;  // scratch after the stage buffers (set by col_pipeline)
-  __device__ __forceinline__ void issue_side(int64_t) const {}
+  static constexpr bool kSide = false;
   __device__ __forceinline__ void issue(float2* buf, int64_t t) const {
     int o, c0;
     int64_t base, by;
@@ -571,7 +607,7 @@ struct OpCol {
 template <int N, int TW, bool INV, bool TMA>
 __global__ void __launch_bounds__(NT, blocks_for_smem(col_smem_c(N, 1), N)) k_col(OpCol<N, TW, INV> op, const float2* __restrict__ twg,
                                             int64_t ntiles, const __grid_constant__ CUtensorMap map) {
-  if constexpr (TMA) col_pipeline_tma<N, fft_rows<N>() * TW, false, 0>(op, twg, ntiles, &map, nullptr);
+  if constexpr (TMA) col_pipeline_tma<N, fft_rows<N>() * TW, false, 0, NT>(op, twg, ntiles, &map, nullptr);
   else col_pipeline<N, fft_rows<N>() * TW>(op, twg, ntiles);
 }
 
@@ -611,7 +647,7 @@ struct OpYinv2 {
   float2 *outp, *outd;
   float kfs;
   float2* extra = nullptr;  // scratch after the stage buffers (set by col_pipeline)
-  __device__ __forceinline__ void issue_side(int64_t) const {}
+  static constexpr bool kSide = false;
   __device__ __forceinline__ void issue(float2* buf, int64_t t) const {
     int o, c0;
     int64_t base, by;
@@ -806,12 +842,11 @@ __device__ __forceinline__ float smoothing_window(float h, int filter) {
 // smoothed by the Gaussian window; 3 the density smoothed by the top-hat or
 // sharp-k window (fp.filter).  The Gaussian keeps a kernel of its own: a
 // per-element switch over the windows slows the pass by a third.
-template <int N, int TW, int MODEL>
+template <int N, int TW, int MODEL, int T>
 struct OpZScreenField {
-  // Store hook of the forward transform: delta(k) out to HBM, the field's
-  // multiplier (-kappa/k^2, or the smoothing window) applied in place.
+  // Between the forward and the inverse transform: delta(k) out to HBM, the field's
+  // multiplier (-kappa/k^2, or the smoothing window) applied.
   struct Field {
-    static constexpr bool kSmem = true;
     float2* dk;  // delta(k) of the tile: element (n, c) at dk[(n / HQ) ra + (n mod HQ) rb + hcol(c)]
     int64_t ra, rb;
     int c0, fy2;
@@ -836,12 +871,12 @@ struct OpZScreenField {
   float2 *dk_out, *w_out;
   ForceParams fp;
   float2* extra = nullptr;  // scratch after the stage buffers (set by col_pipeline)
-  __device__ __forceinline__ void issue_side(int64_t) const {}
+  static constexpr bool kSide = false;
   __device__ __forceinline__ void issue(float2* buf, int64_t t) const {
     int o, c0;
     int64_t base, by;
     geo.tile(t, o, c0, base, by);
-    col_issue<N, TW, TW>(buf, 0, moved(in, by), base, geo.ra, geo.rb, c0);
+    col_issue<N, TW, TW, T>(buf, 0, moved(in, by), base, geo.ra, geo.rb, c0);
   }
   __device__ __forceinline__ void process(float2* buf, const float2* tw, int64_t t) const {
     int iy, c0;
@@ -852,39 +887,35 @@ struct OpZScreenField {
     const int fy = freq_index(iy, N);
     const Field f{moved(dk_out, by) + base, geo.ra, geo.rb, c0, fy * fy, fp.kf * fp.kf, fp.kappa_norm,
                   fp.R2half, fp.norm, fp.filter};
-    fft_tile_call<N, TW, TW, NT, false, 1, TileLoad, Field>(buf, tw, TileLoad{}, f);
-    fft_tile_call<N, TW, TW, NT, true, 1, TileLoad, ColOut>(
-        buf, tw, TileLoad{}, ColOut{moved(w_out, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0});
+    fft_tile_fwd_inv<N, TW, TW, T>(buf, tw, f, ColOut{moved(w_out, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0});
   }
 };
 
-template <int N, int TW, int MODEL, bool TMA>
-__global__ void __launch_bounds__(NT, blocks_for_smem(col_smem_tw(N, TW), N) < 2 ? 1 : 2) k_z_screen_field(OpZScreenField<N, TW, MODEL> op,
+template <int N, int TW, int MODEL, bool TMA, int T>
+__global__ void __launch_bounds__(T, zblocks(N)) k_z_screen_field(OpZScreenField<N, TW, MODEL, T> op,
                                                        const float2* __restrict__ twg,
                                                        int64_t ntiles, const __grid_constant__ CUtensorMap map) {
   if (!op.geo.m.shift) resolve(op.fp, 0);  // one simulation: once per launch
-  if constexpr (TMA) col_pipeline_tma<N, fft_rows<N>() * TW, false, 0>(op, twg, ntiles, &map, nullptr);
-  else col_pipeline<N, fft_rows<N>() * TW>(op, twg, ntiles);
+  if constexpr (TMA) col_pipeline_tma<N, fft_rows<N>() * TW, false, 0, T>(op, twg, ntiles, &map, nullptr);
+  else col_pipeline<N, fft_rows<N>() * TW, T>(op, twg, ntiles);
 }
 
 // ---------------------------------------------------------------- force (z pass)
 // Per tile: the source (S, or delta when unscreened) is staged and transformed
 // forward while delta(k) lands in a second shared-memory tile (screened runs);
-// Phi_tot(k) is formed from both and kept in that second tile, and the two
-// outputs (Phi and -i kz Phi) are inverse transformed one after the other in
-// the staging buffer and stored to HBM.
-template <int N, int TW, bool SCREENED>
+// Phi_tot(k) is formed from both in registers, and the inverse transforms of Phi
+// and of -i kz Phi start from there.  The next tile's delta(k) is on its way while
+// they run.
+template <int N, int TW>
+constexpr size_t zforce_smem() {  // twiddles, two stage buffers, delta(k)
+  return col_smem_tw(N, TW) + (size_t)N * TW * sizeof(float2);
+}
+template <int N, int TW, bool SCREENED, int T>
 struct OpZForce {
-  // One CTA per SM (N >= 512, up to 255 registers): Phi_tot(k) is formed in the
-  // forward transform's last store; with two CTAs (128 registers) that spills,
-  // and a separate pass over the tile forms it instead.
-  static constexpr bool FUSED = blocks_for_smem(col_smem_tw(N, TW) + (size_t)N * TW * 8, N) < 2;
-  // Store hook of the forward transform of S: Phi_tot(k) (App. B), written to
-  // the buffer for the Phi inverse and to `ph` (which held delta(k)) for the
-  // gradient; ready() waits for this tile's delta(k) between the two steps.
+  // Phi_tot(k) (App. B) from the transform of S and delta(k) in `dk`; ready() waits for
+  // this tile's delta(k) between the forward transform's steps.
   struct Combine {
-    static constexpr bool kSmem = true;
-    float2* ph;
+    const float2* dk;
     int c0, fy2;
     float kf2, a2m2, kappa_norm, C;
     __device__ __forceinline__ float2 operator()(float2 src, int n, int c, int at) const {
@@ -894,10 +925,9 @@ struct OpZForce {
       if (k2 > 0.f) {
         const float yuk = __fdividef(k2, k2 + a2m2);
         const float g = __fdividef(-kappa_norm, k2);
-        if (SCREENED) phi = cscale(cadd(ph[at], cscale(src, C * yuk)), g);
+        if (SCREENED) phi = cscale(cadd(dk[at], cscale(src, C * yuk)), g);
         else phi = cscale(src, g * (1.f + C * yuk));
       }
-      ph[at] = phi;
       return phi;
     }
     TmaSide side;  // TMA staging: the barrier of delta(k)'s copy
@@ -907,13 +937,12 @@ struct OpZForce {
       else cp_async_wait<1>();    // delta(k); the next tile's prefetch may stay in flight
     }
   };
-  // Load hook of the gradient transform: -i kz Phi_tot(k), zero on the Nyquist row.
+  // -i kz Phi_tot(k), zero on the Nyquist row.
   struct GradZ {
-    const float2* ph;
     float mkf;
-    __device__ __forceinline__ float2 operator()(const float2*, int n, int, int at) const {
+    __device__ __forceinline__ float2 operator()(float2 phi, int n) const {
       const float kzs = (n == N / 2) ? 0.f : mkf * (float)freq_index(n, N);
-      return cscale(cmul_i(ph[at]), kzs);
+      return cscale(cmul_i(phi), kzs);
     }
   };
   ColGeo<N, TW> geo;
@@ -926,75 +955,40 @@ struct OpZForce {
     int o, c0;
     int64_t base, by;
     geo.tile(t, o, c0, base, by);
-    col_issue<N, TW, TW>(buf, 0, moved(in, by), base, geo.ra, geo.rb, c0);
+    col_issue<N, TW, TW, T>(buf, 0, moved(in, by), base, geo.ra, geo.rb, c0);
   }
+  static constexpr bool kSide = true;
   // delta(k) of the tile into extra; lands while S is transformed
   __device__ __forceinline__ void issue_side(int64_t t) const {
     if (SCREENED) {
       int o, c0;
       int64_t base, by;
       geo.tile(t, o, c0, base, by);
-      col_issue<N, TW, TW>(extra, 0, moved(dk, by), base, geo.ra, geo.rb, c0);
+      col_issue<N, TW, TW, T>(extra, 0, moved(dk, by), base, geo.ra, geo.rb, c0);
     }
   }
-  __device__ __forceinline__ void process(float2* buf, const float2* tw, int64_t t) const {
+  template <class Next>
+  __device__ __forceinline__ void process(float2* buf, const float2* tw, int64_t t, Next next) const {
     int iy, c0;
     int64_t base, by;
     geo.tile(t, iy, c0, base, by);
     ForceParams fp = this->fp;
     resolve(fp, by);
-    float2* ph = extra;  // delta(k) of the tile, then Phi_tot(k), N x TW
     const int fy = freq_index(iy, N);
-    const Combine cmb{ph, c0, fy * fy, fp.kf * fp.kf, fp.a2m2, fp.kappa_norm, fp.C, side};
-    if constexpr (FUSED) {
-      fft_tile_call<N, TW, TW, NT, false, 1, TileLoad, Combine>(buf, tw, TileLoad{}, cmb);
-    } else {
-      fft_tile_call<N, TW, TW, NT, false>(buf, tw);
-      cmb.ready();
-      __syncthreads();
-      const TileLane<N, TW> ln(c0, iy);
-#pragma unroll 4
-      for (int i = 0; i < ln.E; ++i) {
-        const int n = ln.row(i), at = n * TW + ln.c;
-        buf[at] = cmb(buf[at], n, ln.c, at);
-      }
-      __syncthreads();
-    }
-    const GradZ grad{ph, -fp.kf};
-    if constexpr (FUSED) {
-      // both inverse transforms store straight to HBM; the gradient transform
-      // reads ph, not the tile
-      const ColOut o{nullptr, geo.ra, geo.rb, N / 2 + 1 - c0};
-      ColOut op = o, oz = o;
-      op.g = moved(phi_out, by) + base;
-      oz.g = moved(phiz_out, by) + base;
-      fft_tile_call<N, TW, TW, NT, true, 1, TileLoad, ColOut>(buf, tw, TileLoad{}, op);
-      fft_tile_call<N, TW, TW, NT, true, 1, GradZ, ColOut>(buf, tw, grad, oz);
-    } else {
-      const ColOut o{nullptr, geo.ra, geo.rb, N / 2 + 1 - c0};
-      ColOut op = o, oz = o;
-      op.g = moved(phi_out, by) + base;
-      oz.g = moved(phiz_out, by) + base;
-      fft_tile_call<N, TW, TW, NT, true, 1, TileLoad, ColOut>(buf, tw, TileLoad{}, op);
-      const TileLane<N, TW> ln(c0, iy);
-#pragma unroll 4
-      for (int i = 0; i < ln.E; ++i) {
-        const int n = ln.row(i), at = n * TW + ln.c;
-        buf[at] = grad(buf, n, ln.c, at);
-      }
-      __syncthreads();
-      fft_tile_call<N, TW, TW, NT, true, 1, TileLoad, ColOut>(buf, tw, TileLoad{}, oz);
-    }
+    const Combine cmb{extra, c0, fy * fy, fp.kf * fp.kf, fp.a2m2, fp.kappa_norm, fp.C, side};
+    const ColOut op{moved(phi_out, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0};
+    const ColOut oz{moved(phiz_out, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0};
+    fft_tile_fwd_inv2<N, TW, TW, T>(buf, tw, cmb, GradZ{-fp.kf}, next, op, oz);
   }
 };
 
-template <int N, int TW, bool SCREENED, bool TMA>
-__global__ void __launch_bounds__(NT, blocks_for_smem(col_smem_tw(N, TW) + (size_t)N * TW * 8, N) < 2 ? 1 : 2) k_z_force(
-    OpZForce<N, TW, SCREENED> op, const float2* __restrict__ twg, int64_t ntiles,
+template <int N, int TW, bool SCREENED, bool TMA, int T>
+__global__ void __launch_bounds__(T, zblocks(N)) k_z_force(
+    OpZForce<N, TW, SCREENED, T> op, const float2* __restrict__ twg, int64_t ntiles,
     const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap dmap) {
   if (!op.geo.m.shift) resolve(op.fp, 0);  // one simulation: once per launch
-  if constexpr (TMA) col_pipeline_tma<N, fft_rows<N>() * TW, SCREENED, N * TW>(op, twg, ntiles, &map, &dmap);
-  else col_pipeline<N, fft_rows<N>() * TW>(op, twg, ntiles);
+  if constexpr (TMA) col_pipeline_tma<N, fft_rows<N>() * TW, SCREENED, N * TW, T>(op, twg, ntiles, &map, &dmap);
+  else col_pipeline<N, fft_rows<N>() * TW, T>(op, twg, ntiles);
 }
 
 // ---------------------------------------------------------------- LPT reweight (z pass)
@@ -1025,7 +1019,7 @@ struct OpLptZ {
   int64_t zbytes = 0, zchunk = 0;
   float2* extra = nullptr;  // scratch after the stage buffers (set by col_pipeline)
   static constexpr uint32_t kZero = 16384;
-  __device__ __forceinline__ void issue_side(int64_t) const {}
+  static constexpr bool kSide = false;
   __device__ __forceinline__ void issue(float2* buf, int64_t t) const {
     int o, c0;
     int64_t base, by;
@@ -2369,7 +2363,7 @@ cudaError_t fft_yinv2(int Nv, const float2* in, float2* outp, float2* outd, floa
 template <int N>
 static cudaError_t launch_zsf(const float2* in, float2* dk_out, float2* w_out,
                               const ForceParams& fp, const float2* tw, cudaStream_t s, Multi m) {
-  constexpr int TW = ztw(N);
+  constexpr int TW = ztw(N), T = zt(N);
   constexpr size_t sm = col_smem_tw(N, TW);
   const int64_t ntiles = col_tiles<N, TW>() * m.nb;
   CUtensorMap map{};
@@ -2378,11 +2372,11 @@ static cudaError_t launch_zsf(const float2* in, float2* dk_out, float2* w_out,
     constexpr int MODEL = decltype(model)::value;
     constexpr bool TMA = decltype(tma_c)::value;
     constexpr size_t smk = TMA ? tma_smem<N, fft_rows<N>() * TW, 0>() : sm;
-    auto k = k_z_screen_field<N, TW, MODEL, TMA>;
+    auto k = k_z_screen_field<N, TW, MODEL, TMA, T>;
     unsigned grid;
-    cudaError_t e = prep(k, smk, ntiles, grid);
+    cudaError_t e = prep(k, smk, ntiles, grid, T);
     if (e != cudaSuccess) return e;
-    k<<<grid, NT, smk, s>>>(OpZScreenField<N, TW, MODEL>{geo_z<N, TW>(m), in, dk_out, w_out, fp}, tw, ntiles,
+    k<<<grid, T, smk, s>>>(OpZScreenField<N, TW, MODEL, T>{geo_z<N, TW>(m), in, dk_out, w_out, fp}, tw, ntiles,
                             map);
     return cudaGetLastError();
   };
@@ -2437,8 +2431,8 @@ template <int N, bool SCR>
 static cudaError_t launch_zforce_t(const float2* in, const float2* dk, float2* phi,
                                    float2* phiz, const ForceParams& fp,
                                    const float2* tw, cudaStream_t s, Multi m) {
-  constexpr int TW = ztw(N);
-  constexpr size_t sm = col_smem_tw(N, TW) + (size_t)N * TW * sizeof(float2);
+  constexpr int TW = ztw(N), T = zt(N);
+  constexpr size_t sm = zforce_smem<N, TW>();
   const int64_t ntiles = col_tiles<N, TW>() * m.nb;
   CUtensorMap map{}, dmap{};
   const bool tma = tma_shape<N, TW>() && !m.shift && spectrum_map(map, in, N, TW, true) &&
@@ -2446,11 +2440,11 @@ static cudaError_t launch_zforce_t(const float2* in, const float2* dk, float2* p
   auto go = [&](auto tma_c) {
     constexpr bool TMA = decltype(tma_c)::value;
     constexpr size_t smk = TMA ? tma_smem<N, fft_rows<N>() * TW, N * TW>() : sm;
-    auto k = k_z_force<N, TW, SCR, TMA>;
+    auto k = k_z_force<N, TW, SCR, TMA, T>;
     unsigned grid;
-    cudaError_t e = prep(k, smk, ntiles, grid);
+    cudaError_t e = prep(k, smk, ntiles, grid, T);
     if (e != cudaSuccess) return e;
-    k<<<grid, NT, smk, s>>>(OpZForce<N, TW, SCR>{geo_z<N, TW>(m), in, dk, phi, phiz, fp}, tw, ntiles, map,
+    k<<<grid, T, smk, s>>>(OpZForce<N, TW, SCR, T>{geo_z<N, TW>(m), in, dk, phi, phiz, fp}, tw, ntiles, map,
                             dmap);
     return cudaGetLastError();
   };
