@@ -666,14 +666,12 @@ __device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const floa
 // shuffles, one broadcast twiddle read), and one barrier less: x r2c 1.61 ->
 // 1.30 ms and screening x 3.45 -> 3.14 ms at 1024^3, x r2c plane pass 1.21 ->
 // 1.06 ms over 256 meshes of 128^3.  PAIR32 as in fft_rowtile.
-template <int L, int TW, int CW, int NT, class Pre, bool PAIR32, class Store>
-__device__ __forceinline__ void fft_rowtile_r2c(float2* __restrict__ buf, const float2* __restrict__ w1,
-                                                const float2* __restrict__ twr, Pre pre, Store st) {
+template <int L, int TW, int CW, int NT, bool PAIR32, class Store>
+__device__ __forceinline__ void row_r2c_step2(float2* __restrict__ buf, const float2* __restrict__ twr, Store st) {
   constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;
   constexpr int U2 = TW * R1, P2 = (U2 + NT - 1) / NT;
   static_assert(R1 <= 32 && U2 % 32 == 0, "whole warps take part in the shuffles");
   const int tid = threadIdx.x, lane = tid & 31;
-  row_step1<L, TW, CW, NT, false, Pre>(buf, w1, pre);
   auto emit = [&](float2 zk, float2 zm, int c, int k) {
     const float2 b = cconj(zm), E = cscale(cadd(zk, b), 0.5f), D = csub(zk, b);
     const float2 X = cadd(E, cmul(twr[k], make_float2(0.5f * D.y, -0.5f * D.x)));  // O = (-i/2) D
@@ -733,17 +731,88 @@ __device__ __forceinline__ void fft_rowtile_r2c(float2* __restrict__ buf, const 
   __syncthreads();
 }
 
-template <int L, int TW, int CW, int NT, bool INV, class Pre = NoPre, bool PAIR32 = false,
-          class Store = RowStore>
-__device__ __noinline__ void fft_rowtile_call(float2* buf, const float2* w1, Pre pre = Pre(),
-                                              Store st = Store()) {
-  fft_rowtile<L, TW, CW, NT, INV, Pre, PAIR32, Store>(buf, w1, pre, st);
+template <int L, int TW, int CW, int NT, class Pre, bool PAIR32, class Store>
+__device__ __forceinline__ void fft_rowtile_r2c(float2* __restrict__ buf, const float2* __restrict__ w1,
+                                                const float2* __restrict__ twr, Pre pre, Store st) {
+  row_step1<L, TW, CW, NT, false, Pre>(buf, w1, pre);
+  row_r2c_step2<L, TW, CW, NT, PAIR32, Store>(buf, twr, st);
 }
 
-template <int L, int TW, int CW, int NT, class Pre, bool PAIR32, class Store>
-__device__ __noinline__ void fft_rowtile_r2c_call(float2* buf, const float2* w1, const float2* twr, Pre pre,
-                                                  Store st) {
-  fft_rowtile_r2c<L, TW, CW, NT, Pre, PAIR32, Store>(buf, w1, twr, pre, st);
+// Inverse row transform, x = mid(z[n], c, n) on every value, forward real transform
+// of x (fft_rowtile_r2c).  As in the column passes (fft_tile_fwd_inv) the values a
+// thread holds after the inverse are inputs of its own first-step items of the
+// forward transform, n2 = k1 + R1 h, so they stay in registers in between (PAIR32:
+// the thread's 16 values are the item n2 = k1 + 16 half): 6 shared-memory
+// wavefronts per point and warp and three barriers less.
+template <int L, int TW, int CW, int NT, class Pre, class Mid, bool PAIR32, class Store>
+__device__ __forceinline__ void fft_rowtile_inv_r2c(float2* __restrict__ buf, const float2* __restrict__ w1,
+                                                    const float2* __restrict__ twr, Pre pre, Mid mid, Store st) {
+  constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;
+  constexpr int U2 = TW * R1, P2 = (U2 + NT - 1) / NT, H = R2 / R1;
+  const int tid = threadIdx.x;
+  row_step1<L, TW, CW, NT, true, Pre>(buf, w1, pre);
+  if constexpr (PAIR32 && R1 == 16 && R2 == 32 && 2 * U2 == NT) {
+    const int half = (tid >> 4) & 1, c = tid >> 5, k1 = tid & 15, n2 = tid & 31;
+    float2 y[16], v[16];
+    const float2* yr = buf + c * CW + k1 + 16 * half * (R1 + 1);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) y[j] = yr[j * (R1 + 1)];
+    dft32_pair<true>(y, half);
+#pragma unroll
+    for (int n1 = 0; n1 < 16; ++n1) v[pos_of<16>(n1)] = mid(y[n1], c, n2 + 32 * n1);
+    dftR<16, false>(v);
+    if (n2 > 0) {
+#pragma unroll
+      for (int k = 1; k < 16; ++k) v[k] = cmul(v[k], w1[k * R2 + n2]);
+    }
+    __syncthreads();
+    float2* o = buf + c * CW + n2 * (R1 + 1);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) o[k] = v[k];
+  } else {
+    float2 v[P2][R2];
+#pragma unroll
+    for (int i = 0; i < P2; ++i) {
+      const int u = tid + i * NT;
+      if ((U2 % NT) == 0 || u < U2) {
+        const int c = u / R1, k1 = u % R1;
+        const float2* yr = buf + c * CW + k1;
+        float2 y[R2];
+#pragma unroll
+        for (int n2 = 0; n2 < R2; ++n2) y[pos_of<R2>(n2)] = yr[n2 * (R1 + 1)];
+        dftR<R2, true>(y);
+#pragma unroll
+        for (int k2 = 0; k2 < R2; ++k2) y[k2] = mid(y[k2], c, k1 + R1 * k2);
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const int n2 = k1 + R1 * h;
+          float2 t[R1];
+#pragma unroll
+          for (int n1 = 0; n1 < R1; ++n1) t[pos_of<R1>(n1)] = y[h + H * n1];
+          dftR<R1, false>(t);
+          v[i][h * R1] = t[0];
+#pragma unroll
+          for (int k = 1; k < R1; ++k) v[i][h * R1 + k] = n2 > 0 ? cmul(t[k], w1[k * R2 + n2]) : t[k];
+        }
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < P2; ++i) {
+      const int u = tid + i * NT;
+      if ((U2 % NT) == 0 || u < U2) {
+        const int c = u / R1, k1 = u % R1;
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          float2* o = buf + c * CW + (k1 + R1 * h) * (R1 + 1);
+#pragma unroll
+          for (int k = 0; k < R1; ++k) o[k] = v[i][h * R1 + k];
+        }
+      }
+    }
+  }
+  __syncthreads();
+  row_r2c_step2<L, TW, CW, NT, PAIR32, Store>(buf, twr, st);
 }
 
 // Out-of-line copy for kernels that run several transforms per tile: each

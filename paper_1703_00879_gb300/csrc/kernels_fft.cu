@@ -51,9 +51,27 @@ constexpr int col_tw(int N, int NBUF) {
   return (N == 1024 && NBUF == 1) ? 8
          : (4096 / (N * NBUF)) < 4 ? 4 : ((4096 / (N * NBUF)) > 16 ? 16 : 4096 / (N * NBUF));
 }
-// Rows per x-pass tile: about 8192 staged values per tile (~64 KB in flight
-// per CTA pair), 8..64 rows.
-constexpr int row_tw(int N) { return 8192 / N < 8 ? 8 : (8192 / N > 64 ? 64 : 8192 / N); }
+// Tile and CTA of an x pass over rows of N reals: rows per tile, threads, resident
+// CTAs per SM it is compiled for.  RowBig: about 8192 staged values (~64 KB in flight
+// per CTA pair), 8..64 rows, 256 threads.  RowSmall: 128 threads that are all busy in
+// both steps (at 1024 points 8 rows give 128 items of the radix-32 step).
+struct RowShape {
+  int rows, threads, ctas;
+};
+constexpr RowShape row_big(int N) {
+  return N >= 1024 ? RowShape{8, 256, 2} : N == 512 ? RowShape{16, 256, 3} : N == 256 ? RowShape{32, 256, 2} : RowShape{64, 256, 3};
+}
+constexpr RowShape row_small(int N) {
+  return N >= 1024 ? RowShape{8, 128, 2} : N == 512 ? RowShape{8, 128, 5} : N == 256 ? RowShape{16, 128, 5} : N == 128 ? RowShape{16, 128, 6} : RowShape{32, 128, 6};
+}
+// Measured on GB300 (us per launch, big / small): x r2c 1024: 1301 / 1331, 512: 179 / 188,
+// 256: 28.0 / 27.3; force c2r (pair and F_z) 1024: 4332 / 4032, 512: 538 / 540, 256: 82 / 78;
+// LPT c2r (six fields) 512: 1006 / 1091, 256: 139 / 146; screening 1024: 3237 / 3386 (big with
+// its radix-32 step on thread pairs), 512: 351 / 329, 256: 54 / 50.
+constexpr RowShape r2c_shape(int N) { return N == 256 ? row_small(N) : row_big(N); }
+constexpr RowShape c2r_shape(int N) { return N >= 1024 ? row_small(N) : row_big(N); }
+constexpr RowShape pair_shape(int N) { return N >= 1024 || N == 256 ? row_small(N) : row_big(N); }
+constexpr RowShape screen_shape(int N) { return N >= 1024 ? row_big(N) : row_small(N); }
 
 // Resident CTAs per SM that the shared memory of a kernel allows (1..3); used
 // as the register bound of __launch_bounds__ so registers never limit occupancy
@@ -150,10 +168,10 @@ __device__ __forceinline__ void load_tw(float2* tw, const float2* __restrict__ t
 // table exp(-2 pi i k / N) of the real <-> half-spectrum split, entry M + k1 R2 + n2
 // (k1 >= 1) the row transform's first-step twiddle (fft_rowtile), which therefore
 // takes w1 = tw + M.  Together they fill the N entries of the plain table.
-template <int N>
+template <int N, int T>
 __device__ __forceinline__ void load_row_tw(float2* tw, const float2* __restrict__ twg) {
   constexpr int M = N / 2;
-  for (int i = threadIdx.x; i < N; i += NT) {
+  for (int i = threadIdx.x; i < N; i += T) {
     const int j = i - M;
     if (i <= M || j >= Split<M>::R2) tw[i] = twg[i <= M ? i : 2 * row_twiddle<M>(j)];
   }
@@ -1282,9 +1300,9 @@ struct RowCfg {
 // when there are fewer groups than warps; f(group, p0, p1) visits p = p0, p0 +
 // 32, ... < p1 with p0 = segment start + lane (segment starts are multiples of
 // 32, so each warp reads or writes whole lines).
-template <int NG, int LEN, class F>
+template <int T, int NG, int LEN, class F>
 __device__ __forceinline__ void for_groups(F f) {
-  constexpr int NW = NT / 32;
+  constexpr int NW = T / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if constexpr (NG >= NW) {
     for (int g = warp; g < NG; g += NW) f(g, lane, LEN);
@@ -1304,13 +1322,13 @@ __device__ __forceinline__ int piece_col(int p) { return p / (4 * HQ) * 8 + 2 * 
 __device__ __forceinline__ int piece_row(int p) { return (p >> 2) % HQ; }
 
 // Complex half rows (M + 1 values, staged as M + 2 to keep 16-byte pieces).
-template <int N, int TWX>
+template <int N, int TWX, int T>
 __device__ __forceinline__ void stage_complex_rows(float2* st, const float2* __restrict__ in,
                                                    int64_t q0) {
   using C = RowCfg<N, TWX>;
   constexpr int P = (int)half_pitch(N), LEN = HQ * P / 2;  // 16-byte pieces per row group
   const float2* src = in + hrow_q(q0, P);
-  for_groups<TWX / HQ, LEN>([&](int gr, int p0, int p1) {
+  for_groups<T, TWX / HQ, LEN>([&](int gr, int p0, int p1) {
     int k = piece_col(p0);
     float2* d = st + (HQ * gr + piece_row(p0)) * C::CW + k;
     const float2* g = src + (int64_t)gr * HQ * P + 2 * p0;
@@ -1322,7 +1340,7 @@ __device__ __forceinline__ void stage_complex_rows(float2* st, const float2* __r
 // A pair tile: TWX/2 rows of a and the same rows of b (first group-major row q0), row
 // group i of a at tile rows 2 HQ i + 2 j (plane j), of b at 2 HQ i + 2 j + 1, so that
 // tile rows 2w and 2w + 1 are the same real row of a and of b.
-template <int N, int TWX>
+template <int N, int TWX, int T>
 __device__ __forceinline__ void stage_complex_rows_pair(float2* st, const float2* __restrict__ a,
                                                         const float2* __restrict__ b, int64_t q0) {
   using C = RowCfg<N, TWX>;
@@ -1330,7 +1348,7 @@ __device__ __forceinline__ void stage_complex_rows_pair(float2* st, const float2
   constexpr int P = (int)half_pitch(N), LEN = HQ * P / 2;
   const float2* srca = a + hrow_q(q0, P);
   const float2* srcb = b + hrow_q(q0, P);
-  for_groups<TWX / HQ, LEN>([&](int gr, int p0, int p1) {
+  for_groups<T, TWX / HQ, LEN>([&](int gr, int p0, int p1) {
     const int job = gr & 1, i = gr >> 1;
     int k = piece_col(p0);
     float2* d = st + (2 * HQ * i + 2 * piece_row(p0) + job) * C::CW + k;
@@ -1342,21 +1360,21 @@ __device__ __forceinline__ void stage_complex_rows_pair(float2* st, const float2
 
 // real rows of N floats: row r at floats [pitch r, pitch r + N), i.e. the M
 // complex values z[j] = x[2j] + i x[2j+1] at st[r * CW + j] when pitch = 2 CW
-template <int N, int TWX>
+template <int N, int TWX, int T>
 __device__ __forceinline__ void stage_real_rows(float* st, const float* __restrict__ in, int64_t q0,
                                                 int pitch_floats) {
   constexpr int CH = N / 4;             // 16-byte pieces per row
   constexpr int BLK = TWX / HQ * CH;    // pieces per plane
   const float* src = in + real_row_q(q0, N) * N;
-  if constexpr (BLK % NT == 0) {
+  if constexpr (BLK % T == 0) {
 #pragma unroll
-    for (int i = 0; i < HQ * BLK / NT; ++i) {
-      const int h = i * NT / BLK;  // plane, constant per iteration
-      const int e = threadIdx.x + i * NT - h * BLK;
+    for (int i = 0; i < HQ * BLK / T; ++i) {
+      const int h = i * T / BLK;  // plane, constant per iteration
+      const int e = threadIdx.x + i * T - h * BLK;
       cp_async16(st + (HQ * (e / CH) + h) * pitch_floats + 4 * (e % CH), src + (int64_t)h * N * N + 4 * e, true);
     }
   } else {
-    for (int i = threadIdx.x; i < HQ * BLK; i += NT) {
+    for (int i = threadIdx.x; i < HQ * BLK; i += T) {
       const int h = i / BLK, e = i - h * BLK;
       cp_async16(st + (HQ * (e / CH) + h) * pitch_floats + 4 * (e % CH), src + (int64_t)h * N * N + 4 * e, true);
     }
@@ -1406,14 +1424,6 @@ struct C2rCombine {
   }
 };
 
-// Resident CTAs per SM for the plain row passes: 3 when three tiles fit in
-// shared memory and the transform is short enough (<= 256 points) to stay in
-// 85 registers, else 2.
-template <int N, int TWX>
-constexpr int row_blocks() {
-  return (N <= 512 && RowCfg<N, TWX>::smem <= 74 * 1024) ? 3 : 2;
-}
-
 struct ScaleOffset {
   float scale, offset;
   __device__ __forceinline__ float2 operator()(float2 v, int, int) const {
@@ -1445,8 +1455,8 @@ __device__ __forceinline__ void bulk_real_rows(float* st, const float* __restric
     bulk_load(st + r * pitch_floats, src + ((int64_t)(r % HQ) * N + r / HQ) * N, N * sizeof(float), bar);
 }
 
-template <int N, int TWX, bool BULK>
-__global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xr2c(const float* __restrict__ in, float2* __restrict__ out,
+template <int N, int TWX, int T, int CTAS, bool BULK>
+__global__ void __launch_bounds__(T, CTAS) k_xr2c(const float* __restrict__ in, float2* __restrict__ out,
                                                 float scale, float offset,
                                                 const float2* __restrict__ twg, int64_t ntiles,
                                                 Multi m) {
@@ -1467,7 +1477,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xr2c(const float* 
       fence_bar_init();
       fail = 0;
     }
-    load_row_tw<N>(tw, twg);
+    load_row_tw<N, T>(tw, twg);
     __syncthreads();
     uint32_t par = 0, pend = 0;
     int64_t t = blockIdx.x;
@@ -1495,7 +1505,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xr2c(const float* 
       __syncthreads();
       if (fail) break;
       const HalfRowOut<P> o{out + hrow_q(row_tile<N, TWX>(t, m).row0, P)};
-      fft_rowtile_r2c<M, TWX, C::CW, NT, ScaleOffset, false, HalfRowOut<P>>(cur ? st1 : st0, tw + M, tw,
+      fft_rowtile_r2c<M, TWX, C::CW, T, ScaleOffset, false, HalfRowOut<P>>(cur ? st1 : st0, tw + M, tw,
                                                                            ScaleOffset{scale, offset}, o);
       cur ^= 1;
     }
@@ -1506,11 +1516,11 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xr2c(const float* 
     }
     return;
   }
-  load_row_tw<N>(tw, twg);
+  load_row_tw<N, T>(tw, twg);
   int64_t t = blockIdx.x;
   if (t < ntiles) {
     const RowTile r = row_tile<N, TWX>(t, m);
-    stage_real_rows<N, TWX>(reinterpret_cast<float*>(st0), moved(in, r.by), r.row0, 2 * C::CW);
+    stage_real_rows<N, TWX, T>(reinterpret_cast<float*>(st0), moved(in, r.by), r.row0, 2 * C::CW);
   }
   cp_async_commit();
   int cur = 0;
@@ -1518,14 +1528,14 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xr2c(const float* 
     const int64_t tn = t + gridDim.x;
     if (tn < ntiles) {
       const RowTile r = row_tile<N, TWX>(tn, m);
-      stage_real_rows<N, TWX>(reinterpret_cast<float*>(cur ? st0 : st1), moved(in, r.by), r.row0, 2 * C::CW);
+      stage_real_rows<N, TWX, T>(reinterpret_cast<float*>(cur ? st0 : st1), moved(in, r.by), r.row0, 2 * C::CW);
     }
     cp_async_commit();
     cp_async_wait<1>();
     __syncthreads();
     const RowTile r = row_tile<N, TWX>(t, m);
     const HalfRowOut<P> o{moved(out, r.by) + hrow_q(r.row0, P)};
-    fft_rowtile_r2c<M, TWX, C::CW, NT, ScaleOffset, false, HalfRowOut<P>>(cur ? st1 : st0, tw + M, tw,
+    fft_rowtile_r2c<M, TWX, C::CW, T, ScaleOffset, false, HalfRowOut<P>>(cur ? st1 : st0, tw + M, tw,
                                                                          ScaleOffset{scale, offset}, o);
     cur ^= 1;
   }
@@ -1622,8 +1632,8 @@ __device__ __forceinline__ void amax_flush(const SimHeader* h, int job, float a)
     atomicMax(reinterpret_cast<unsigned*>(const_cast<float*>(&h->lq_amax[job])), ua);
 }
 
-template <int N, int TWX, int OUT = 0>
-__global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r(const __grid_constant__ RowJobs jobs,
+template <int N, int TWX, int T, int CTAS, int OUT = 0>
+__global__ void __launch_bounds__(T, CTAS) k_xc2r(const __grid_constant__ RowJobs jobs,
                                                 const float2* __restrict__ twg, int64_t tiles_per_job,
                                                 Multi m) {
   using C = RowCfg<N, TWX>;
@@ -1632,12 +1642,12 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r(const __grid_
   float2* tw = sm;
   float2* st0 = sm + N;
   float2* st1 = st0 + C::stage;
-  load_row_tw<N>(tw, twg);
+  load_row_tw<N, T>(tw, twg);
   const int64_t ntiles = tiles_per_job * jobs.njobs * m.nb;
   int64_t t = blockIdx.x;
   if (t < ntiles) {
     const JobTile j = job_tile<N, TWX>(t, jobs, m);
-    stage_complex_rows<N, TWX>(st0, moved(static_cast<const float2*>(jobs.in[j.job]), j.by), j.row0);
+    stage_complex_rows<N, TWX, T>(st0, moved(static_cast<const float2*>(jobs.in[j.job]), j.by), j.row0);
   }
   cp_async_commit();
   int cur = 0;
@@ -1651,7 +1661,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r(const __grid_
     const int64_t tn = t + gridDim.x;
     if (tn < ntiles) {
       const JobTile jn = job_tile<N, TWX>(tn, jobs, m);
-      stage_complex_rows<N, TWX>(cur ? st0 : st1, moved(static_cast<const float2*>(jobs.in[jn.job]), jn.by),
+      stage_complex_rows<N, TWX, T>(cur ? st0 : st1, moved(static_cast<const float2*>(jobs.in[jn.job]), jn.by),
                                  jn.row0);
     }
     cp_async_commit();
@@ -1665,7 +1675,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r(const __grid_
     if constexpr (OUT == 0) {
       float* out = moved(static_cast<float*>(jobs.out[j.job]), j.by);
       const RealRowOut<M> o{reinterpret_cast<float2*>(out + real_row_q(j.row0, N) * N)};
-      fft_rowtile<M, TWX, C::CW, NT, true, Pre, false, RealRowOut<M>>(buf, tw + M, pre, o);
+      fft_rowtile<M, TWX, C::CW, T, true, Pre, false, RealRowOut<M>>(buf, tw + M, pre, o);
     } else {
       const SimHeader* h = moved(jobs.hdr, j.by);
       if (j.q != run_q) {  // the same for every thread of the CTA
@@ -1679,7 +1689,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r(const __grid_
       float tile_max = 0.f;
       const RealRowOut16<M, OUT> o{out + real_row_q(j.row0, N) * M,
                                    1.f / h->lq_scale[j.job], &tile_max};
-      fft_rowtile<M, TWX, C::CW, NT, true, Pre, false, RealRowOut16<M, OUT>>(buf, tw + M, pre, o);
+      fft_rowtile<M, TWX, C::CW, T, true, Pre, false, RealRowOut16<M, OUT>>(buf, tw + M, pre, o);
       run_max = fmaxf(run_max, tile_max);
     }
     __syncthreads();
@@ -1724,8 +1734,8 @@ struct PairRowOut {
 // c2r of the rows of a (x derivative i kfs kx on load) and of b into the (x, y)
 // pairs of one interleaved real field (App. B: F_x and F_y of the force mesh),
 // pair tiles of TWX/2 rows of each.
-template <int N, int TWX>
-__global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r_pair(
+template <int N, int TWX, int T, int CTAS>
+__global__ void __launch_bounds__(T, CTAS) k_xc2r_pair(
     const float2* __restrict__ a, const float2* __restrict__ b, float2* __restrict__ out, float kfs,
     const float2* __restrict__ twg, int64_t tiles_per_sim, Multi m) {
   using C = RowCfg<N, TWX>;
@@ -1735,7 +1745,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r_pair(
   float2* tw = sm;
   float2* st0 = sm + N;
   float2* st1 = st0 + C::stage;
-  load_row_tw<N>(tw, twg);
+  load_row_tw<N, T>(tw, twg);
   const int64_t ntiles = tiles_per_sim * m.nb;
   auto tile = [&](int64_t t, int64_t& q0, int64_t& by) {
     const int64_t s = t / tiles_per_sim;
@@ -1746,7 +1756,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r_pair(
   if (t < ntiles) {
     int64_t q0, by;
     tile(t, q0, by);
-    stage_complex_rows_pair<N, TWX>(st0, moved(a, by), moved(b, by), q0);
+    stage_complex_rows_pair<N, TWX, T>(st0, moved(a, by), moved(b, by), q0);
   }
   cp_async_commit();
   int cur = 0;
@@ -1757,7 +1767,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r_pair(
     if (tn < ntiles) {
       int64_t qn, bn;
       tile(tn, qn, bn);
-      stage_complex_rows_pair<N, TWX>(cur ? st0 : st1, moved(a, bn), moved(b, bn), qn);
+      stage_complex_rows_pair<N, TWX, T>(cur ? st0 : st1, moved(a, bn), moved(b, bn), qn);
     }
     cp_async_commit();
     cp_async_wait<1>();
@@ -1765,7 +1775,7 @@ __global__ void __launch_bounds__(NT, row_blocks<N, TWX>()) k_xc2r_pair(
     float2* buf = cur ? st1 : st0;
     float2* o = moved(out, by);
     const PairRowOut<N, R1> st{o + real_row_q(q0, N) * N};
-    fft_rowtile<M, TWX, C::CW, NT, true, C2rCombine2<N, C::CW>, false, PairRowOut<N, R1>>(
+    fft_rowtile<M, TWX, C::CW, T, true, C2rCombine2<N, C::CW>, false, PairRowOut<N, R1>>(
         buf, tw + M, C2rCombine2<N, C::CW>{buf, tw, kfs, 0.f}, st);
     __syncthreads();
     cur ^= 1;
@@ -1824,8 +1834,8 @@ constexpr size_t xscreen_smem() {
   return RowCfg<N, TWX>::smem;
 }
 
-template <int N, int TWX, int MODEL>
-__global__ void __launch_bounds__(NT, 2) k_x_screen(const float2* __restrict__ w_in,
+template <int N, int TWX, int T, int CTAS, int MODEL>
+__global__ void __launch_bounds__(T, CTAS) k_x_screen(const float2* __restrict__ w_in,
                                                     const float* __restrict__ rho,
                                                     float2* __restrict__ s_out,
                                                     ForceParams fp0, const float2* __restrict__ twg,
@@ -1837,11 +1847,11 @@ __global__ void __launch_bounds__(NT, 2) k_x_screen(const float2* __restrict__ w
   float2* tw = sm;
   float2* st0 = sm + N;
   float2* st1 = st0 + C::stage;
-  load_row_tw<N>(tw, twg);
+  load_row_tw<N, T>(tw, twg);
   int64_t t = blockIdx.x;
   if (t < ntiles) {
     const RowTile r = row_tile<N, TWX>(t, m);
-    stage_complex_rows<N, TWX>(st0, moved(w_in, r.by), r.row0);
+    stage_complex_rows<N, TWX, T>(st0, moved(w_in, r.by), r.row0);
   }
   cp_async_commit();
   int cur = 0;
@@ -1857,18 +1867,17 @@ __global__ void __launch_bounds__(NT, 2) k_x_screen(const float2* __restrict__ w
     // the next tile's w rows into the other buffer land while this tile is transformed
     if (tn < ntiles) {
       const RowTile rn = row_tile<N, TWX>(tn, m);
-      stage_complex_rows<N, TWX>(cur ? st0 : st1, moved(w_in, rn.by), rn.row0);
+      stage_complex_rows<N, TWX, T>(cur ? st0 : st1, moved(w_in, rn.by), rn.row0);
     }
     cp_async_commit();
-    fft_rowtile_call<M, TWX, C::CW, NT, true, C2rCombine<N, C::CW>, true>(buf, tw + M,
-                                                                           C2rCombine<N, C::CW>{buf, tw, 0.f});
-    // S = delta eps(w) is formed as the forward transform loads it
+    // S = delta eps(w) is formed between the inverse and the forward transform
     const float* rho_t = moved(rho, r.by);
     const ScreenSourceRows<M, MODEL> src{reinterpret_cast<const float2*>(rho_t + real_row_q(row0, N) * N),
                                          fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef};
     constexpr int P = (int)half_pitch(N);
-    fft_rowtile_r2c_call<M, TWX, C::CW, NT, ScreenSourceRows<M, MODEL>, true, HalfRowOut<P>>(
-        buf, tw + M, tw, src, HalfRowOut<P>{moved(s_out, r.by) + hrow_q(row0, P)});
+    fft_rowtile_inv_r2c<M, TWX, C::CW, T, C2rCombine<N, C::CW>, ScreenSourceRows<M, MODEL>, true, HalfRowOut<P>>(
+        buf, tw + M, tw, C2rCombine<N, C::CW>{buf, tw, 0.f}, src,
+        HalfRowOut<P>{moved(s_out, r.by) + hrow_q(row0, P)});
     cur ^= 1;
   }
   cp_async_wait<0>();
@@ -2065,10 +2074,10 @@ __global__ void __launch_bounds__(NT) k_plane_screen(const float2* __restrict__ 
   cp_async_wait<0>();
   __syncthreads();
   plane_yinv<N>(a, tw);
-  fft_rowtile<M, N, C::CW, NT, true, C2rCombine<N, C::CW>>(a, tw + N, C2rCombine<N, C::CW>{a, tw, 0.f});
   const ScreenSource<M, MODEL> src{reinterpret_cast<const float2*>(moved(rho, by) + (int64_t)z * N * N),
                                          fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef};
-  fft_rowtile_r2c<M, N, C::CW, NT, ScreenSource<M, MODEL>, false, RowStore>(a, tw + N, tw, src, RowStore{});
+  fft_rowtile_inv_r2c<M, N, C::CW, NT, C2rCombine<N, C::CW>, ScreenSource<M, MODEL>, false, RowStore>(
+      a, tw + N, tw, C2rCombine<N, C::CW>{a, tw, 0.f}, src, RowStore{});
   constexpr int64_t P = half_pitch(N);
   float2* g = moved(s_out, by) + hrow(z, 0, N, P);
 #pragma unroll 1
@@ -2082,11 +2091,6 @@ template <int N, int NBUF>
 constexpr size_t col_smem() {
   static_assert(col_rows(N) == fft_rows<N>(), "column stage rows");
   return col_smem_c(N, NBUF);
-}
-
-template <int N>
-constexpr size_t row_smem() {
-  return RowCfg<N, row_tw(N)>::smem;
 }
 
 // Along y: o = z, n = y.  Along z: o = y, n = z (rows of a plane group 8 elements apart).
@@ -2123,17 +2127,18 @@ void set_grid_cap(int max_ctas) { g_grid_cap = max_ctas > 0 ? max_ctas : 0; }
 template <int N>
 static cudaError_t launch_xr2c(const float* in, float2* out, float scale, float offset,
                                const float2* tw, cudaStream_t s, Multi m) {
-  constexpr int TWX = row_tw(N);
+  constexpr RowShape SH = r2c_shape(N);
+  constexpr int TWX = SH.rows, T = SH.threads;
   const int64_t tps = (int64_t)N * N / TWX;
   const int64_t ntiles = tps * m.nb;
   auto go = [&](auto bulk_c) {
     constexpr bool BULK = decltype(bulk_c)::value;
-    const size_t sm = row_smem<N>() + (BULK ? 2 * sizeof(uint64_t) + 16 : 0);
-    auto k = k_xr2c<N, TWX, BULK>;
+    const size_t sm = RowCfg<N, TWX>::smem + (BULK ? 2 * sizeof(uint64_t) + 16 : 0);
+    auto k = k_xr2c<N, TWX, T, SH.ctas, BULK>;
     unsigned grid;
-    cudaError_t e = prep(k, sm, ntiles, grid);
+    cudaError_t e = prep(k, sm, ntiles, grid, T);
     if (e != cudaSuccess) return e;
-    k<<<grid, NT, sm, s>>>(in, out, scale, offset, tw, ntiles, m);
+    k<<<grid, T, sm, s>>>(in, out, scale, offset, tw, ntiles, m);
     return cudaGetLastError();
   };
   // one 1024-point simulation: 1-D bulk copies stage the real rows (1.93 -> 1.90 ms at 1024^3)
@@ -2152,8 +2157,9 @@ cudaError_t fft_xr2c(int Nv, const float* in, float2* out, float scale, float of
 template <int N>
 static cudaError_t launch_xc2r_multi(int njobs, const float2* const* in, float* const* out,
                                      const float* kfs, const float2* tw, cudaStream_t s, Multi m) {
-  constexpr int TWX = row_tw(N);
-  const size_t sm = row_smem<N>();
+  constexpr RowShape SH = c2r_shape(N);
+  constexpr int TWX = SH.rows, T = SH.threads;
+  const size_t sm = RowCfg<N, TWX>::smem;
   RowJobs jobs{};
   jobs.njobs = njobs;
   fast_div_magic((uint32_t)njobs, jobs.jmul, jobs.jshift);
@@ -2163,11 +2169,11 @@ static cudaError_t launch_xc2r_multi(int njobs, const float2* const* in, float* 
     jobs.kfs[i] = kfs[i];
   }
   const int64_t tpj = (int64_t)N * N / TWX;
-  auto k = k_xc2r<N, TWX>;
+  auto k = k_xc2r<N, TWX, T, SH.ctas>;
   unsigned grid;
-  cudaError_t e = prep(k, sm, tpj * njobs * m.nb, grid);
+  cudaError_t e = prep(k, sm, tpj * njobs * m.nb, grid, T);
   if (e != cudaSuccess) return e;
-  k<<<grid, NT, sm, s>>>(jobs, tw, tpj, m);
+  k<<<grid, T, sm, s>>>(jobs, tw, tpj, m);
   return cudaGetLastError();
 }
 
@@ -2184,14 +2190,15 @@ static cudaError_t launch_xc2r_pair(const float2* a, const float2* b, float* xy,
   if constexpr (N < 256) {
     return cudaErrorInvalidValue;
   } else {
-    constexpr int TWX = row_tw(N);
-    const size_t sm = row_smem<N>();
+    constexpr RowShape SH = pair_shape(N);
+  constexpr int TWX = SH.rows, T = SH.threads;
+    const size_t sm = RowCfg<N, TWX>::smem;
     const int64_t tps = (int64_t)N * N / (TWX / 2);
-    auto k = k_xc2r_pair<N, TWX>;
+    auto k = k_xc2r_pair<N, TWX, T, SH.ctas>;
     unsigned grid;
-    cudaError_t e = prep(k, sm, tps * m.nb, grid);
+    cudaError_t e = prep(k, sm, tps * m.nb, grid, T);
     if (e != cudaSuccess) return e;
-    k<<<grid, NT, sm, s>>>(a, b, reinterpret_cast<float2*>(xy), kfs, tw, tps, m);
+    k<<<grid, T, sm, s>>>(a, b, reinterpret_cast<float2*>(xy), kfs, tw, tps, m);
     return cudaGetLastError();
   }
 }
@@ -2205,8 +2212,9 @@ cudaError_t fft_xc2r_pair(int Nv, const float2* a, const float2* b, float* xy, f
 template <int N, int OUT>
 static cudaError_t launch_xc2r_multi16(int njobs, const float2* const* in, void* const* out, const float* kfs,
                                        const SimHeader* hdr, const float2* tw, cudaStream_t s, Multi m) {
-  constexpr int TWX = row_tw(N);
-  const size_t sm = row_smem<N>();
+  constexpr RowShape SH = c2r_shape(N);
+  constexpr int TWX = SH.rows, T = SH.threads;
+  const size_t sm = RowCfg<N, TWX>::smem;
   RowJobs jobs{};
   jobs.njobs = njobs;
   jobs.hdr = hdr;
@@ -2217,11 +2225,11 @@ static cudaError_t launch_xc2r_multi16(int njobs, const float2* const* in, void*
     jobs.kfs[i] = kfs[i];
   }
   const int64_t tpj = (int64_t)N * N / TWX;
-  auto k = k_xc2r<N, TWX, OUT>;
+  auto k = k_xc2r<N, TWX, T, SH.ctas, OUT>;
   unsigned grid;
-  cudaError_t e = prep(k, sm, tpj * njobs * m.nb, grid);
+  cudaError_t e = prep(k, sm, tpj * njobs * m.nb, grid, T);
   if (e != cudaSuccess) return e;
-  k<<<grid, NT, sm, s>>>(jobs, tw, tpj, m);
+  k<<<grid, T, sm, s>>>(jobs, tw, tpj, m);
   return cudaGetLastError();
 }
 
@@ -2401,21 +2409,22 @@ cudaError_t mesh_z_screen_field(int Nv, const float2* in, float2* dk_out, float2
 template <int N>
 static cudaError_t launch_xscreen(const float2* w_in, const float* rho, float2* s_out,
                                   const ForceParams& fp, const float2* tw, cudaStream_t s, Multi m) {
-  constexpr int TWX = row_tw(N);
+  constexpr RowShape SH = screen_shape(N);
+  constexpr int TWX = SH.rows, T = SH.threads;
   constexpr size_t sm = xscreen_smem<N, TWX>();
   const int64_t tps = (int64_t)N * N / TWX;
   const int64_t ntiles = tps * m.nb;
   unsigned grid;
   if (fp.model == 1) {
-    auto k = k_x_screen<N, TWX, 1>;
-    cudaError_t e = prep(k, sm, ntiles, grid);
+    auto k = k_x_screen<N, TWX, T, SH.ctas, 1>;
+    cudaError_t e = prep(k, sm, ntiles, grid, T);
     if (e != cudaSuccess) return e;
-    k<<<grid, NT, sm, s>>>(w_in, rho, s_out, fp, tw, ntiles, m);
+    k<<<grid, T, sm, s>>>(w_in, rho, s_out, fp, tw, ntiles, m);
   } else {
-    auto k = k_x_screen<N, TWX, 2>;
-    cudaError_t e = prep(k, sm, ntiles, grid);
+    auto k = k_x_screen<N, TWX, T, SH.ctas, 2>;
+    cudaError_t e = prep(k, sm, ntiles, grid, T);
     if (e != cudaSuccess) return e;
-    k<<<grid, NT, sm, s>>>(w_in, rho, s_out, fp, tw, ntiles, m);
+    k<<<grid, T, sm, s>>>(w_in, rho, s_out, fp, tw, ntiles, m);
   }
   return cudaGetLastError();
 }
