@@ -509,6 +509,59 @@ __device__ __forceinline__ void fft_tile_fwd_inv2(float2* __restrict__ buf, cons
   col_inv2<IR1, IR2, TW, PITCH, NT>(buf, st2);
 }
 
+// Inverse transforms of the tile's columns to st and of i kfs f_n times them (f_n the
+// signed frequency, zero on the Nyquist row) to st2.  The first step reads each value
+// once and forms both transforms' intermediates, the derivative's in buf2
+// (fft_rows<L>() rows, free).  The caller synchronises before the call and before it
+// reuses the buffers.
+template <int L, int TW, int PITCH, int NT, class Store>
+__device__ __forceinline__ void fft_tile_inv_deriv(float2* __restrict__ buf, float2* __restrict__ buf2,
+                                                   const float2* __restrict__ tw, float kfs, Store st, Store st2) {
+  constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;
+  constexpr int U = TW * R2, P = (U + NT - 1) / NT;
+  static_assert(PITCH % 8 == 0, "column tiles: row pitch a multiple of 8");
+  float2 v[P][R1];
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    const int u = threadIdx.x + i * NT;
+    if ((U % NT) == 0 || u < U) {
+      const int c = u % TW, n2 = u / TW;
+      float2 d[R1];
+#pragma unroll
+      for (int n1 = 0; n1 < R1; ++n1) {
+        const int n = R2 * n1 + n2;
+        const float2 x = buf[n * PITCH + c];
+        const float f = n == L / 2 ? 0.f : kfs * (float)(n < L / 2 ? n : n - L);
+        v[i][pos_of<R1>(n1)] = x;
+        d[pos_of<R1>(n1)] = cscale(cmul_i(x), f);
+      }
+      dftR<R1, true>(d);
+      dftR<R1, true>(v[i]);
+      float2* y = buf2 + n2 * (R1 + 1) * PITCH + c;
+      y[0] = d[0];
+#pragma unroll
+      for (int k1 = 1; k1 < R1; ++k1) {
+        const float2 w = n2 > 0 ? cconj(tw[n2 * k1]) : make_float2(1.f, 0.f);
+        y[k1 * PITCH] = cmul(d[k1], w);
+        v[i][k1] = cmul(v[i][k1], w);
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    const int u = threadIdx.x + i * NT;
+    if ((U % NT) == 0 || u < U) {
+      float2* y = buf + u / TW * (R1 + 1) * PITCH + u % TW;
+#pragma unroll
+      for (int k1 = 0; k1 < R1; ++k1) y[k1 * PITCH] = v[i][k1];
+    }
+  }
+  __syncthreads();
+  col_inv2<R1, R2, TW, PITCH, NT>(buf, st);
+  col_inv2<R1, R2, TW, PITCH, NT>(buf2, st2);
+}
+
 // Row pitch (complex values) of a row-major tile transformed in place by
 // fft_rowtile<L>: at least L + R2 - 1 (room for the padded intermediate) and
 // 8 mod 16, so that the half-warps of both steps hit distinct bank pairs.

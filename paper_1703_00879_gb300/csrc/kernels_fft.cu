@@ -104,6 +104,16 @@ constexpr int zt(int N) { return N <= 512 ? 128 : NT; }
 // Resident CTAs per SM they are compiled for (shared memory; 3 at 512 points: 295 us).
 constexpr int zblocks(int N) { return N <= 256 ? 4 : N <= 512 ? 2 : 1; }
 
+// Tiles, threads and resident CTAs per SM of the y passes (and the plain z pass): as the
+// fused z passes, small CTAs without idle threads; the y inverse with its derivative reads
+// each input once and starts both transforms from it (fft_tile_inv_deriv).  Per launch,
+// us: y forward 512^3 216 -> 190, 256^3 31.2 -> 27.5; force y inverse (three arrays in two
+// launches and the screening field's) 512^3 238 -> 222 mean, 1024^3 1810 -> 1713.
+__host__ __device__ constexpr int ytw(int N) { return N >= 256 ? 8 : 16; }
+__host__ __device__ constexpr int yt(int N) { return N >= 1024 ? 256 : 128; }
+constexpr int ycol_blocks(int N) { return N >= 1024 ? 1 : N == 512 ? 3 : 5; }
+constexpr int yinv_blocks(int N) { return N >= 1024 ? 1 : N == 512 ? 2 : 4; }
+
 int sm_count() {
   static int n = 0;
   if (n == 0) {
@@ -601,6 +611,7 @@ __global__ void k_wait_probe(uint64_t limit_ns) {
 // out = transform of in along the tile axis; out may alias in.
 template <int N, int TW, bool INV>
 struct OpCol {
+  static constexpr int T = yt(N);
   ColGeo<N, TW> geo;
   const float2* in;
   float2* out;
@@ -610,113 +621,39 @@ struct OpCol {
     int o, c0;
     int64_t base, by;
     geo.tile(t, o, c0, base, by);
-    col_issue<N, TW, TW>(buf, 0, moved(in, by), base, geo.ra, geo.rb, c0);
+    col_issue<N, TW, TW, T>(buf, 0, moved(in, by), base, geo.ra, geo.rb, c0);
   }
   // outputs go to HBM from the last step's registers (ColOut)
   __device__ __forceinline__ void process(float2* buf, const float2* tw, int64_t t) const {
     int o, c0;
     int64_t base, by;
     geo.tile(t, o, c0, base, by);
-    fft_tile<N, TW, TW, NT, INV, 1, TileLoad, ColOut>(
+    fft_tile<N, TW, TW, T, INV, 1, TileLoad, ColOut>(
         buf, tw, TileLoad{}, ColOut{moved(out, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0});
   }
 };
 
 template <int N, int TW, bool INV, bool TMA>
-__global__ void __launch_bounds__(NT, blocks_for_smem(col_smem_c(N, 1), N)) k_col(OpCol<N, TW, INV> op, const float2* __restrict__ twg,
+__global__ void __launch_bounds__(yt(N), ycol_blocks(N)) k_col(OpCol<N, TW, INV> op, const float2* __restrict__ twg,
                                             int64_t ntiles, const __grid_constant__ CUtensorMap map) {
-  if constexpr (TMA) col_pipeline_tma<N, fft_rows<N>() * TW, false, 0, NT>(op, twg, ntiles, &map, nullptr);
-  else col_pipeline<N, fft_rows<N>() * TW>(op, twg, ntiles);
+  constexpr int T = yt(N);
+  if constexpr (TMA) col_pipeline_tma<N, fft_rows<N>() * TW, false, 0, T>(op, twg, ntiles, &map, nullptr);
+  else col_pipeline<N, fft_rows<N>() * TW, T>(op, twg, ntiles);
 }
 
 // ---------------------------------------------------------------- y inverse, two outputs
-template <int N, int TW>
-struct OpYinv2 {
-  // Load hook of the two-array transform: columns c < TW are the staged input,
-  // columns TW + c its y derivative i kfs f_n (zero on the Nyquist row), formed
-  // from column c as the first step loads it.
-  struct PairLoad {
-    float kfs;
-    __device__ __forceinline__ float2 operator()(const float2* buf, int n, int c, int at) const {
-      const bool d = c >= TW;
-      const float2 v = buf[d ? at - TW : at];
-      const float f = (n == N / 2) ? 0.f : kfs * (float)freq_index(n, N);
-      const float a = d ? 0.f : 1.f, b = d ? f : 0.f;  // v (a + i b)
-      return make_float2(a * v.x - b * v.y, a * v.y + b * v.x);
-    }
-  };
-  // Store hook: columns c < TW to the plain output, TW + c to the derivative,
-  // straight from the last step's registers.
-  struct PairOut {
-    static constexpr bool kSmem = false;
-    float2 *gp, *gd;
-    int64_t ra, rb;
-    int live;
-    __device__ __forceinline__ float2 operator()(float2 v, int n, int c, int) const {
-      const bool d = c >= TW;
-      const int cc = d ? c - TW : c;
-      if (cc < live) (d ? gd : gp)[(n / HQ) * ra + (n % HQ) * rb + hcol(cc)] = v;
-      return v;
-    }
-    __device__ __forceinline__ void ready() const {}
-  };
-  ColGeo<N, TW> geo;
-  const float2* in;
-  float2 *outp, *outd;
-  float kfs;
-  float2* extra = nullptr;  // scratch after the stage buffers (set by col_pipeline)
-  static constexpr bool kSide = false;
-  __device__ __forceinline__ void issue(float2* buf, int64_t t) const {
-    int o, c0;
-    int64_t base, by;
-    geo.tile(t, o, c0, base, by);
-    col_issue<N, TW, 2 * TW>(buf, 0, moved(in, by), base, geo.ra, geo.rb, c0);
-  }
-  __device__ __forceinline__ void process(float2* buf, const float2* tw, int64_t t) const {
-    constexpr int TP = 2 * TW;
-    int o, c0;
-    int64_t base, by;
-    geo.tile(t, o, c0, base, by);
-    fft_tile<N, TP, TP, NT, true, 1, PairLoad, PairOut>(
-        buf, tw, PairLoad{kfs},
-        PairOut{moved(outp, by) + base, moved(outd, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0});
-  }
-};
-
-template <int N, int TW>
-__global__ void __launch_bounds__(NT, blocks_for_smem(col_smem_c(N, 2), N)) k_yinv2(OpYinv2<N, TW> op, const float2* __restrict__ twg,
-                                              int64_t ntiles) {
-  col_pipeline<N, fft_rows<N>() * 2 * TW>(op, twg, ntiles);
-}
-
-// y inverse with the y derivative as a second output, for long columns (512
-// and 1024 points) where a two-array tile would need 32-byte rows: three tile
-// buffers of TW columns rotate between the input (transformed in place for the
-// plain output), the derivative and the prefetch of the next input, so the
-// input is read from HBM once with TW-column (64-byte) rows.  Given input
-// buffer I, the derivative goes to (I + 1) mod 3 and the prefetch to (I + 2)
-// mod 3, which holds the next tile's input.
-// Load hook: i kfs f_n times element (n, c) of another tile (zero on the Nyquist row).
-template <int N>
-struct DerivLoad {
-  const float2* src;
-  float kfs;
-  __device__ __forceinline__ float2 operator()(const float2*, int n, int, int at) const {
-    const float f = (n == N / 2) ? 0.f : kfs * (float)freq_index(n, N);
-    return cscale(cmul_i(src[at]), f);
-  }
-};
-
+// y inverse with the y derivative as a second output: three tile buffers rotate
+// between the input (its intermediate written in place for the plain output), the
+// derivative's intermediate and the prefetch of the next input, so the input is read
+// from HBM once, and from shared memory once (fft_tile_inv_deriv).  Given input
+// buffer I, the derivative goes to (I + 1) mod 3 and the prefetch to (I + 2) mod 3,
+// which holds the next tile's input.
 template <int N, int TW>
 constexpr size_t yinv2r_smem() {
   return (N + 3 * (size_t)fft_rows<N>() * TW) * sizeof(float2);
 }
-template <int N, int TW>
-struct Yinv2rCfg {
-  static constexpr bool ONE_CTA = blocks_for_smem(yinv2r_smem<N, TW>(), N) < 2;
-};
 
-// Both transforms of tile t from input buffer bi (the derivative into bd).
+// Both transforms of tile t from input buffer bi (the derivative's intermediate in bd).
 template <int N, int TW>
 __device__ __forceinline__ void yinv2r_tile(const ColGeo<N, TW>& geo, float2* bi, float2* bd,
                                             const float2* tw, float2* __restrict__ outp,
@@ -724,30 +661,15 @@ __device__ __forceinline__ void yinv2r_tile(const ColGeo<N, TW>& geo, float2* bi
   int o, c0;
   int64_t base, by;
   geo.tile(t, o, c0, base, by);
-  const ColOut out{nullptr, geo.ra, geo.rb, N / 2 + 1 - c0};
-  ColOut od = out, op = out;
-  od.g = moved(outd, by) + base;
-  op.g = moved(outp, by) + base;
-  if constexpr (Yinv2rCfg<N, TW>::ONE_CTA) {
-    // one CTA per SM: the derivative transform runs first, its first step
-    // reading the input (times i kfs f_n) from bi, which the plain transform
-    // then overwrites; both store straight to HBM
-    fft_tile_call<N, TW, TW, NT, true, 1, DerivLoad<N>, ColOut>(bd, tw, DerivLoad<N>{bi, kfs}, od);
-    fft_tile_call<N, TW, TW, NT, true, 1, TileLoad, ColOut>(bi, tw, TileLoad{}, op);
-  } else {
-    // two CTAs per SM (128 registers, where the load hook spills): a pass over the tile
-    const DerivLoad<N> dl{bi, kfs};
-    for (int e = threadIdx.x; e < N * TW; e += NT) bd[e] = dl(bd, e / TW, 0, e);
-    __syncthreads();
-    fft_tile_call<N, TW, TW, NT, true, 1, TileLoad, ColOut>(bd, tw, TileLoad{}, od);
-    fft_tile_call<N, TW, TW, NT, true, 1, TileLoad, ColOut>(bi, tw, TileLoad{}, op);
-  }
+  const ColOut op{moved(outp, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0};
+  const ColOut od{moved(outd, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0};
+  fft_tile_inv_deriv<N, TW, TW, yt(N)>(bi, bd, tw, kfs, op, od);
 }
 
 // TMA: buffer i's copies complete on barrier i (after the three buffers; the
 // failure flag follows), as in col_pipeline_tma.
 template <int N, int TW, bool TMA>
-__global__ void __launch_bounds__(NT, blocks_for_smem(yinv2r_smem<N, TW>(), N)) k_yinv2r(
+__global__ void __launch_bounds__(yt(N), yinv_blocks(N)) k_yinv2r(
     ColGeo<N, TW> geo, const float2* __restrict__ in, float2* __restrict__ outp,
     float2* __restrict__ outd, float kfs, const float2* __restrict__ twg, int64_t ntiles,
     const __grid_constant__ CUtensorMap map) {
@@ -768,7 +690,7 @@ __global__ void __launch_bounds__(NT, blocks_for_smem(yinv2r_smem<N, TW>(), N)) 
       fence_bar_init();
       fail = (smem_u32(sm) & 127) ? 1 : 0;
     }
-    load_tw(tw, twg, N);
+    load_tw<yt(N)>(tw, twg, N);
     __syncthreads();
     if (fail) {
       if (lead) atomicAdd(&g_tile_load_failures, 1u);
@@ -809,13 +731,13 @@ __global__ void __launch_bounds__(NT, blocks_for_smem(yinv2r_smem<N, TW>(), N)) 
         if ((pend >> i) & 1u) bar_wait(&bars[i], (par >> i) & 1u);
     }
   } else {
-    load_tw(tw, twg, N);
+    load_tw<yt(N)>(tw, twg, N);
     int64_t t = blockIdx.x;
     if (t < ntiles) {
       int o, c0;
       int64_t base, by;
       geo.tile(t, o, c0, base, by);
-      col_issue<N, TW, TW>(buf(0), 0, moved(in, by), base, geo.ra, geo.rb, c0);
+      col_issue<N, TW, TW, yt(N)>(buf(0), 0, moved(in, by), base, geo.ra, geo.rb, c0);
     }
     cp_async_commit();
     int I = 0;
@@ -826,7 +748,7 @@ __global__ void __launch_bounds__(NT, blocks_for_smem(yinv2r_smem<N, TW>(), N)) 
         int o, c0;
         int64_t base, by;
         geo.tile(tn, o, c0, base, by);
-        col_issue<N, TW, TW>(buf(F), 0, moved(in, by), base, geo.ra, geo.rb, c0);
+        col_issue<N, TW, TW, yt(N)>(buf(F), 0, moved(in, by), base, geo.ra, geo.rb, c0);
       }
       cp_async_commit();
       cp_async_wait<1>();  // tile t's input has landed
@@ -2296,8 +2218,8 @@ constexpr bool tma_shape() {
 template <int N>
 static cudaError_t launch_col(float2* data, int axis, bool inv, const float2* tw,
                               cudaStream_t s, Multi m) {
-  constexpr int TW = col_tw(N, 1);
-  constexpr size_t sm = col_smem<N, 1>();
+  constexpr int TW = ytw(N);
+  constexpr size_t sm = col_smem_tw(N, TW);
   const int64_t ntiles = col_tiles<N, TW>() * m.nb;
   const ColGeo<N, TW> geo = axis == 1 ? geo_y<N, TW>(m) : geo_z<N, TW>(m);
   CUtensorMap map{};
@@ -2307,9 +2229,9 @@ static cudaError_t launch_col(float2* data, int axis, bool inv, const float2* tw
     constexpr size_t smk = TMA ? tma_smem<N, fft_rows<N>() * TW, 0>() : sm;
     auto k = k_col<N, TW, INV, TMA>;
     unsigned grid;
-    cudaError_t e = prep(k, smk, ntiles, grid);
+    cudaError_t e = prep(k, smk, ntiles, grid, yt(N));
     if (e != cudaSuccess) return e;
-    k<<<grid, NT, smk, s>>>(OpCol<N, TW, INV>{geo, data, data}, tw, ntiles, map);
+    k<<<grid, yt(N), smk, s>>>(OpCol<N, TW, INV>{geo, data, data}, tw, ntiles, map);
     return cudaGetLastError();
   };
   using T = std::true_type;
@@ -2329,37 +2251,23 @@ cudaError_t fft_col(int Nv, float2* data, int axis, bool inv, const float2* tw, 
 template <int N>
 static cudaError_t launch_yinv2(const float2* in, float2* outp, float2* outd, float kfs,
                                 const float2* tw, cudaStream_t s, Multi m) {
-  if constexpr (N >= 512) {
-    // one pass with three rotating single-array tile buffers (k_yinv2r)
-    constexpr int TW = col_tw(N, 1);
-    const int64_t ntiles = col_tiles<N, TW>() * m.nb;
-    CUtensorMap map{};
-    const bool tma = tma_shape<N, TW>() && !m.shift && spectrum_map(map, in, N, TW, false);
-    auto go = [&](auto tma_c) {
-      constexpr bool TMA = decltype(tma_c)::value;
-      constexpr size_t sm = yinv2r_smem<N, TW>() + (TMA ? 4 * sizeof(uint64_t) : 0);
-      auto k = k_yinv2r<N, TW, TMA>;
-      unsigned grid;
-      cudaError_t e = prep(k, sm, ntiles, grid);
-      if (e != cudaSuccess) return e;
-      k<<<grid, NT, sm, s>>>(geo_y<N, TW>(m), in, outp, outd, kfs, tw, ntiles, map);
-      return cudaGetLastError();
-    };
-    if constexpr (tma_shape<N, TW>()) {
-      if (tma) return go(std::true_type{});
-    }
-    return go(std::false_type{});
-  } else {
-    constexpr int TW = col_tw(N, 2);
-    constexpr size_t sm = col_smem<N, 2>();
-    const int64_t ntiles = col_tiles<N, TW>() * m.nb;
-    auto k = k_yinv2<N, TW>;
+  constexpr int TW = ytw(N);
+  const int64_t ntiles = col_tiles<N, TW>() * m.nb;
+  CUtensorMap map{};
+  auto go = [&](auto tma_c) {
+    constexpr bool TMA = decltype(tma_c)::value;
+    constexpr size_t sm = yinv2r_smem<N, TW>() + (TMA ? 4 * sizeof(uint64_t) : 0);
+    auto k = k_yinv2r<N, TW, TMA>;
     unsigned grid;
-    cudaError_t e = prep(k, sm, ntiles, grid);
+    cudaError_t e = prep(k, sm, ntiles, grid, yt(N));
     if (e != cudaSuccess) return e;
-    k<<<grid, NT, sm, s>>>(OpYinv2<N, TW>{geo_y<N, TW>(m), in, outp, outd, kfs}, tw, ntiles);
+    k<<<grid, yt(N), sm, s>>>(geo_y<N, TW>(m), in, outp, outd, kfs, tw, ntiles, map);
     return cudaGetLastError();
+  };
+  if constexpr (tma_shape<N, TW>()) {
+    if (!m.shift && spectrum_map(map, in, N, TW, false)) return go(std::true_type{});
   }
+  return go(std::false_type{});
 }
 
 cudaError_t fft_yinv2(int Nv, const float2* in, float2* outp, float2* outd, float kfs,
