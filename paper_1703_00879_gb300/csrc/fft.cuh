@@ -590,9 +590,11 @@ struct NoPre {
 // 24 per point and warp, LSU pipe 81 % busy).  At 512^3 / 1024^3 (ms): x r2c
 // 1.86 -> 1.61, screening x 3.83 -> 3.45, force x c2r 5.20 -> 4.42, LPT x
 // 1.17 -> 1.01.
-// PAIR32: for L = 16 x 32 with half as many step-2 items as threads, step 2
-// runs on thread pairs (dft32_pair), halving its registers per thread.
-// The caller synchronises before the call; returns after a barrier.
+// Each warp owns TW 32 / NT consecutive rows (RowMap), so the steps are ordered by
+// warp barriers alone and the warps of a CTA drift apart: while one computes another
+// loads.  PAIR32: for L = 16 x 32 with one row per warp, step 2 runs on lane pairs
+// (dft32_pair).  The caller makes the warp's rows visible to it before the call and
+// synchronises the warp before it reuses them.
 // Store hook of fft_rowtile's last step: output k of row c as st(X[k], c, k);
 // with kSmem = false the hook writes the output itself and the tile keeps the
 // intermediate.
@@ -608,47 +610,59 @@ __host__ __device__ constexpr int row_twiddle(int i) {
   return (i / Split<L>::R2) * (i % Split<L>::R2);
 }
 
-// Step 1 of the row transforms, with the barriers that separate it from step 2.
+// Item idx = lane + 32 i of a warp's rows with R items per row: tile row c, item q.
+// With fewer than 32 items in all, lanes repeat them (the same values, written twice).
+template <int TW, int NT, int R>
+struct RowMap {
+  static constexpr int RW = TW * 32 / NT, U = RW * R, P = (U + 31) / 32;
+  static_assert(RW * NT == TW * 32 && (U % 32 == 0 || 32 % U == 0), "whole rows per warp");
+  int c0, idx0;
+  __device__ __forceinline__ RowMap() {
+    c0 = (threadIdx.x >> 5) * RW;
+    idx0 = (threadIdx.x & 31) % (U < 32 ? U : 32);
+  }
+  __device__ __forceinline__ int c(int i) const { return c0 + (idx0 + 32 * i) / R; }
+  __device__ __forceinline__ int q(int i) const { return (idx0 + 32 * i) % R; }
+};
+
+// Step 1 of the row transforms, with the warp barriers that separate it from step 2.
 template <int L, int TW, int CW, int NT, bool INV, class Pre>
 __device__ __forceinline__ void row_step1(float2* __restrict__ buf, const float2* __restrict__ w1, Pre pre) {
   constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;
-  constexpr int U1 = TW * R2, P1 = (U1 + NT - 1) / NT;
+  using Map = RowMap<TW, NT, R2>;
   static_assert(CW >= L + R2 - 1, "row pitch too small for the intermediate");
-  const int tid = threadIdx.x;
-  {
-    float2 v[P1][R1];
+  const Map mp;
+  float2 v[Map::P][R1];
 #pragma unroll
-    for (int i = 0; i < P1; ++i) {
-      const int u = tid + i * NT;
-      if ((U1 % NT) == 0 || u < U1) {
-        const int c = u / R2, n2 = u % R2;
-        const float2* x = buf + c * CW + n2;
+  for (int i = 0; i < Map::P; ++i) {
+    const int c = mp.c(i), n2 = mp.q(i);
+    const float2* x = buf + c * CW + n2;
 #pragma unroll
-        for (int n1 = 0; n1 < R1; ++n1) v[i][pos_of<R1>(n1)] = pre(x[R2 * n1], c, R2 * n1 + n2);
-        dftR<R1, INV>(v[i]);
-        if (n2 > 0) {
+    for (int n1 = 0; n1 < R1; ++n1) v[i][pos_of<R1>(n1)] = pre(x[R2 * n1], c, R2 * n1 + n2);
+    dftR<R1, INV>(v[i]);
+    if (n2 > 0) {
 #pragma unroll
-          for (int k1 = 1; k1 < R1; ++k1) {
-            float2 w = w1[k1 * R2 + n2];
-            if (INV) w.y = -w.y;
-            v[i][k1] = cmul(v[i][k1], w);
-          }
-        }
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < P1; ++i) {
-      const int u = tid + i * NT;
-      if ((U1 % NT) == 0 || u < U1) {
-        const int c = u / R2, n2 = u % R2;
-        float2* y = buf + c * CW + n2 * (R1 + 1);
-#pragma unroll
-        for (int k1 = 0; k1 < R1; ++k1) y[k1] = v[i][k1];
+      for (int k1 = 1; k1 < R1; ++k1) {
+        float2 w = w1[k1 * R2 + n2];
+        if (INV) w.y = -w.y;
+        v[i][k1] = cmul(v[i][k1], w);
       }
     }
   }
-  __syncthreads();
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < Map::P; ++i) {
+    float2* y = buf + mp.c(i) * CW + mp.q(i) * (R1 + 1);
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) y[k1] = v[i][k1];
+  }
+  __syncwarp();
+}
+
+// Lane pairs for the radix-32 step of L = 16 x 32 rows: one row per warp.
+template <int L, int TW, int NT, bool PAIR32>
+__host__ __device__ constexpr bool row_pairs() {
+  return PAIR32 && Split<L>::R1 == 16 && Split<L>::R2 == 32 && TW * 32 == NT;
 }
 
 template <int L, int TW, int CW, int NT, bool INV, class Pre = NoPre, bool PAIR32 = false,
@@ -656,55 +670,43 @@ template <int L, int TW, int CW, int NT, bool INV, class Pre = NoPre, bool PAIR3
 __device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const float2* __restrict__ w1,
                                             Pre pre = Pre(), Store st = Store()) {
   constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;
-  constexpr int U2 = TW * R1, P2 = (U2 + NT - 1) / NT;
-  const int tid = threadIdx.x;
   row_step1<L, TW, CW, NT, INV, Pre>(buf, w1, pre);
-  if constexpr (PAIR32 && R1 == 16 && R2 == 32 && 2 * U2 == NT) {
-    // step 2 on thread pairs (dft32_pair): U2 items would leave half the threads
-    // idle; half the registers per thread
-    const int half = (tid >> 4) & 1, u = (tid >> 5) * 16 + (tid & 15);
-    const int c = u / R1, k1 = u % R1;
+  if constexpr (row_pairs<L, TW, NT, PAIR32>()) {
+    const int lane = threadIdx.x & 31, half = lane >> 4, c = threadIdx.x >> 5, k1 = lane & 15;
     float2 y[16];
     const float2* yr = buf + c * CW + k1 + 16 * half * (R1 + 1);
 #pragma unroll
     for (int j = 0; j < 16; ++j) y[j] = yr[j * (R1 + 1)];
     dft32_pair<INV>(y, half);
-    __syncthreads();
-    float2* X = buf + c * CW + k1 + R1 * half;
+    if constexpr (Store::kSmem) __syncwarp();
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
-      const float2 o = st(y[k], c, k1 + R1 * (2 * k + half));
-      if constexpr (Store::kSmem) X[2 * R1 * k] = o;
+      const int n = k1 + R1 * (2 * k + half);
+      const float2 o = st(y[k], c, n);
+      if constexpr (Store::kSmem) buf[c * CW + n] = o;
     }
   } else {
-    float2 y[P2][R2];
+    using Map = RowMap<TW, NT, R1>;
+    const Map mp;
+    float2 y[Map::P][R2];
 #pragma unroll
-    for (int i = 0; i < P2; ++i) {
-      const int u = tid + i * NT;
-      if ((U2 % NT) == 0 || u < U2) {
-        const int c = u / R1, k1 = u % R1;
-        const float2* yr = buf + c * CW + k1;
+    for (int i = 0; i < Map::P; ++i) {
+      const float2* yr = buf + mp.c(i) * CW + mp.q(i);
 #pragma unroll
-        for (int n2 = 0; n2 < R2; ++n2) y[i][pos_of<R2>(n2)] = yr[n2 * (R1 + 1)];
-        dftR<R2, INV>(y[i]);
-      }
+      for (int n2 = 0; n2 < R2; ++n2) y[i][pos_of<R2>(n2)] = yr[n2 * (R1 + 1)];
+      dftR<R2, INV>(y[i]);
     }
-    __syncthreads();
+    if constexpr (Store::kSmem) __syncwarp();
 #pragma unroll
-    for (int i = 0; i < P2; ++i) {
-      const int u = tid + i * NT;
-      if ((U2 % NT) == 0 || u < U2) {
-        const int c = u / R1, k1 = u % R1;
-        float2* X = buf + c * CW + k1;
+    for (int i = 0; i < Map::P; ++i) {
+      const int c = mp.c(i), k1 = mp.q(i);
 #pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) {
-          const float2 o = st(y[i][k2], c, k1 + R1 * k2);
-          if constexpr (Store::kSmem) X[R1 * k2] = o;
-        }
+      for (int k2 = 0; k2 < R2; ++k2) {
+        const float2 o = st(y[i][k2], c, k1 + R1 * k2);
+        if constexpr (Store::kSmem) buf[c * CW + k1 + R1 * k2] = o;
       }
     }
   }
-  __syncthreads();
 }
 
 // Forward row transform of real rows packed as z[n] = x[2n] + i x[2n+1] (L
@@ -722,24 +724,23 @@ __device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const floa
 template <int L, int TW, int CW, int NT, bool PAIR32, class Store>
 __device__ __forceinline__ void row_r2c_step2(float2* __restrict__ buf, const float2* __restrict__ twr, Store st) {
   constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;
-  constexpr int U2 = TW * R1, P2 = (U2 + NT - 1) / NT;
-  static_assert(R1 <= 32 && U2 % 32 == 0, "whole warps take part in the shuffles");
-  const int tid = threadIdx.x, lane = tid & 31;
+  static_assert(R1 <= 32, "a row's partner lanes within the warp");
+  const int lane = threadIdx.x & 31;
   auto emit = [&](float2 zk, float2 zm, int c, int k) {
     const float2 b = cconj(zm), E = cscale(cadd(zk, b), 0.5f), D = csub(zk, b);
     const float2 X = cadd(E, cmul(twr[k], make_float2(0.5f * D.y, -0.5f * D.x)));  // O = (-i/2) D
     const float2 o = st(X, c, k);
     if constexpr (Store::kSmem) buf[c * CW + k] = o;
   };
-  if constexpr (PAIR32 && R1 == 16 && R2 == 32 && 2 * U2 == NT) {
+  if constexpr (row_pairs<L, TW, NT, PAIR32>()) {
     // a row per warp; half h of lane (k1, h) holds Z[k1 + 16 (2k + h)] at y[k]
-    const int half = lane >> 4, c = tid >> 5, k1 = lane & 15;
+    const int half = lane >> 4, c = threadIdx.x >> 5, k1 = lane & 15;
     float2 y[16];
     const float2* yr = buf + c * CW + k1 + 16 * half * (R1 + 1);
 #pragma unroll
     for (int j = 0; j < 16; ++j) y[j] = yr[j * (R1 + 1)];
     dft32_pair<false>(y, half);
-    if constexpr (Store::kSmem) __syncthreads();
+    if constexpr (Store::kSmem) __syncwarp();
     const int partner = k1 ? ((1 - half) << 4) | (16 - k1) : lane;
     const bool own = k1 == 0 && half == 0;
 #pragma unroll
@@ -751,37 +752,31 @@ __device__ __forceinline__ void row_r2c_step2(float2* __restrict__ buf, const fl
     }
     if (own) emit(y[0], y[0], c, L);
   } else {
-    float2 y[P2][R2];
+    using Map = RowMap<TW, NT, R1>;
+    const Map mp;
+    float2 y[Map::P][R2];
 #pragma unroll
-    for (int i = 0; i < P2; ++i) {
-      const int u = tid + i * NT;
-      if ((U2 % NT) == 0 || u < U2) {
-        const int c = u / R1, k1 = u % R1;
-        const float2* yr = buf + c * CW + k1;
+    for (int i = 0; i < Map::P; ++i) {
+      const float2* yr = buf + mp.c(i) * CW + mp.q(i);
 #pragma unroll
-        for (int n2 = 0; n2 < R2; ++n2) y[i][pos_of<R2>(n2)] = yr[n2 * (R1 + 1)];
-        dftR<R2, false>(y[i]);
-      }
+      for (int n2 = 0; n2 < R2; ++n2) y[i][pos_of<R2>(n2)] = yr[n2 * (R1 + 1)];
+      dftR<R2, false>(y[i]);
     }
-    if constexpr (Store::kSmem) __syncthreads();
+    if constexpr (Store::kSmem) __syncwarp();
 #pragma unroll
-    for (int i = 0; i < P2; ++i) {
-      const int u = tid + i * NT;
-      if ((U2 % NT) == 0 || u < U2) {
-        const int c = u / R1, k1 = u % R1;
-        const int partner = (lane & ~(R1 - 1)) | ((R1 - k1) & (R1 - 1));
+    for (int i = 0; i < Map::P; ++i) {
+      const int c = mp.c(i), k1 = mp.q(i);
+      const int partner = (lane & ~(R1 - 1)) | ((R1 - k1) & (R1 - 1));
 #pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) {
-          float2 zm = make_float2(__shfl_sync(0xffffffffu, y[i][R2 - 1 - k2].x, partner),
-                                  __shfl_sync(0xffffffffu, y[i][R2 - 1 - k2].y, partner));
-          if (k1 == 0) zm = y[i][(R2 - k2) % R2];
-          emit(y[i][k2], zm, c, k1 + R1 * k2);
-        }
-        if (k1 == 0) emit(y[i][0], y[i][0], c, L);
+      for (int k2 = 0; k2 < R2; ++k2) {
+        float2 zm = make_float2(__shfl_sync(0xffffffffu, y[i][R2 - 1 - k2].x, partner),
+                                __shfl_sync(0xffffffffu, y[i][R2 - 1 - k2].y, partner));
+        if (k1 == 0) zm = y[i][(R2 - k2) % R2];
+        emit(y[i][k2], zm, c, k1 + R1 * k2);
       }
+      if (k1 == 0) emit(y[i][0], y[i][0], c, L);
     }
   }
-  __syncthreads();
 }
 
 template <int L, int TW, int CW, int NT, class Pre, bool PAIR32, class Store>
@@ -800,12 +795,10 @@ __device__ __forceinline__ void fft_rowtile_r2c(float2* __restrict__ buf, const 
 template <int L, int TW, int CW, int NT, class Pre, class Mid, bool PAIR32, class Store>
 __device__ __forceinline__ void fft_rowtile_inv_r2c(float2* __restrict__ buf, const float2* __restrict__ w1,
                                                     const float2* __restrict__ twr, Pre pre, Mid mid, Store st) {
-  constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;
-  constexpr int U2 = TW * R1, P2 = (U2 + NT - 1) / NT, H = R2 / R1;
-  const int tid = threadIdx.x;
+  constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2, H = R2 / R1;
   row_step1<L, TW, CW, NT, true, Pre>(buf, w1, pre);
-  if constexpr (PAIR32 && R1 == 16 && R2 == 32 && 2 * U2 == NT) {
-    const int half = (tid >> 4) & 1, c = tid >> 5, k1 = tid & 15, n2 = tid & 31;
+  if constexpr (row_pairs<L, TW, NT, PAIR32>()) {
+    const int n2 = threadIdx.x & 31, half = n2 >> 4, c = threadIdx.x >> 5, k1 = n2 & 15;
     float2 y[16], v[16];
     const float2* yr = buf + c * CW + k1 + 16 * half * (R1 + 1);
 #pragma unroll
@@ -818,53 +811,49 @@ __device__ __forceinline__ void fft_rowtile_inv_r2c(float2* __restrict__ buf, co
 #pragma unroll
       for (int k = 1; k < 16; ++k) v[k] = cmul(v[k], w1[k * R2 + n2]);
     }
-    __syncthreads();
+    __syncwarp();
     float2* o = buf + c * CW + n2 * (R1 + 1);
 #pragma unroll
     for (int k = 0; k < 16; ++k) o[k] = v[k];
   } else {
-    float2 v[P2][R2];
+    using Map = RowMap<TW, NT, R1>;
+    const Map mp;
+    float2 v[Map::P][R2];
 #pragma unroll
-    for (int i = 0; i < P2; ++i) {
-      const int u = tid + i * NT;
-      if ((U2 % NT) == 0 || u < U2) {
-        const int c = u / R1, k1 = u % R1;
-        const float2* yr = buf + c * CW + k1;
-        float2 y[R2];
+    for (int i = 0; i < Map::P; ++i) {
+      const int c = mp.c(i), k1 = mp.q(i);
+      const float2* yr = buf + c * CW + k1;
+      float2 y[R2];
 #pragma unroll
-        for (int n2 = 0; n2 < R2; ++n2) y[pos_of<R2>(n2)] = yr[n2 * (R1 + 1)];
-        dftR<R2, true>(y);
+      for (int n2 = 0; n2 < R2; ++n2) y[pos_of<R2>(n2)] = yr[n2 * (R1 + 1)];
+      dftR<R2, true>(y);
 #pragma unroll
-        for (int k2 = 0; k2 < R2; ++k2) y[k2] = mid(y[k2], c, k1 + R1 * k2);
+      for (int k2 = 0; k2 < R2; ++k2) y[k2] = mid(y[k2], c, k1 + R1 * k2);
 #pragma unroll
-        for (int h = 0; h < H; ++h) {
-          const int n2 = k1 + R1 * h;
-          float2 t[R1];
+      for (int h = 0; h < H; ++h) {
+        const int n2 = k1 + R1 * h;
+        float2 t[R1];
 #pragma unroll
-          for (int n1 = 0; n1 < R1; ++n1) t[pos_of<R1>(n1)] = y[h + H * n1];
-          dftR<R1, false>(t);
-          v[i][h * R1] = t[0];
+        for (int n1 = 0; n1 < R1; ++n1) t[pos_of<R1>(n1)] = y[h + H * n1];
+        dftR<R1, false>(t);
+        v[i][h * R1] = t[0];
 #pragma unroll
-          for (int k = 1; k < R1; ++k) v[i][h * R1 + k] = n2 > 0 ? cmul(t[k], w1[k * R2 + n2]) : t[k];
-        }
+        for (int k = 1; k < R1; ++k) v[i][h * R1 + k] = n2 > 0 ? cmul(t[k], w1[k * R2 + n2]) : t[k];
       }
     }
-    __syncthreads();
+    __syncwarp();
 #pragma unroll
-    for (int i = 0; i < P2; ++i) {
-      const int u = tid + i * NT;
-      if ((U2 % NT) == 0 || u < U2) {
-        const int c = u / R1, k1 = u % R1;
+    for (int i = 0; i < Map::P; ++i) {
+      const int c = mp.c(i), k1 = mp.q(i);
 #pragma unroll
-        for (int h = 0; h < H; ++h) {
-          float2* o = buf + c * CW + (k1 + R1 * h) * (R1 + 1);
+      for (int h = 0; h < H; ++h) {
+        float2* o = buf + c * CW + (k1 + R1 * h) * (R1 + 1);
 #pragma unroll
-          for (int k = 0; k < R1; ++k) o[k] = v[i][h * R1 + k];
-        }
+        for (int k = 0; k < R1; ++k) o[k] = v[i][h * R1 + k];
       }
     }
   }
-  __syncthreads();
+  __syncwarp();
   row_r2c_step2<L, TW, CW, NT, PAIR32, Store>(buf, twr, st);
 }
 

@@ -64,11 +64,15 @@ constexpr RowShape row_big(int N) {
 constexpr RowShape row_small(int N) {
   return N >= 1024 ? RowShape{8, 128, 2} : N == 512 ? RowShape{8, 128, 5} : N == 256 ? RowShape{16, 128, 5} : N == 128 ? RowShape{16, 128, 6} : RowShape{32, 128, 6};
 }
-// Measured on GB300 (us per launch, big / small): x r2c 1024: 1301 / 1331, 512: 179 / 188,
-// 256: 28.0 / 27.3; force c2r (pair and F_z) 1024: 4332 / 4032, 512: 538 / 540, 256: 82 / 78;
-// LPT c2r (six fields) 512: 1006 / 1091, 256: 139 / 146; screening 1024: 3237 / 3386 (big with
-// its radix-32 step on thread pairs), 512: 351 / 329, 256: 54 / 50.
-constexpr RowShape r2c_shape(int N) { return N == 256 ? row_small(N) : row_big(N); }
+// Measured on GB300 (us per launch, big / small, with CTA barriers between the steps): x r2c
+// 512: 179 / 188, 256: 28.0 / 27.3; force c2r (pair and F_z) 1024: 4332 / 4032, 512: 538 / 540,
+// 256: 82 / 78; LPT c2r (six fields) 512: 1006 / 1091, 256: 139 / 146; screening 1024: 3237 /
+// 3386 (big with its radix-32 step on lane pairs), 512: 351 / 329, 256: 54 / 50.  With whole rows
+// per warp and warp barriers only (fft_rowtile) and the tile staged by the CTA in memory order:
+// force c2r 1024: 3876, 512: 522; LPT c2r 256: 130; r2c 512: 179, 1024: 1318 (small).  The
+// screening pass, the one far from the DRAM rate, also stages per warp and has no CTA barrier:
+// 1024: 2409, 512: 298, 256: 45; the others lose 3-10 % to the shorter pieces that way.
+constexpr RowShape r2c_shape(int N) { return N == 256 || N >= 1024 ? row_small(N) : row_big(N); }
 constexpr RowShape c2r_shape(int N) { return N >= 1024 ? row_small(N) : row_big(N); }
 constexpr RowShape pair_shape(int N) { return N >= 1024 || N == 256 ? row_small(N) : row_big(N); }
 constexpr RowShape screen_shape(int N) { return N >= 1024 ? row_big(N) : row_small(N); }
@@ -1303,6 +1307,38 @@ __device__ __forceinline__ void stage_real_rows(float* st, const float* __restri
   }
 }
 
+// A warp stages its own RW = TWX 32 / T rows (RowMap), so a row pass needs no barrier
+// of the CTA: 16-byte pieces of R rows of one group, 64 R / HQ-th parts of it,
+// R = min(RW, HQ); lane l takes piece l of each run of 32, which covers 8 / R chunks.
+template <int N, int CW, int R, int RSTEP>
+__device__ __forceinline__ void stage_group_rows(float2* st, const float2* __restrict__ g) {
+  // rows j = 0 .. R - 1 of the group part at g, row j at st + j RSTEP CW
+  static_assert(8 % R == 0, "whole chunks per 32 pieces");
+  const int lane = threadIdx.x & 31, j = (lane >> 2) % R;
+  int k = lane / (4 * R) * 8 + 2 * (lane & 3);
+  const float2* src = g + lane / (4 * R) * (8 * HQ) + j * 8 + 2 * (lane & 3);
+  float2* d = st + j * RSTEP * CW + k;
+#pragma unroll 4
+  for (; k < N / 2 + 2; k += 64 / R, d += 64 / R, src += 8 / R * (8 * HQ)) cp_async16(d, src, true);
+}
+
+template <int N, int TWX, int T>
+__device__ __forceinline__ void stage_complex_rows_warp(float2* st, const float2* __restrict__ in,
+                                                   int64_t q0) {
+  using C = RowCfg<N, TWX>;
+  constexpr int P = (int)half_pitch(N), RW = TWX * 32 / T, R = RW < HQ ? RW : HQ;
+  const int c0 = (threadIdx.x >> 5) * RW;
+#pragma unroll
+  for (int b = 0; b < RW; b += R)
+    stage_group_rows<N, C::CW, R, 1>(st + (c0 + b) * C::CW, in + hrow_q(q0 + c0 + b, P));
+}
+
+// Real row of tile row r relative to the tile's first: plane r mod HQ, y r / HQ.
+template <int N>
+__device__ __forceinline__ int tile_real_row(int r) {
+  return (r % HQ) * N + r / HQ;
+}
+
 // Store hook of the forward row transforms (fft_rowtile_r2c): X[k] of tile row r into
 // the interleaved half spectrum, g = the tile's first row group.  A warp holds 16 (or
 // fewer) consecutive k of adjacent tile rows: whole 64-byte chunks of adjacent planes.
@@ -1427,8 +1463,9 @@ __global__ void __launch_bounds__(T, CTAS) k_xr2c(const float* __restrict__ in, 
       __syncthreads();
       if (fail) break;
       const HalfRowOut<P> o{out + hrow_q(row_tile<N, TWX>(t, m).row0, P)};
-      fft_rowtile_r2c<M, TWX, C::CW, T, ScaleOffset, false, HalfRowOut<P>>(cur ? st1 : st0, tw + M, tw,
+      fft_rowtile_r2c<M, TWX, C::CW, T, ScaleOffset, true, HalfRowOut<P>>(cur ? st1 : st0, tw + M, tw,
                                                                            ScaleOffset{scale, offset}, o);
+      __syncthreads();
       cur ^= 1;
     }
     if (lead && fail) {
@@ -1447,17 +1484,17 @@ __global__ void __launch_bounds__(T, CTAS) k_xr2c(const float* __restrict__ in, 
   cp_async_commit();
   int cur = 0;
   for (; t < ntiles; t += gridDim.x) {
+    cp_async_wait<0>();  // this thread's copies of tile t (the only group in flight)
+    __syncthreads();     // tile t has landed, and every warp is done with the other buffer
     const int64_t tn = t + gridDim.x;
     if (tn < ntiles) {
       const RowTile r = row_tile<N, TWX>(tn, m);
       stage_real_rows<N, TWX, T>(reinterpret_cast<float*>(cur ? st0 : st1), moved(in, r.by), r.row0, 2 * C::CW);
     }
     cp_async_commit();
-    cp_async_wait<1>();
-    __syncthreads();
     const RowTile r = row_tile<N, TWX>(t, m);
     const HalfRowOut<P> o{moved(out, r.by) + hrow_q(r.row0, P)};
-    fft_rowtile_r2c<M, TWX, C::CW, T, ScaleOffset, false, HalfRowOut<P>>(cur ? st1 : st0, tw + M, tw,
+    fft_rowtile_r2c<M, TWX, C::CW, T, ScaleOffset, true, HalfRowOut<P>>(cur ? st1 : st0, tw + M, tw,
                                                                          ScaleOffset{scale, offset}, o);
     cur ^= 1;
   }
@@ -1500,12 +1537,6 @@ __device__ __forceinline__ JobTile job_tile(int64_t t64, const RowJobs& jobs, co
   const uint32_t t = (uint32_t)t64, q = t / TPJ;     // q = simulation * njobs + job
   const uint32_t b = fast_div(q, jobs.jmul, jobs.jshift);
   return JobTile{(int)(q - b * (uint32_t)jobs.njobs), (int64_t)(t - q * TPJ) * TWX, shift_of(m, (int)b), q};
-}
-
-// Real row of tile row r relative to the tile's first: plane r mod HQ, y r / HQ.
-template <int N>
-__device__ __forceinline__ int tile_real_row(int r) {
-  return (r % HQ) * N + r / HQ;
 }
 
 // Store hook of the c2r row transform: tile row r's M complex outputs (2M reals) to its
@@ -1580,6 +1611,8 @@ __global__ void __launch_bounds__(T, CTAS) k_xc2r(const __grid_constant__ RowJob
   int run_job = 0;
   for (; t < ntiles; t += gridDim.x) {
     const JobTile j = job_tile<N, TWX>(t, jobs, m);
+    cp_async_wait<0>();  // this thread's copies of tile t (the only group in flight)
+    __syncthreads();     // tile t has landed, and every warp is done with the other buffer
     const int64_t tn = t + gridDim.x;
     if (tn < ntiles) {
       const JobTile jn = job_tile<N, TWX>(tn, jobs, m);
@@ -1587,8 +1620,6 @@ __global__ void __launch_bounds__(T, CTAS) k_xc2r(const __grid_constant__ RowJob
                                  jn.row0);
     }
     cp_async_commit();
-    cp_async_wait<1>();
-    __syncthreads();
     float2* buf = cur ? st1 : st0;
     // the c2r pre-processing rides on the transform's first loads
     using Pre = C2rCombine<N, C::CW>;
@@ -1614,7 +1645,6 @@ __global__ void __launch_bounds__(T, CTAS) k_xc2r(const __grid_constant__ RowJob
       fft_rowtile<M, TWX, C::CW, T, true, Pre, false, RealRowOut16<M, OUT>>(buf, tw + M, pre, o);
       run_max = fmaxf(run_max, tile_max);
     }
-    __syncthreads();
     cur ^= 1;
   }
   if constexpr (OUT != 0) amax_flush(run_h, run_job, run_max);
@@ -1685,6 +1715,8 @@ __global__ void __launch_bounds__(T, CTAS) k_xc2r_pair(
   for (; t < ntiles; t += gridDim.x) {
     int64_t q0, by;
     tile(t, q0, by);
+    cp_async_wait<0>();  // this thread's copies of tile t (the only group in flight)
+    __syncthreads();     // tile t has landed, and every warp is done with the other buffer
     const int64_t tn = t + gridDim.x;
     if (tn < ntiles) {
       int64_t qn, bn;
@@ -1692,14 +1724,11 @@ __global__ void __launch_bounds__(T, CTAS) k_xc2r_pair(
       stage_complex_rows_pair<N, TWX, T>(cur ? st0 : st1, moved(a, bn), moved(b, bn), qn);
     }
     cp_async_commit();
-    cp_async_wait<1>();
-    __syncthreads();
     float2* buf = cur ? st1 : st0;
     float2* o = moved(out, by);
     const PairRowOut<N, R1> st{o + real_row_q(q0, N) * N};
     fft_rowtile<M, TWX, C::CW, T, true, C2rCombine2<N, C::CW>, false, PairRowOut<N, R1>>(
         buf, tw + M, C2rCombine2<N, C::CW>{buf, tw, kfs, 0.f}, st);
-    __syncthreads();
     cur ^= 1;
   }
   cp_async_wait<0>();
@@ -1770,10 +1799,11 @@ __global__ void __launch_bounds__(T, CTAS) k_x_screen(const float2* __restrict__
   float2* st0 = sm + N;
   float2* st1 = st0 + C::stage;
   load_row_tw<N, T>(tw, twg);
+  __syncthreads();
   int64_t t = blockIdx.x;
   if (t < ntiles) {
     const RowTile r = row_tile<N, TWX>(t, m);
-    stage_complex_rows<N, TWX, T>(st0, moved(w_in, r.by), r.row0);
+    stage_complex_rows_warp<N, TWX, T>(st0, moved(w_in, r.by), r.row0);
   }
   cp_async_commit();
   int cur = 0;
@@ -1785,11 +1815,11 @@ __global__ void __launch_bounds__(T, CTAS) k_x_screen(const float2* __restrict__
     const int64_t tn = t + gridDim.x;
     float2* buf = cur ? st1 : st0;
     cp_async_wait<0>();  // w rows of this tile (the only group in flight)
-    __syncthreads();
+    __syncwarp();
     // the next tile's w rows into the other buffer land while this tile is transformed
     if (tn < ntiles) {
       const RowTile rn = row_tile<N, TWX>(tn, m);
-      stage_complex_rows<N, TWX, T>(cur ? st0 : st1, moved(w_in, rn.by), rn.row0);
+      stage_complex_rows_warp<N, TWX, T>(cur ? st0 : st1, moved(w_in, rn.by), rn.row0);
     }
     cp_async_commit();
     // S = delta eps(w) is formed between the inverse and the forward transform
@@ -1864,6 +1894,7 @@ __global__ void __launch_bounds__(NT) k_plane_r2c(const float* __restrict__ in, 
   __syncthreads();
   fft_rowtile_r2c<C::M, N, C::CW, NT, ScaleOffset, false, RowStore>(buf, tw + N, tw, ScaleOffset{scale, offset},
                                                                    RowStore{});
+  __syncthreads();
   constexpr int64_t P = half_pitch(N);
   float2* g = moved(out, by) + hrow(z, 0, N, P);
 #pragma unroll 1
@@ -2000,6 +2031,7 @@ __global__ void __launch_bounds__(NT) k_plane_screen(const float2* __restrict__ 
                                          fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef};
   fft_rowtile_inv_r2c<M, N, C::CW, NT, C2rCombine<N, C::CW>, ScreenSource<M, MODEL>, false, RowStore>(
       a, tw + N, tw, C2rCombine<N, C::CW>{a, tw, 0.f}, src, RowStore{});
+  __syncthreads();
   constexpr int64_t P = half_pitch(N);
   float2* g = moved(s_out, by) + hrow(z, 0, N, P);
 #pragma unroll 1
