@@ -34,6 +34,10 @@ __device__ __forceinline__ float2 csub(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
+// a conj(w) with the roundings spelled out
+__device__ __forceinline__ float2 cmul_conj(float2 a, float2 w) {
+  return make_float2(fmaf(a.x, w.x, a.y * w.y), fmaf(a.y, w.x, -(a.x * w.y)));
+}
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return __fmul2_rn(a, make_float2(s, s)); }
 // multiply by +i
@@ -533,18 +537,22 @@ __device__ __forceinline__ void fft_tile_inv_deriv(float2* __restrict__ buf, flo
         const float2 x = buf[n * PITCH + c];
         const float f = n == L / 2 ? 0.f : kfs * (float)(n < L / 2 ? n : n - L);
         v[i][pos_of<R1>(n1)] = x;
-        d[pos_of<R1>(n1)] = cscale(cmul_i(x), f);
+        // rounded products: left to the compiler they may fuse with the first butterflies
+        d[pos_of<R1>(n1)] = make_float2(__fmul_rn(-f, x.y), __fmul_rn(f, x.x));
       }
       dftR<R1, true>(d);
       dftR<R1, true>(v[i]);
-      float2* y = buf2 + n2 * (R1 + 1) * PITCH + c;
-      y[0] = d[0];
+      if (n2 > 0) {
 #pragma unroll
-      for (int k1 = 1; k1 < R1; ++k1) {
-        const float2 w = n2 > 0 ? cconj(tw[n2 * k1]) : make_float2(1.f, 0.f);
-        y[k1 * PITCH] = cmul(d[k1], w);
-        v[i][k1] = cmul(v[i][k1], w);
+        for (int k1 = 1; k1 < R1; ++k1) {
+          const float2 w = tw[n2 * k1];
+          d[k1] = cmul_conj(d[k1], w);
+          v[i][k1] = cmul_conj(v[i][k1], w);
+        }
       }
+      float2* y = buf2 + n2 * (R1 + 1) * PITCH + c;
+#pragma unroll
+      for (int k1 = 0; k1 < R1; ++k1) y[k1 * PITCH] = d[k1];
     }
   }
   __syncthreads();
