@@ -922,8 +922,8 @@ int force_group(const Group& g, double a, bool device_params, bool ini = false) 
       if (sub->lead)
         CK(mesh_z_screen_field(N, sub->lead->Cd, sub->lead->Ck, sub->lead->Cw, fp_of(sub->lead), tw, st,
                                sub->m));
-    prof_end(ctx, ST_Z_SCREEN_FIELD, e, (g.fr_screened.lead ? 1 : 0) + (g.dgp_screened.lead ? 1 : 0),
-             sc.m.nb * 3 * H);
+    const int nfr = g.fr_screened.lead ? g.fr_screened.m.nb : 0, ndgp = g.dgp_screened.lead ? g.dgp_screened.m.nb : 0;
+    prof_end(ctx, ST_Z_SCREEN_FIELD, e, (nfr ? 1 : 0) + (ndgp ? 1 : 0), (nfr * 3.0 + ndgp * 2.0) * H);
     if (plane) {
       // y inverse, x c2r, S = delta eps, x r2c and y forward in one pass per plane
       e = prof_begin(ctx, ST_X_SCREEN_SOURCE);
@@ -949,9 +949,12 @@ int force_group(const Group& g, double a, bool device_params, bool ini = false) 
       prof_end(ctx, ST_MESH_Y, e, 1, sc.m.nb * 2 * H);
     }
     e = prof_begin(ctx, ST_Z_FORCE);
-    CK(mesh_z_force(N, sc.lead->Cd, sc.lead->Ck, sc.lead->Cphi, sc.lead->Cphz, fp_of(sc.lead), tw, st,
-                    sc.m));
-    prof_end(ctx, ST_Z_FORCE, e, 1, sc.m.nb * 4 * H);
+    // delta(k) (Ck) only where the coupling depends on k: the nDGP source holds both parts
+    for (const Group::Sub* sub : {&g.fr_screened, &g.dgp_screened})
+      if (sub->lead)
+        CK(mesh_z_force(N, sub->lead->Cd, sub->lead->Ck, sub->lead->Cphi, sub->lead->Cphz, fp_of(sub->lead), tw,
+                        st, sub->m));
+    prof_end(ctx, ST_Z_FORCE, e, (nfr ? 1 : 0) + (ndgp ? 1 : 0), (nfr * 4.0 + ndgp * 3.0) * H);
   }
   if (const Group::Sub& un = g.unscreened; un.lead) {
     e = prof_begin(ctx, ST_Z_FORCE);

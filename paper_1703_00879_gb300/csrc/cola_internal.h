@@ -181,17 +181,19 @@ cudaError_t fft_col(int N, float2* data, int axis, bool inv, const float2* tw, c
 // transform of (i kfs f_y) times the input (out_deriv).
 cudaError_t fft_yinv2(int N, const float2* in, float2* out_plain, float2* out_deriv, float kfs,
                       const float2* tw, cudaStream_t s, Multi m = {});
-// Screening field: forward z of delta (after x, y) -> delta(k) stored in dk_out;
+// Screening field: forward z of delta (after x, y) -> delta(k) stored in dk_out (f(R));
 // Phi_N(k) (f(R)) or W(kR) delta(k) (nDGP) -> inverse z -> w_out.
 cudaError_t mesh_z_screen_field(int N, const float2* in, float2* dk_out, float2* w_out,
                                 const ForceParams& fp, const float2* tw, cudaStream_t s,
                                 Multi m = {});
-// S = delta eps: c2r of the screening field rows, eps, times delta from rho, r2c.
+// c2r of the screening field rows, eps, the source S = delta eps (f(R)) or
+// delta (1 + C eps) (nDGP) with delta from rho, r2c.
 cudaError_t mesh_x_screen_source(int N, const float2* w_in, const float* rho, float2* s_out,
                                  const ForceParams& fp, const float2* tw, cudaStream_t s,
                                  Multi m = {});
 // Forward z of the source (S or delta), Phi_tot(k) and -i kz Phi_tot, inverse z.
-// dk (delta(k) after the forward z pass) is read when screened, may be null otherwise.
+// dk (delta(k) after the forward z pass) is read for screened f(R), may be null otherwise
+// (a screened nDGP source already holds delta and its fifth force).
 cudaError_t mesh_z_force(int N, const float2* in, const float2* dk, float2* phi_out,
                          float2* phiz_out, const ForceParams& fp, const float2* tw, cudaStream_t s,
                          Multi m = {});
@@ -300,8 +302,8 @@ cudaError_t fft_plane_lpt(int N, const float2* const* lc, float* const* out, flo
                           cudaStream_t s, Multi m = {}, float* zero_dst = nullptr, int64_t zero_floats = 0,
                           bool* zeroed = nullptr);
 // N <= 128: the screening source in one pass per z-plane: from the screening field w
-// (z already inverse-transformed), y and x inverse, S = delta eps(w) with delta from
-// rho, x (r2c) and y forward into s_out (z not transformed).
+// (z already inverse-transformed), y and x inverse, the source as mesh_x_screen_source with
+// delta from rho, x (r2c) and y forward into s_out (z not transformed).
 cudaError_t fft_plane_screen(int N, const float2* w_in, const float* rho, float2* s_out, const ForceParams& fp,
                              const float2* tw, cudaStream_t s, Multi m = {});
 // Runs the transform kernels' bounded mbarrier wait on a phase that never completes

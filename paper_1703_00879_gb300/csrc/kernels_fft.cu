@@ -788,8 +788,9 @@ __device__ __forceinline__ float smoothing_window(float h, int filter) {
 // per-element switch over the windows slows the pass by a third.
 template <int N, int TW, int MODEL, int T>
 struct OpZScreenField {
-  // Between the forward and the inverse transform: delta(k) out to HBM, the field's
-  // multiplier (-kappa/k^2, or the smoothing window) applied.
+  // Between the forward and the inverse transform: delta(k) out to HBM (chameleon-type
+  // models: the force pass needs it; the Vainshtein source carries its delta), the
+  // field's multiplier (-kappa/k^2, or the smoothing window) applied.
   struct Field {
     float2* dk;  // delta(k) of the tile: element (n, c) at dk[(n / HQ) ra + (n mod HQ) rb + hcol(c)]
     int64_t ra, rb;
@@ -797,7 +798,7 @@ struct OpZScreenField {
     float kf2, kappa_norm, R2half, norm;
     int filter;
     __device__ __forceinline__ float2 operator()(float2 v, int n, int c, int) const {
-      if (c0 + c < N / 2 + 1) dk[(n / HQ) * ra + (n % HQ) * rb + hcol(c)] = v;
+      if (MODEL == 1 && c0 + c < N / 2 + 1) dk[(n / HQ) * ra + (n % HQ) * rb + hcol(c)] = v;
       const int fx = c0 + c, fz = freq_index(n, N);
       const float k2 = kf2 * (float)(fx * fx + fy2 + fz * fz);
       float m = 0.f;
@@ -919,7 +920,9 @@ struct OpZForce {
     ForceParams fp = this->fp;
     resolve(fp, by);
     const int fy = freq_index(iy, N);
-    const Combine cmb{extra, c0, fy * fy, fp.kf * fp.kf, fp.a2m2, fp.kappa_norm, fp.C, side};
+    // a Vainshtein source already holds its fifth force (screen_source)
+    const float C = !SCREENED && fp.screened ? 0.f : fp.C;
+    const Combine cmb{extra, c0, fy * fy, fp.kf * fp.kf, fp.a2m2, fp.kappa_norm, C, side};
     const ColOut op{moved(phi_out, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0};
     const ColOut oz{moved(phiz_out, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0};
     fft_tile_fwd_inv2<N, TW, TW, T>(buf, tw, cmb, GradZ{-fp.kf}, next, op, oz);
@@ -1749,18 +1752,29 @@ __device__ __forceinline__ float screen_eps(float w, float p) {
   }
 }
 
-// Load hook of the forward transform of a screening pass: element j of tile row
-// r is S = delta eps(w), w the screening field (the tile value) and delta =
-// rho / rho_bar - 1 from consecutive density rows in global memory (M float2
-// per row, read-only path); used by the plane pass.
+// The source of a screening pass at density contrast d = rho / rho_bar - 1 and screening
+// field w.  Chameleon-type models: S = d eps(w), which the force pass combines with
+// delta(k) mode by mode (the coupling depends on k).  Vainshtein: the range is infinite,
+// Phi_tot = -kappa (delta + C S) / k^2 with C independent of k, so the source is the
+// whole d + C d eps(w): delta(k) is neither written nor read again (two of the fourteen
+// half-spectrum streams of the screened force).
+template <int MODEL>
+__device__ __forceinline__ float screen_source(float d, float w, float p, float C) {
+  const float e = d * screen_eps<MODEL>(w, p);
+  return MODEL == 1 ? e : fmaf(C, e, d);
+}
+
+// Between the transforms of a screening pass: element j of tile row r is the source at w
+// (the tile value) and the density read from consecutive rows in global memory (M
+// float2 per row, read-only path); used by the plane pass.
 template <int M, int MODEL>
 struct ScreenSource {
   const float2* rho;
-  float inv_rhobar, p;
+  float inv_rhobar, p, C;
   __device__ __forceinline__ float2 operator()(float2 w, int r, int j) const {
     const float2 rv = __ldg(rho + r * M + j);
     const float d0 = rv.x * inv_rhobar - 1.f, d1 = rv.y * inv_rhobar - 1.f;
-    return make_float2(d0 * screen_eps<MODEL>(w.x, p), d1 * screen_eps<MODEL>(w.y, p));
+    return make_float2(screen_source<MODEL>(d0, w.x, p, C), screen_source<MODEL>(d1, w.y, p, C));
   }
 };
 
@@ -1769,15 +1783,15 @@ struct ScreenSource {
 template <int M, int MODEL>
 struct ScreenSourceRows {
   const float2* rho;
-  float inv_rhobar, p;
+  float inv_rhobar, p, C;
   __device__ __forceinline__ float2 operator()(float2 w, int r, int j) const {
     const float2 rv = __ldg(rho + tile_real_row<2 * M>(r) * M + j);
     const float d0 = rv.x * inv_rhobar - 1.f, d1 = rv.y * inv_rhobar - 1.f;
-    return make_float2(d0 * screen_eps<MODEL>(w.x, p), d1 * screen_eps<MODEL>(w.y, p));
+    return make_float2(screen_source<MODEL>(d0, w.x, p, C), screen_source<MODEL>(d1, w.y, p, C));
   }
 };
 
-// Screening source S = delta eps: c2r of the screening field rows, eps from the
+// Screening source (screen_source): c2r of the screening field rows, eps from the
 // field and delta from rho (read from global memory by the forward transform's
 // loads), r2c.  Shared memory: twiddles, two row tiles (double-buffered field rows).
 template <int N, int TWX>
@@ -1825,7 +1839,7 @@ __global__ void __launch_bounds__(T, CTAS) k_x_screen(const float2* __restrict__
     // S = delta eps(w) is formed between the inverse and the forward transform
     const float* rho_t = moved(rho, r.by);
     const ScreenSourceRows<M, MODEL> src{reinterpret_cast<const float2*>(rho_t + real_row_q(row0, N) * N),
-                                         fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef};
+                                         fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef, fp.C};
     constexpr int P = (int)half_pitch(N);
     fft_rowtile_inv_r2c<M, TWX, C::CW, T, C2rCombine<N, C::CW>, ScreenSourceRows<M, MODEL>, true, HalfRowOut<P>>(
         buf, tw + M, tw, C2rCombine<N, C::CW>{buf, tw, 0.f}, src,
@@ -2028,7 +2042,7 @@ __global__ void __launch_bounds__(NT) k_plane_screen(const float2* __restrict__ 
   __syncthreads();
   plane_yinv<N>(a, tw);
   const ScreenSource<M, MODEL> src{reinterpret_cast<const float2*>(moved(rho, by) + (int64_t)z * N * N),
-                                         fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef};
+                                         fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef, fp.C};
   fft_rowtile_inv_r2c<M, N, C::CW, NT, C2rCombine<N, C::CW>, ScreenSource<M, MODEL>, false, RowStore>(
       a, tw + N, tw, C2rCombine<N, C::CW>{a, tw, 0.f}, src, RowStore{});
   __syncthreads();
@@ -2406,9 +2420,10 @@ static cudaError_t launch_zforce_t(const float2* in, const float2* dk, float2* p
 cudaError_t mesh_z_force(int Nv, const float2* in, const float2* dk, float2* phi_out,
                          float2* phiz_out, const ForceParams& fp, const float2* tw, cudaStream_t s,
                          Multi m) {
-  if (fp.screened && dk == nullptr) return cudaErrorInvalidValue;
-  COLA_SWITCH_N(Nv, return fp.screened ? launch_zforce_t<N, true>(in, dk, phi_out, phiz_out, fp, tw, s, m)
-                                       : launch_zforce_t<N, false>(in, dk, phi_out, phiz_out, fp, tw, s, m));
+  const bool two = fp.screened && fp.model == 1;  // S and delta(k)
+  if (two && dk == nullptr) return cudaErrorInvalidValue;
+  COLA_SWITCH_N(Nv, return two ? launch_zforce_t<N, true>(in, dk, phi_out, phiz_out, fp, tw, s, m)
+                               : launch_zforce_t<N, false>(in, dk, phi_out, phiz_out, fp, tw, s, m));
   return cudaSuccess;
 }
 
