@@ -695,11 +695,10 @@ struct TableLayout {
 void context_layout(cola_ctx* c, const cola_config& cfg, Layout& L) {
   const int64_t P = (int64_t)cfg.Np * cfg.Np * cfg.Np, M = (int64_t)cfg.Nmesh * cfg.Nmesh * cfg.Nmesh;
   const int64_t hp = half_elems(cfg.Np), hm = half_elems(cfg.Nmesh);
-  for (int d = 0; d < 3; ++d) {
-    L.add(&c->s[d], P);
-    L.add(&c->v[d], P);
-    L.add(&c->acc[d], P);
-  }
+  // the components of each particle vector follow one another (P floats are whole
+  // 256-byte units), so a [3][P] array is one copy
+  for (float** q : {c->s, c->v, c->acc})
+    for (int d = 0; d < 3; ++d) L.add(&q[d], P);
   for (int f = 0; f < 2; ++f) {
     L.add(&c->phi[f], hp);
     if (cfg.seed_precision) L.add(reinterpret_cast<uint32_t**>(&c->seedq[f]), hp);
@@ -1811,8 +1810,7 @@ int cola_export(cola_ctx* ctx, int32_t which, void* dst, int32_t where) {
     case COLA_F_ACC: {
       if (!ctx->ic_done) return fail(ctx, COLA_ESTATE, "no particle state before cola_ic");
       float* const* arr = which == COLA_F_DISP ? ctx->s : which == COLA_F_DV ? ctx->v : ctx->acc;
-      for (int c = 0; c < 3; ++c) CHECK_RC(copy_out(ctx, d + c * pb, arr[c], pb, where));
-      return COLA_OK;
+      return copy_out(ctx, d, arr[0], 3 * pb, where);
     }
     case COLA_F_RHO:
       if (!ctx->have_force) return fail(ctx, COLA_ESTATE, "no deposit yet");
@@ -1872,9 +1870,7 @@ int cola_import_state(cola_ctx* ctx, const float* disp, const float* dv, const f
   const size_t pb = (size_t)ctx->P * sizeof(float);
   const float* src[3] = {disp, dv, acc};
   float* const* dstv[3] = {ctx->s, ctx->v, ctx->acc};
-  for (int q = 0; q < 3; ++q)
-    for (int c = 0; c < 3; ++c)
-      CHECK_RC(copy_in(ctx, dstv[q][c], reinterpret_cast<const char*>(src[q]) + c * pb, pb, where));
+  for (int q = 0; q < 3; ++q) CHECK_RC(copy_in(ctx, dstv[q][0], src[q], 3 * pb, where));
   ctx->hh.step = steps_done;
   CK(set_header(ctx->hdr, ctx->hh, ctx->st));
   ctx->step = steps_done;
