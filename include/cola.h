@@ -179,9 +179,9 @@ int cola_ic_from_potentials(cola_ctx* ctx, const float* phi1, const float* phi2,
  * LPT reweight and inverse FFTs of the displacement and acceleration fields,
  * the drift with CIC deposit, the forward FFT, the screened Poisson solve,
  * the force inverse FFTs and the CIC gather with the kick.  Within one call of
- * two or more steps (FP32 fields, per-k LPT path) the kick of each step but
- * the last and the drift + deposit of the next run as one pass over the
- * particles, with the next step's LPT fields formed first; the state after the
+ * two or more steps (FP32 fields; the per-k or the scale-independent LPT path)
+ * the kick of each step but the last and the drift + deposit of the next run as one
+ * pass over the particles, with the next step's LPT fields formed first; the state after the
  * call is that of the same number of single steps (up to the order of the
  * deposit's float additions).  Asynchronous on the stream.  Errors:
  * COLA_ESTATE (before cola_ic), COLA_EINVAL (past the last step), COLA_ECUDA. */
@@ -369,7 +369,7 @@ int cola_batch_set_plan(cola_batch* b, const cola_batch_plan* plan);
 int cola_batch_get_plan(const cola_batch* b, cola_batch_plan* out);
 /* Advances every context by nsteps (-1: to the last step).  With two or more
  * steps, direct particle kernels (deposit_box = gather_box = 0) and every
- * context on the FP32 per-k LPT path, the step boundaries are fused as in
+ * context on an FP32 LPT path, the step boundaries are fused as in
  * cola_step (the kick of each step but the last and the drift + deposit of
  * the next in one pass): nsteps + 1 graph launches, the same state as nsteps
  * single steps up to the order of the deposit's float additions.  When stage

@@ -1270,9 +1270,10 @@ int enqueue_step(cola_ctx* ctx, int n) { return enqueue_group_step(single_group(
 // but the last and the drift + deposit of the next in one pass
 // (k_kick_drift_deposit): step n+1's LPT fields are formed before step n's kick,
 // its kick fields into the other slot.  The particle state after the K steps is
-// the one K separate steps leave.  FP32 fields, per-k LPT path.
+// the one K separate steps leave.  FP32 fields: the per-k path with FP32 seeds, or
+// the scale-independent path (whose Psi1, Psi2 are FP32 and serve both steps).
 bool fused_steps_ok(const cola_ctx* ctx, int K) {
-  return K >= 2 && !ctx->lpt_fast && !ctx->cfg.seed_precision && ctx->lrk[0] != nullptr;
+  return K >= 2 && (ctx->lpt_fast || (!ctx->cfg.seed_precision && ctx->lrk[0] != nullptr));
 }
 
 // The boundary between step n and step n + 1 of every simulation of g in the
@@ -1285,19 +1286,21 @@ int enqueue_group_mid(const Group& g, int n, int cur) {
   const Multi m = g.all;
   const PartParams pp = part_params(ctx);
   const double Pb = (double)ctx->P, Mb = (double)ctx->M;
+  const bool fast = ctx->lpt_fast;
+  const LptMix mix = fast ? lpt_mix_of(ctx, 1, 1, false) : LptMix{};
   bool zeroed = false;
-  CHECK_RC(run_lpt(ctx, 0, 2, true, m, ctx->rho, ctx->M, &zeroed, 1 - cur));
+  if (!fast) CHECK_RC(run_lpt(ctx, 0, 2, true, m, ctx->rho, ctx->M, &zeroed, 1 - cur));
   if (!zeroed) {
     cudaEvent_t e = prof_begin(ctx, ST_RHO_ZERO);
     CK(zero_f32(ctx->rho, ctx->M, ctx->st, m));
     prof_end(ctx, ST_RHO_ZERO, e, 1, m.nb * 4.0 * Mb);
   }
-  const float* const* ka = cur ? ctx->lrk : ctx->lr + 3;
+  const float* const* ka = fast ? ctx->lr : cur ? ctx->lrk : ctx->lr + 3;
   cudaEvent_t e = prof_begin(ctx, ST_KICK_DRIFT_DEPOSIT);
   CK(part_kick_drift_deposit(pp, ctx->s[0], ctx->s[1], ctx->s[2], ctx->v[0], ctx->v[1], ctx->v[2], ka[0], ka[1],
                              ka[2], ctx->lr[0], ctx->lr[1], ctx->lr[2], ctx->F[0], ctx->F[1], ctx->F[2],
                              ctx->fpairs, ctx->rho,
-                             ctx->hdr, ctx->P, ctx->st, m));
+                             ctx->hdr, ctx->P, ctx->st, m, mix));
   prof_end(ctx, ST_KICK_DRIFT_DEPOSIT, e, 1, m.nb * (72.0 * Pb + 20.0 * Mb));
   CK(step_advance(ctx->hdr, ctx->st, m));
   return force_group(g, ctx->a[n + 2], true);

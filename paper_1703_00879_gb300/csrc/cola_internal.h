@@ -256,12 +256,13 @@ cudaError_t part_gather_kick(const PartParams& pp, const float* sx, const float*
 // End of step n (hdr->step = n) and start of step n + 1 in one pass: kick with A_n,
 // closing half kick and drift of step n + 1 with its drift field dp, CIC deposit into rho
 // (zeroed by the caller); acc is not written.  FP32 fields, lattice of Np^3 particles.
+// mix on (row0 1, add_step): A and dp both are Psi1, mix.q2 Psi2.
 cudaError_t part_kick_drift_deposit(const PartParams& pp, float* sx, float* sy, float* sz, float* vx,
                                     float* vy, float* vz, const float* Ax, const float* Ay,
                                     const float* Az, const float* dpx, const float* dpy,
                                     const float* dpz, const float* F0, const float* F1, const float* Fz,
                                     bool pairs, float* rho, const SimHeader* hdr, int64_t P, cudaStream_t s,
-                                    Multi m = {});
+                                    Multi m = {}, LptMix mix = {});
 // The (x, y) pairs of fxy (n cells) into x[0..n) and y[0..n) (either may be null).
 cudaError_t split_pairs(const float2* fxy, float* x, float* y, int64_t n, cudaStream_t s);
 // Per simulation: lq_used = lq_scale (the scale the fields just written, table
