@@ -1203,6 +1203,123 @@ __global__ void __launch_bounds__(NT, 1) k_lpt_z8(ColGeo<N, 8> geo, const void* 
   cp_async_wait<0>();
 }
 
+// The LPT z pass for FP32 seeds up to 256 points: small CTAs as in the other z passes.  A
+// thread reads the seeds of its first-step items, forms d = c1 phi1 + c2 phi2 and A = e1
+// phi1 + e2 phi2 (one table lookup per mode for all four coefficients) and keeps them in
+// registers; the four outputs d, i kz d, A, i kz A are then transformed one after the other
+// through one tile buffer.  Three buffers rotate: the two seed tiles, whose room is free once
+// they are in registers, and one more, so that the next tile's seeds land meanwhile.
+// Against two- and four-array tiles of 256 threads (k_lpt_z, k_lpt_z8): 142 -> 104 us at
+// 256^3, 718 -> 488 us over 256 lattices of 64^3.  A launch of few tiles (one lattice of 64^3
+// or 128^3) is bound by the length of one tile's chain instead and keeps k_lpt_z (10.5 and
+// 24.8 us against 11.1 and 26.8).
+template <int N>
+struct LptZr {
+  static constexpr int TW = ztw(N), T = 128, BUF = fft_rows<N>() * TW;
+  static constexpr size_t smem = (N + 3 * (size_t)BUF) * sizeof(float2);
+};
+
+template <int N>
+__global__ void __launch_bounds__(128, 4) k_lpt_zr(ColGeo<N, LptZr<N>::TW> geo, const float2* __restrict__ phi1,
+                                                   const float2* __restrict__ phi2, float2* __restrict__ o0,
+                                                   float2* __restrict__ o1, float2* __restrict__ o2,
+                                                   float2* __restrict__ o3, LptParams lp0,
+                                                   const float2* __restrict__ twg, int64_t ntiles) {
+  using C = LptZr<N>;
+  constexpr int TW = C::TW, T = C::T, R1 = Split<N>::R1, R2 = Split<N>::R2;
+  constexpr int U = TW * R2, P = (U + T - 1) / T;
+  extern __shared__ __align__(128) float2 sm[];
+  float2* tw = sm;
+  float2 *X = sm + N, *Y = X + C::BUF, *Z = Y + C::BUF;
+  load_tw<T>(tw, twg, N);
+  auto issue = [&](float2* a, float2* b, int64_t t) {
+    int o, c0;
+    int64_t base, by;
+    geo.tile(t, o, c0, base, by);
+    col_issue<N, TW, TW, T>(a, 0, moved(phi1, by), base, geo.ra, geo.rb, c0);
+    col_issue<N, TW, TW, T>(b, 0, moved(phi2, by), base, geo.ra, geo.rb, c0);
+  };
+  if (!geo.m.shift) resolve(lp0, 0);  // one simulation: once per launch
+  int64_t t = blockIdx.x;
+  if (t < ntiles) issue(X, Y, t);
+  cp_async_commit();
+  for (; t < ntiles; t += gridDim.x) {
+    cp_async_wait<0>();
+    __syncthreads();  // tile t's seeds have landed
+    int iy, c0;
+    int64_t base, by;
+    geo.tile(t, iy, c0, base, by);
+    LptParams lp = lp0;
+    resolve(lp, by);
+    const float4* __restrict__ tab = lp.row;
+    const float kf2 = lp.kf * lp.kf;
+    const int fy = freq_index(iy, N);
+    float2 d[P][R1], A[P][R1];
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+      const int u = threadIdx.x + i * T;
+      if ((U % T) == 0 || u < U) {
+        const int c = u % TW, n2 = u / TW, fx = c0 + c;
+#pragma unroll
+        for (int n1 = 0; n1 < R1; ++n1) {
+          const int n = R2 * n1 + n2, fz = freq_index(n, N);
+          const float k2 = kf2 * (float)(fx * fx + fy * fy + fz * fz);
+          d[i][n1] = A[i][n1] = make_float2(0.f, 0.f);
+          if (k2 > 0.f) {
+            const float uu = (0.5f * __logf(k2) - lp.lnk0) * lp.inv_dlnk;
+            const int i0 = min(max((int)floorf(uu), 0), lp.nk - 2);
+            const float f = uu - (float)i0;
+            const float4 t0 = __ldg(tab + i0), t1 = __ldg(tab + i0 + 1);
+            const float2 p1 = X[n * TW + c], p2 = Y[n * TW + c];
+            d[i][n1] = cscale(cadd(cscale(p1, t0.x * (1.f - f) + t1.x * f), cscale(p2, t0.y * (1.f - f) + t1.y * f)),
+                              lp.norm);
+            A[i][n1] = cscale(cadd(cscale(p1, t0.z * (1.f - f) + t1.z * f), cscale(p2, t0.w * (1.f - f) + t1.w * f)),
+                              lp.norm);
+          }
+        }
+      }
+    }
+    __syncthreads();  // every thread has its seeds
+    if (t + gridDim.x < ntiles) issue(Y, Z, t + gridDim.x);
+    cp_async_commit();
+    auto emit = [&](const float2 (&src)[P][R1], bool deriv, float2* out) {
+#pragma unroll
+      for (int i = 0; i < P; ++i) {
+        const int u = threadIdx.x + i * T;
+        if ((U % T) == 0 || u < U) {
+          const int c = u % TW, n2 = u / TW;
+          float2 v[R1];
+#pragma unroll
+          for (int n1 = 0; n1 < R1; ++n1) {
+            const int n = R2 * n1 + n2;
+            const float kz = (n == N / 2) ? 0.f : lp.kf * (float)freq_index(n, N);
+            v[pos_of<R1>(n1)] = deriv ? cscale(cmul_i(src[i][n1]), kz) : src[i][n1];
+          }
+          dftR<R1, true>(v);
+          float2* y = X + n2 * (R1 + 1) * TW + c;
+          y[0] = v[0];
+#pragma unroll
+          for (int k1 = 1; k1 < R1; ++k1) y[k1 * TW] = n2 > 0 ? cmul_conj(v[k1], tw[n2 * k1]) : v[k1];
+        }
+      }
+      __syncthreads();
+      col_inv2<R1, R2, TW, TW, T>(X, ColOut{moved(out, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0});
+    };
+    emit(d, false, o0);
+    __syncthreads();
+    emit(d, true, o1);
+    __syncthreads();
+    emit(A, false, o2);
+    __syncthreads();
+    emit(A, true, o3);
+    float2* x = X;
+    X = Y;
+    Y = Z;
+    Z = x;
+  }
+  cp_async_wait<0>();
+}
+
 // ---------------------------------------------------------------- x passes (rows)
 // A row tile holds TWX rows of the half-length complex transform (M = N/2)
 // row-major in shared memory, row r at st[r * CW + k] (CW = rowtile_pitch<M>),
@@ -2509,6 +2626,20 @@ static cudaError_t launch_lpt8(const void* p1, const void* p2, float2* o0, float
   return cudaGetLastError();
 }
 template <int N>
+static cudaError_t launch_lptr(const void* p1, const void* p2, float2* o0, float2* o1, float2* o2, float2* o3,
+                               const LptParams& lp, const float2* tw, cudaStream_t s, Multi m) {
+  constexpr size_t sm = LptZr<N>::smem;
+  constexpr int TW = LptZr<N>::TW, T = LptZr<N>::T;
+  const int64_t ntiles = col_tiles<N, TW>() * m.nb;
+  auto k = k_lpt_zr<N>;
+  unsigned grid;
+  cudaError_t e = prep(k, sm, ntiles, grid, T);
+  if (e != cudaSuccess) return e;
+  k<<<grid, T, sm, s>>>(geo_z<N, TW>(m), static_cast<const float2*>(p1), static_cast<const float2*>(p2), o0, o1, o2, o3,
+                        lp, tw, ntiles);
+  return cudaGetLastError();
+}
+template <int N>
 static cudaError_t launch_lpt(const void* p1, const void* p2, float2* o0, float2* o1, float2* o2,
                               float2* o3, const LptParams& lp, const float2* tw,
                               cudaStream_t s, Multi m, float* zd, int64_t zn, bool* zeroed) {
@@ -2517,11 +2648,16 @@ static cudaError_t launch_lpt(const void* p1, const void* p2, float2* o0, float2
   if constexpr (N == 256 || N == 512) {
     if (lp.seed_prec == 1) return launch_lpt8<N, 1>(p1, p2, o0, o1, o2, o3, lp, tw, s, m);
     if (lp.seed_prec == 2) return launch_lpt8<N, 2>(p1, p2, o0, o1, o2, o3, lp, tw, s, m);
-    if constexpr (N == 256) return launch_lpt8<N, 0>(p1, p2, o0, o1, o2, o3, lp, tw, s, m);
   }
   if (lp.seed_prec == 1) return launch_lpt_t<N, 1>(p1, p2, o0, o1, o2, o3, lp, tw, s, m, zd, zn, zeroed);
   if (lp.seed_prec == 2) return launch_lpt_t<N, 2>(p1, p2, o0, o1, o2, o3, lp, tw, s, m, zd, zn, zeroed);
-  return launch_lpt_t<N, 0>(p1, p2, o0, o1, o2, o3, lp, tw, s, m, zd, zn, zeroed);
+  if constexpr (N <= 256) {
+    // three tiles and more per resident CTA (4 per SM), or the short chain of k_lpt_z
+    if (N == 256 || col_tiles<N, LptZr<N>::TW>() * m.nb >= 12 * (int64_t)sm_count())
+      return launch_lptr<N>(p1, p2, o0, o1, o2, o3, lp, tw, s, m);
+  }
+  if constexpr (N != 256) return launch_lpt_t<N, 0>(p1, p2, o0, o1, o2, o3, lp, tw, s, m, zd, zn, zeroed);
+  else return cudaErrorInvalidValue;
 }
 
 cudaError_t lpt_z(int Nv, const void* phi1, const void* phi2, float2* o0, float2* o1, float2* o2,
