@@ -124,6 +124,39 @@ __device__ __forceinline__ void resolve(ForceParams& fp, int64_t by) {
 }
 
 
+// Programmatic dependent launches.  The kernels of a step up to 128 points follow one
+// another at a few microseconds each, a good part of it the launch latency between
+// dependent kernels; launched with launch_pdl, a kernel's CTAs become resident while the one
+// before drains and load their twiddles meanwhile.  Such a kernel calls pdl_wait() before it
+// touches anything an earlier kernel writes (twiddle tables are never written by one): it
+// returns once every earlier kernel of the stream has completed and its writes are
+// visible.  pdl_go() lets the next kernel of the stream become resident once every CTA has
+// called it (or ended): it is called when a CTA's input has landed or its last tile begins,
+// not earlier, since waiting CTAs take shared memory and L1 from the running ones.  Both do
+// nothing in a kernel launched the ordinary way.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+//
+// `small` (one simulation on lattices up to 64^3 and meshes up to 128^3, whose kernels run 3 to
+// 25 us) selects it: the whole 32^3 f(R) run of ten steps 513 -> 315 us, eight steps at 64^3 /
+// 128^3 1036 -> 1000 us.  Larger launches are launched the ordinary way: a 256-member batch pass
+// measured 64.9 ms that way and 66.6 ms with it, 512^3 / 1024^3 139.4 and 140.1 ms.
+template <class... P, class... A>
+cudaError_t launch_pdl(bool small, void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... a) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = small ? 1 : 0;
+  return cudaLaunchKernelEx(&c, k, P(a)...);
+}
+
 // Parameters of the per-k LPT reweight (Sec. 4.1): table of float4 per log-k node.
 struct LptParams {
   const SimHeader* hdr;  // table and seed scales of the simulation (moved per simulation)

@@ -191,6 +191,15 @@ __device__ __forceinline__ void load_row_tw(float2* tw, const float2* __restrict
   }
 }
 
+// Start of a kernel launched with launch_pdl: the twiddle table to the start of shared
+// memory, then the wait for the kernels before.
+template <int T>
+__device__ __forceinline__ void pdl_begin(const float2* __restrict__ twg, int n) {
+  extern __shared__ __align__(128) float2 sm[];
+  load_tw<T>(sm, twg, n);
+  pdl_wait();
+}
+
 // ---------------------------------------------------------------- cp.async helpers
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool valid) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
@@ -352,7 +361,7 @@ __device__ __forceinline__ void col_pipeline(Op op, const float2* __restrict__ t
   float2* b0 = sm + N;
   float2* b1 = b0 + BUFELEMS;
   op.extra = b1 + BUFELEMS;  // optional per-op scratch after the two stage buffers
-  load_tw<T>(tw, twg, N);
+  if (!Op::kTwReady) load_tw<T>(tw, twg, N);
   int64_t t = blockIdx.x;
   if (t < ntiles) op.issue(b0, t);
   cp_async_commit();
@@ -367,6 +376,7 @@ __device__ __forceinline__ void col_pipeline(Op op, const float2* __restrict__ t
     cp_async_commit();
     cp_async_wait<Op::kSide ? 2 : 1>();  // tile t's main input has landed
     __syncthreads();
+    if (Op::kTwReady && tn >= ntiles) pdl_go();  // the CTA's last tile
     if constexpr (Op::kSide) {
       op.process(cur ? b1 : b0, tw, t, [&] {
         if (tn < ntiles) op.issue_side(tn);
@@ -532,7 +542,7 @@ __device__ __forceinline__ void col_pipeline_tma(Op op, const float2* __restrict
     fence_bar_init();
     fail = (smem_u32(sm) & 127) ? 1 : 0;  // no copy goes into a misaligned buffer
   }
-  load_tw<T>(tw, twg, N);
+  if (!Op::kTwReady) load_tw<T>(tw, twg, N);
   __syncthreads();
   if (fail) {
     if (lead) atomicAdd(&g_tile_load_failures, 1u);
@@ -568,6 +578,7 @@ __device__ __forceinline__ void col_pipeline_tma(Op op, const float2* __restrict
     }
     __syncthreads();
     if (fail) break;
+    if (Op::kTwReady && tn >= ntiles) pdl_go();  // the CTA's last tile
     if constexpr (SIDE) {
       op.side = TmaSide{&bars[2], (par >> 2) & 1u, &fail};
       // after the tile's second input has been read: the next tile's (unless this one's
@@ -615,6 +626,7 @@ __global__ void k_wait_probe(uint64_t limit_ns) {
 // out = transform of in along the tile axis; out may alias in.
 template <int N, int TW, bool INV>
 struct OpCol {
+  static constexpr bool kTwReady = false;
   static constexpr int T = yt(N);
   ColGeo<N, TW> geo;
   const float2* in;
@@ -788,6 +800,7 @@ __device__ __forceinline__ float smoothing_window(float h, int filter) {
 // per-element switch over the windows slows the pass by a third.
 template <int N, int TW, int MODEL, int T>
 struct OpZScreenField {
+  static constexpr bool kTwReady = true;
   // Between the forward and the inverse transform: delta(k) out to HBM (chameleon-type
   // models: the force pass needs it; the Vainshtein source carries its delta), the
   // field's multiplier (-kappa/k^2, or the smoothing window) applied.
@@ -840,6 +853,7 @@ template <int N, int TW, int MODEL, bool TMA, int T>
 __global__ void __launch_bounds__(T, zblocks(N)) k_z_screen_field(OpZScreenField<N, TW, MODEL, T> op,
                                                        const float2* __restrict__ twg,
                                                        int64_t ntiles, const __grid_constant__ CUtensorMap map) {
+  pdl_begin<T>(twg, N);
   if (!op.geo.m.shift) resolve(op.fp, 0);  // one simulation: once per launch
   if constexpr (TMA) col_pipeline_tma<N, fft_rows<N>() * TW, false, 0, T>(op, twg, ntiles, &map, nullptr);
   else col_pipeline<N, fft_rows<N>() * TW, T>(op, twg, ntiles);
@@ -857,6 +871,7 @@ constexpr size_t zforce_smem() {  // twiddles, two stage buffers, delta(k)
 }
 template <int N, int TW, bool SCREENED, int T>
 struct OpZForce {
+  static constexpr bool kTwReady = true;
   // Phi_tot(k) (App. B) from the transform of S and delta(k) in `dk`; ready() waits for
   // this tile's delta(k) between the forward transform's steps.
   struct Combine {
@@ -933,6 +948,7 @@ template <int N, int TW, bool SCREENED, bool TMA, int T>
 __global__ void __launch_bounds__(T, zblocks(N)) k_z_force(
     OpZForce<N, TW, SCREENED, T> op, const float2* __restrict__ twg, int64_t ntiles,
     const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap dmap) {
+  pdl_begin<T>(twg, N);
   if (!op.geo.m.shift) resolve(op.fp, 0);  // one simulation: once per launch
   if constexpr (TMA) col_pipeline_tma<N, fft_rows<N>() * TW, SCREENED, N * TW, T>(op, twg, ntiles, &map, &dmap);
   else col_pipeline<N, fft_rows<N>() * TW, T>(op, twg, ntiles);
@@ -954,6 +970,7 @@ __device__ __forceinline__ float2 dequant(uint32_t w, float scale) {
 
 template <int N, int TW, int PREC>
 struct OpLptZ {
+  static constexpr bool kTwReady = true;
   ColGeo<N, TW> geo;
   const void *phi1, *phi2;
   float2 *o0, *o1, *o2, *o3;
@@ -1062,6 +1079,7 @@ struct OpLptZ {
 template <int N, int TW, int PREC>
 __global__ void __launch_bounds__(NT, blocks_for_smem(col_smem_c(N, 4), N)) k_lpt_z(OpLptZ<N, TW, PREC> op,
                                               const float2* __restrict__ twg, int64_t ntiles) {
+  pdl_begin<NT>(twg, N);
   if (!op.geo.m.shift) resolve(op.lp, 0);  // one simulation: once per launch
   col_pipeline<N, fft_rows<N>() * 4 * TW>(op, twg, ntiles);
   if (op.zdst && threadIdx.x == 0) bulk_store_drain();  // the zero fill completes with the kernel
@@ -1231,7 +1249,7 @@ __global__ void __launch_bounds__(128, 4) k_lpt_zr(ColGeo<N, LptZr<N>::TW> geo, 
   extern __shared__ __align__(128) float2 sm[];
   float2* tw = sm;
   float2 *X = sm + N, *Y = X + C::BUF, *Z = Y + C::BUF;
-  load_tw<T>(tw, twg, N);
+  pdl_begin<T>(twg, N);
   auto issue = [&](float2* a, float2* b, int64_t t) {
     int o, c0;
     int64_t base, by;
@@ -1281,6 +1299,7 @@ __global__ void __launch_bounds__(128, 4) k_lpt_zr(ColGeo<N, LptZr<N>::TW> geo, 
     }
     __syncthreads();  // every thread has its seeds
     if (t + gridDim.x < ntiles) issue(Y, Z, t + gridDim.x);
+    else pdl_go();  // the CTA's last tile
     cp_async_commit();
     auto emit = [&](const float2 (&src)[P][R1], bool deriv, float2* out) {
 #pragma unroll
@@ -2017,12 +2036,14 @@ __global__ void __launch_bounds__(NT) k_plane_r2c(const float* __restrict__ in, 
   float2* tw = sm;
   float2* buf = sm + N + C::M;
   const int z = blockIdx.x;
-  const int64_t by = shift_of(m, blockIdx.y);
   load_plane_tw<N>(tw, twg);
+  pdl_wait();
+  const int64_t by = shift_of(m, blockIdx.y);
   stage_real_plane<N>(buf, moved(in, by) + (int64_t)z * N * N);
   cp_async_commit();
   cp_async_wait<0>();
   __syncthreads();
+  pdl_go();
   fft_rowtile_r2c<C::M, N, C::CW, NT, ScaleOffset, false, RowStore>(buf, tw + N, tw, ScaleOffset{scale, offset},
                                                                    RowStore{});
   __syncthreads();
@@ -2146,7 +2167,6 @@ __global__ void __launch_bounds__(NT) k_plane_grad(PlaneJobs jobs, const float2*
   float2* tw = sm;
   float2* a = sm + N + C::M;
   const int z = blockIdx.x / jobs.n, q = blockIdx.x - z * jobs.n;
-  const int64_t by = shift_of(m, blockIdx.y), off = (int64_t)z * N * N;
   const float2* in = jobs.in[0];
   float* out = jobs.out[0];
 #pragma unroll
@@ -2156,6 +2176,8 @@ __global__ void __launch_bounds__(NT) k_plane_grad(PlaneJobs jobs, const float2*
       out = jobs.out[i];
     }
   load_plane_tw<N>(tw, twg);
+  pdl_wait();
+  const int64_t by = shift_of(m, blockIdx.y), off = (int64_t)z * N * N;
   stage_complex_plane<N>(a, moved(in, by), z);
   cp_async_commit();
   if (jobs.zdst) {  // this CTA's share of the zero fill while its plane lands
@@ -2165,6 +2187,7 @@ __global__ void __launch_bounds__(NT) k_plane_grad(PlaneJobs jobs, const float2*
   }
   cp_async_wait<0>();
   __syncthreads();
+  pdl_go();
   if ((jobs.dy >> q) & 1) plane_yinv<N, HERM, true>(a, tw, jobs.kfs);
   else plane_yinv<N, HERM, false>(a, tw, 0.f);
   plane_xc2r<N>(a, tw, ((jobs.dx >> q) & 1) ? jobs.kfs : 0.f, moved(out, by) + off);
@@ -2186,13 +2209,15 @@ __global__ void __launch_bounds__(NT) k_plane_screen(const float2* __restrict__ 
   float2* tw = sm;
   float2* a = sm + N + C::M;
   const int z = blockIdx.x;
+  load_plane_tw<N>(tw, twg);
+  pdl_wait();
   const int64_t by = shift_of(m, blockIdx.y);
   resolve(fp, by);
-  load_plane_tw<N>(tw, twg);
   stage_complex_plane<N>(a, moved(w_in, by), z);
   cp_async_commit();
   cp_async_wait<0>();
   __syncthreads();
+  pdl_go();
   plane_yinv<N, true, false>(a, tw, 0.f);
   const ScreenSource<M, MODEL> src{reinterpret_cast<const float2*>(moved(rho, by) + (int64_t)z * N * N),
                                          fp.inv_rhobar, MODEL == 1 ? fp.fr_thr : fp.dgp_coef, fp.C};
@@ -2491,9 +2516,8 @@ static cudaError_t launch_zsf(const float2* in, float2* dk_out, float2* w_out,
     unsigned grid;
     cudaError_t e = prep(k, smk, ntiles, grid, T);
     if (e != cudaSuccess) return e;
-    k<<<grid, T, smk, s>>>(OpZScreenField<N, TW, MODEL, T>{geo_z<N, TW>(m), in, dk_out, w_out, fp}, tw, ntiles,
+    return launch_pdl(N <= 128 && m.nb == 1, k, dim3(grid), T, smk, s, OpZScreenField<N, TW, MODEL, T>{geo_z<N, TW>(m), in, dk_out, w_out, fp}, tw, ntiles,
                             map);
-    return cudaGetLastError();
   };
   auto pick = [&](auto tma_c) {
     if (fp.model == 1) return go(std::integral_constant<int, 1>{}, tma_c);
@@ -2560,9 +2584,8 @@ static cudaError_t launch_zforce_t(const float2* in, const float2* dk, float2* p
     unsigned grid;
     cudaError_t e = prep(k, smk, ntiles, grid, T);
     if (e != cudaSuccess) return e;
-    k<<<grid, T, smk, s>>>(OpZForce<N, TW, SCR, T>{geo_z<N, TW>(m), in, dk, phi, phiz, fp}, tw, ntiles, map,
+    return launch_pdl(N <= 128 && m.nb == 1, k, dim3(grid), T, smk, s, OpZForce<N, TW, SCR, T>{geo_z<N, TW>(m), in, dk, phi, phiz, fp}, tw, ntiles, map,
                             dmap);
-    return cudaGetLastError();
   };
   if constexpr (tma_shape<N, TW>()) {
     if (tma) return go(std::true_type{});
@@ -2607,8 +2630,7 @@ static cudaError_t launch_lpt_t(const void* p1, const void* p2, float2* o0, floa
     const int64_t tps = col_tiles<N, TW>();
     op.zchunk = ((op.zbytes + tps - 1) / tps + 15) / 16 * 16;
   }
-  k<<<grid, NT, sm, s>>>(op, tw, ntiles);
-  e = cudaGetLastError();
+  e = launch_pdl(N <= 128 && m.nb == 1, k, dim3(grid), NT, sm, s, op, tw, ntiles);
   if (e == cudaSuccess && zeroed) *zeroed = zf;
   return e;
 }
@@ -2635,9 +2657,8 @@ static cudaError_t launch_lptr(const void* p1, const void* p2, float2* o0, float
   unsigned grid;
   cudaError_t e = prep(k, sm, ntiles, grid, T);
   if (e != cudaSuccess) return e;
-  k<<<grid, T, sm, s>>>(geo_z<N, TW>(m), static_cast<const float2*>(p1), static_cast<const float2*>(p2), o0, o1, o2, o3,
+  return launch_pdl(N <= 128 && m.nb == 1, k, dim3(grid), T, sm, s, geo_z<N, TW>(m), static_cast<const float2*>(p1), static_cast<const float2*>(p2), o0, o1, o2, o3,
                         lp, tw, ntiles);
-  return cudaGetLastError();
 }
 template <int N>
 static cudaError_t launch_lpt(const void* p1, const void* p2, float2* o0, float2* o1, float2* o2,
@@ -2681,8 +2702,7 @@ static cudaError_t launch_plane_r2c(const float* in, float2* out, float scale, f
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
-    k<<<dim3(N, m.nb), NT, sm, s>>>(in, out, scale, offset, tw, m);
-    return cudaGetLastError();
+    return launch_pdl(N <= 128 && m.nb == 1, k, dim3(N, m.nb), NT, sm, s, in, out, scale, offset, tw, m);
   }
 }
 
@@ -2703,8 +2723,7 @@ static cudaError_t launch_plane_grad(const PlaneJobs& jobs, const float2* tw, cu
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
-    k<<<dim3(jobs.n * N, m.nb), NT, sm, s>>>(jobs, tw, m);
-    return cudaGetLastError();
+    return launch_pdl(N <= 128 && m.nb == 1, k, dim3(jobs.n * N, m.nb), NT, sm, s, jobs, tw, m);
   }
 }
 
@@ -2754,8 +2773,7 @@ static cudaError_t launch_plane_screen(const float2* w_in, const float* rho, flo
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
-    k<<<dim3(N, m.nb), NT, sm, s>>>(w_in, rho, s_out, fp, tw, m);
-    return cudaGetLastError();
+    return launch_pdl(N <= 128 && m.nb == 1, k, dim3(N, m.nb), NT, sm, s, w_in, rho, s_out, fp, tw, m);
   }
 }
 

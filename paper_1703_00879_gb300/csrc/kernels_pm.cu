@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(NTP) k_drift_deposit(
     const float* __restrict__ dpx, const float* __restrict__ dpy,
     const float* __restrict__ dpz, float* __restrict__ rho, StepDt dt, int64_t P, Multi m,
     LptMix mix) {
+  pdl_wait();
   const int64_t p = (int64_t)blockIdx.x * NTP + threadIdx.x;
   const bool valid = p < P;
   const int64_t by = shift_of(m, blockIdx.y);
@@ -274,6 +275,7 @@ __global__ void __launch_bounds__(NTP) k_drift_deposit(
     lattice(pp, p, ix, iy, iz);
     c = cic_setup(pp, ix, iy, iz, nx, ny, nz);
   }
+  pdl_go();
   cic_deposit_merged(rho, pp.Nm, c, valid);
 }
 
@@ -290,6 +292,7 @@ __global__ void __launch_bounds__(NTP) k_gather_kick(
     float* __restrict__ az, const float* __restrict__ Ax, const float* __restrict__ Ay,
     const float* __restrict__ Az, const float* __restrict__ F0, const float* __restrict__ F1,
     const float* __restrict__ Fz, StepDt dt, int64_t P, Multi m, LptMix mix) {
+  pdl_wait();
   const int64_t p0 = (int64_t)blockIdx.x * NTP * PPT + threadIdx.x;
   const int64_t by = shift_of(m, blockIdx.y);
   sx = moved(sx, by);
@@ -341,6 +344,7 @@ __global__ void __launch_bounds__(NTP) k_gather_kick(
       gz[u] = cic_interp(Fz, pp.Nm, c);
     }
   }
+  pdl_go();
   float4 cf = make_float4(0.f, 0.f, 0.f, 0.f);
   if (mix.on) cf = mix_coeffs(mix, by);
   float qs[3] = {1.f, 1.f, 1.f};
@@ -400,6 +404,7 @@ __global__ void __launch_bounds__(NTP, MINB) k_kick_drift_deposit(
     const float* __restrict__ dpx, const float* __restrict__ dpy, const float* __restrict__ dpz,
     const float* __restrict__ F0, const float* __restrict__ F1, const float* __restrict__ Fz,
     float* __restrict__ rho, const SimHeader* __restrict__ hdr, int64_t P, Multi m, LptMix mix) {
+  pdl_wait();
   const int64_t p0 = (int64_t)blockIdx.x * NTP * Q + threadIdx.x;
   const int64_t by = shift_of(m, blockIdx.y);
   sx = moved(sx, by);
@@ -455,6 +460,7 @@ __global__ void __launch_bounds__(NTP, MINB) k_kick_drift_deposit(
       gz[u] = cic_interp(Fz, pp.Nm, c);
     }
   }
+  pdl_go();
 #pragma unroll
   for (int u = 0; u < Q; ++u) {
     const int64_t p = patch84(pp, p0 + u * NTP);
@@ -1105,6 +1111,8 @@ __global__ void __launch_bounds__(NTP) k_pk_bin(const float2* __restrict__ dk, i
 inline unsigned blocks_for(int64_t n) { return (unsigned)((n + NTP - 1) / NTP); }
 
 __global__ void k_step_advance(SimHeader* hdr, Multi m) {
+  pdl_go();
+  pdl_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b < m.nb) moved(hdr, shift_of(m, b))->step += 1;
 }
@@ -1236,9 +1244,8 @@ cudaError_t part_drift_deposit(const PartParams& pp, float* sx, float* sy, float
         pp, sx, sy, sz, vx, vy, vz, ax, ay, az, dpx, dpy, dpz, rho, dt, m, mix, g_dep_box);
     return cudaGetLastError();
   }
-  k_drift_deposit<<<dim3(blocks_for(P), m.nb), NTP, 0, s>>>(pp, sx, sy, sz, vx, vy, vz, ax, ay, az,
-                                                            dpx, dpy, dpz, rho, dt, P, m, mix);
-  return cudaGetLastError();
+  return launch_pdl(P <= (1 << 18) && m.nb == 1, k_drift_deposit, dim3(blocks_for(P), m.nb), NTP, 0, s, pp, sx, sy, sz, vx, vy, vz, ax, ay, az,
+                    dpx, dpy, dpz, rho, dt, P, m, mix);
 }
 
 cudaError_t part_gather_kick(const PartParams& pp, const float* sx, const float* sy,
@@ -1255,9 +1262,8 @@ cudaError_t part_gather_kick(const PartParams& pp, const float* sx, const float*
     return cudaGetLastError();
   }
   auto k = pairs ? k_gather_kick<true> : k_gather_kick<false>;
-  k<<<dim3((unsigned)((P + NTP * PPT - 1) / (NTP * PPT)), m.nb), NTP, 0, s>>>(
-      pp, sx, sy, sz, vx, vy, vz, ax, ay, az, Ax, Ay, Az, F0, F1, Fz, dt, P, m, mix);
-  return cudaGetLastError();
+  return launch_pdl(P <= (1 << 18) && m.nb == 1, k, dim3((unsigned)((P + NTP * PPT - 1) / (NTP * PPT)), m.nb), NTP, 0, s, pp, sx, sy, sz, vx, vy, vz,
+                    ax, ay, az, Ax, Ay, Az, F0, F1, Fz, dt, P, m, mix);
 }
 
 cudaError_t split_pairs(const float2* fxy, float* x, float* y, int64_t n, cudaStream_t s) {
@@ -1278,9 +1284,8 @@ cudaError_t part_kick_drift_deposit(const PartParams& pp, float* sx, float* sy, 
   constexpr int Q = 2;
   auto k = mix.on ? (pairs ? k_kick_drift_deposit<Q, 4, true, true> : k_kick_drift_deposit<Q, 4, false, true>)
                   : (pairs ? k_kick_drift_deposit<Q, 4, true, false> : k_kick_drift_deposit<Q, 4, false, false>);
-  k<<<dim3((unsigned)((P + NTP * Q - 1) / (NTP * Q)), m.nb), NTP, 0, s>>>(
-      pp, sx, sy, sz, vx, vy, vz, Ax, Ay, Az, dpx, dpy, dpz, F0, F1, Fz, rho, hdr, P, m, mix);
-  return cudaGetLastError();
+  return launch_pdl(P <= (1 << 18) && m.nb == 1, k, dim3((unsigned)((P + NTP * Q - 1) / (NTP * Q)), m.nb), NTP, 0, s, pp, sx, sy, sz, vx, vy, vz, Ax,
+                    Ay, Az, dpx, dpy, dpz, F0, F1, Fz, rho, hdr, P, m, mix);
 }
 
 cudaError_t part_snapshot(const PartParams& pp, const float* sx, const float* sy, const float* sz,
@@ -1341,8 +1346,7 @@ cudaError_t count_nonfinite(const float* const* f, int nf, int64_t n, unsigned l
 }
 
 cudaError_t step_advance(SimHeader* hdr, cudaStream_t s, Multi m) {
-  k_step_advance<<<(m.nb + 127) / 128, 128, 0, s>>>(hdr, m);
-  return cudaGetLastError();
+  return launch_pdl(m.nb == 1, k_step_advance, dim3((m.nb + 127) / 128), 128, 0, s, hdr, m);
 }
 
 cudaError_t set_header(SimHeader* hdr, const SimHeader& v, cudaStream_t s) {
