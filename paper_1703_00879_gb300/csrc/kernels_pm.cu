@@ -192,19 +192,24 @@ __global__ void __launch_bounds__(NTP) k_deposit(PartParams pp, const float* __r
   cic_deposit(rho, pp.Nm, cic_setup(pp, ix, iy, iz, sx[p], sy[p], sz[p]));
 }
 
-// Particle of work item i of the gather: a warp takes an 8 x 4 patch of the
-// Lagrangian lattice (8 along x, 4 along y) instead of 32 along x.  Loads of
-// per-particle arrays still fill whole 32-byte sectors, and once the particles
-// have clustered a compact patch touches fewer mesh sectors than a line (the
-// last step's gather 9.95 -> 6.9 ms at 512^3 / 1024^3).  The deposit keeps
-// lines: its atomics from a patch collide more (4.0 -> 4.5 ms at the first step).
-__device__ __forceinline__ int64_t patch84(const PartParams& pp, int64_t i) {
+// Particle of work item i of the gather: a warp takes a 16 x 2 patch of the
+// Lagrangian lattice (16 along x, 2 along y).  Both kinds of access count there: each
+// per-particle array costs a wavefront per lattice row of the patch and each mesh load one
+// per 128-byte line it touches.  A line of 32 touches the most mesh rows once the
+// particles have clustered; 8 x 4 spends twice the wavefronts on the particle arrays (18
+// of the fused pass's 34 accesses per particle).  Per launch, 8 x 4 -> 16 x 2: fused pass 512^3 /
+// 1024^3 9.27 -> 9.09 ms, 256^3 / 512^3 895 -> 864 us, 256 x 64^3 / 128^3 3.61 -> 3.39 ms, 256^3 /
+// 256^3 scale-independent 739 -> 630 us; gather + kick 5.35 -> 4.95 ms, 584 -> 545, 2460 -> 2397,
+// 421 -> 371 us (lines of 32: 9.95 ms against 6.9 with 8 x 4 at the last step of a 512^3 run).
+// The deposit alone keeps lines: its atomics from a patch collide more (4.0 -> 4.5 ms at the
+// first step).
+__device__ __forceinline__ int64_t patch16x2(const PartParams& pp, int64_t i) {
   const int lane = (int)(i & 31);
   const int64_t w = i >> 5;
-  const int xw = pp.lgNp - 3;                      // warps along x per 4-row band
-  const int64_t xh = w & ((1 << xw) - 1), band = w >> xw;  // band = z Np/4 + y/4
-  const int64_t x = (xh << 3) | (lane & 7);
-  const int64_t yz = (band << 2) | (lane >> 3);    // y + z Np (4 | Np)
+  const int xw = pp.lgNp - 4;                      // warps along x per 2-row band
+  const int64_t xh = w & ((1 << xw) - 1), band = w >> xw;  // band = z Np/2 + y/2
+  const int64_t x = (xh << 4) | (lane & 15);
+  const int64_t yz = (band << 1) | (lane >> 4);    // y + z Np (2 | Np)
   return (yz << pp.lgNp) | x;
 }
 
@@ -318,7 +323,7 @@ __global__ void __launch_bounds__(NTP) k_gather_kick(
   float px[PPT], py[PPT], pz[PPT];
 #pragma unroll
   for (int u = 0; u < PPT; ++u) {
-    const int64_t p = patch84(pp, p0 + u * NTP);
+    const int64_t p = patch16x2(pp, p0 + u * NTP);
     if (p0 + u * NTP < P) {
       px[u] = sx[p];
       py[u] = sy[p];
@@ -328,7 +333,7 @@ __global__ void __launch_bounds__(NTP) k_gather_kick(
   float gx[PPT], gy[PPT], gz[PPT];
 #pragma unroll
   for (int u = 0; u < PPT; ++u) {
-    const int64_t p = patch84(pp, p0 + u * NTP);
+    const int64_t p = patch16x2(pp, p0 + u * NTP);
     if (p0 + u * NTP < P) {
       int ix, iy, iz;
       lattice(pp, p, ix, iy, iz);
@@ -354,7 +359,7 @@ __global__ void __launch_bounds__(NTP) k_gather_kick(
   }
 #pragma unroll
   for (int u = 0; u < PPT; ++u) {
-    const int64_t p = patch84(pp, p0 + u * NTP);
+    const int64_t p = patch16x2(pp, p0 + u * NTP);
     if (p0 + u * NTP < P) {
       float lx, ly, lz;
       if (dt.lq) {  // 16-bit kick fields, one scale per field
@@ -390,12 +395,12 @@ __global__ void __launch_bounds__(NTP) k_gather_kick(
 // are those of k_gather_kick followed by k_drift_deposit, so the particle state
 // is the same bit for bit; acc is not stored (the next gather forms it again)
 // and delta_v and s are read and written once instead of twice.  hdr->step = n.
-// Particles as in the gather (8 x 4 lattice patches per warp, PPT per thread).
+// Particles as in the gather (16 x 2 lattice patches per warp, PPT per thread).
 // MIX (the scale-independent path): A and dp hold Psi1 (one set of arrays) and mix.q2
 // Psi2; A_n and dPsi_{n+1} are formed from them with rows 1 + n and 2 + n of the growth
 // table, so the pass reads the six fields once for both (72 bytes per particle instead
-// of the 156 of the two kernels).  256^3 particles / 256^3 mesh, LCDM: 739 us against 443
-// for the drift + deposit and 421 for the gather + kick.
+// of the 156 of the two kernels).  256^3 particles / 256^3 mesh, LCDM: 630 us against 443
+// for the drift + deposit and 371 for the gather + kick.
 template <int Q, int MINB, bool XY, bool MIX>
 __global__ void __launch_bounds__(NTP, MINB) k_kick_drift_deposit(
     PartParams pp, float* __restrict__ sx, float* __restrict__ sy, float* __restrict__ sz,
@@ -434,7 +439,7 @@ __global__ void __launch_bounds__(NTP, MINB) k_kick_drift_deposit(
   float px[Q], py[Q], pz[Q];
 #pragma unroll
   for (int u = 0; u < Q; ++u) {
-    const int64_t p = patch84(pp, p0 + u * NTP);
+    const int64_t p = patch16x2(pp, p0 + u * NTP);
     if (p0 + u * NTP < P) {
       px[u] = sx[p];
       py[u] = sy[p];
@@ -444,7 +449,7 @@ __global__ void __launch_bounds__(NTP, MINB) k_kick_drift_deposit(
   float gx[Q], gy[Q], gz[Q];
 #pragma unroll
   for (int u = 0; u < Q; ++u) {
-    const int64_t p = patch84(pp, p0 + u * NTP);
+    const int64_t p = patch16x2(pp, p0 + u * NTP);
     if (p0 + u * NTP < P) {
       int ix, iy, iz;
       lattice(pp, p, ix, iy, iz);
@@ -463,7 +468,7 @@ __global__ void __launch_bounds__(NTP, MINB) k_kick_drift_deposit(
   pdl_go();
 #pragma unroll
   for (int u = 0; u < Q; ++u) {
-    const int64_t p = patch84(pp, p0 + u * NTP);
+    const int64_t p = patch16x2(pp, p0 + u * NTP);
     const bool valid = p0 + u * NTP < P;
     Cic c{};
     if (valid) {
