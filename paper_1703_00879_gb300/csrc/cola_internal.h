@@ -210,6 +210,9 @@ cudaError_t fft_xc2r_multi16(int N, int njobs, const float2* const* in, void* co
 // axis 1 = y, 2 = z; in place
 cudaError_t fft_col(int N, float2* data, int axis, bool inv, const float2* tw, cudaStream_t s,
                     Multi m = {});
+// y pass between the interleaved half spectrum `data` and the dense one: forward data ->
+// dense, inverse dense -> data (one simulation).
+cudaError_t fft_y_dense(int N, float2* data, float2* dense, bool inv, const float2* tw, cudaStream_t s);
 // y inverse pass producing the plain transform (out_plain may alias in) and the
 // transform of (i kfs f_y) times the input (out_deriv).
 cudaError_t fft_yinv2(int N, const float2* in, float2* out_plain, float2* out_deriv, float kfs,

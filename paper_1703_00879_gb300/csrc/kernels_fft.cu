@@ -623,8 +623,34 @@ __global__ void k_wait_probe(uint64_t limit_ns) {
 }
 
 // ---------------------------------------------------------------- plain column pass
-// out = transform of in along the tile axis; out may alias in.
-template <int N, int TW, bool INV>
+// Dense half spectra [z][y][kx] of the public API (rows of N/2 + 1 values, no padding) as
+// the far side of a y pass: stores of a column transform, and the staging of its tiles
+// (8-byte pieces: an odd row length leaves no 16-byte alignment).
+template <int N>
+struct DenseOut {
+  static constexpr bool kSmem = false;
+  float2* g;  // element (row 0, column 0) of the tile
+  int live;
+  __device__ __forceinline__ float2 operator()(float2 v, int n, int c, int) const {
+    if (c < live) g[n * (N / 2 + 1) + c] = v;
+    return v;
+  }
+  __device__ __forceinline__ void ready() const {}
+};
+template <int N, int TW, int T>
+__device__ __forceinline__ void col_issue_dense(float2* buf, const float2* __restrict__ g, int live) {
+  const int c = threadIdx.x % TW;
+  const int sz = c < live ? 8 : 0;  // 0: zero-fill, nothing read
+#pragma unroll 4
+  for (int n = threadIdx.x / TW; n < N; n += T / TW)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(smem_u32(buf + n * TW + c)),
+                 "l"(g + (c < live ? n * (N / 2 + 1) + c : 0)), "r"(sz)
+                 : "memory");
+}
+
+// out = transform of in along the tile axis; out may alias in.  DENSE (along y): 1 the
+// output, 2 the input is a dense half spectrum.
+template <int N, int TW, bool INV, int DENSE>
 struct OpCol {
   static constexpr bool kTwReady = false;
   static constexpr int T = yt(N);
@@ -637,20 +663,26 @@ struct OpCol {
     int o, c0;
     int64_t base, by;
     geo.tile(t, o, c0, base, by);
-    col_issue<N, TW, TW, T>(buf, 0, moved(in, by), base, geo.ra, geo.rb, c0);
+    if constexpr (DENSE == 2)
+      col_issue_dense<N, TW, T>(buf, in + (int64_t)o * N * (N / 2 + 1) + c0, N / 2 + 1 - c0);
+    else col_issue<N, TW, TW, T>(buf, 0, moved(in, by), base, geo.ra, geo.rb, c0);
   }
-  // outputs go to HBM from the last step's registers (ColOut)
+  // outputs go to HBM from the last step's registers
   __device__ __forceinline__ void process(float2* buf, const float2* tw, int64_t t) const {
     int o, c0;
     int64_t base, by;
     geo.tile(t, o, c0, base, by);
-    fft_tile<N, TW, TW, T, INV, 1, TileLoad, ColOut>(
-        buf, tw, TileLoad{}, ColOut{moved(out, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0});
+    if constexpr (DENSE == 1)
+      fft_tile<N, TW, TW, T, INV, 1, TileLoad, DenseOut<N>>(
+          buf, tw, TileLoad{}, DenseOut<N>{out + (int64_t)o * N * (N / 2 + 1) + c0, N / 2 + 1 - c0});
+    else
+      fft_tile<N, TW, TW, T, INV, 1, TileLoad, ColOut>(
+          buf, tw, TileLoad{}, ColOut{moved(out, by) + base, geo.ra, geo.rb, N / 2 + 1 - c0});
   }
 };
 
-template <int N, int TW, bool INV, bool TMA>
-__global__ void __launch_bounds__(yt(N), ycol_blocks(N)) k_col(OpCol<N, TW, INV> op, const float2* __restrict__ twg,
+template <int N, int TW, bool INV, bool TMA, int DENSE>
+__global__ void __launch_bounds__(yt(N), ycol_blocks(N)) k_col(OpCol<N, TW, INV, DENSE> op, const float2* __restrict__ twg,
                                             int64_t ntiles, const __grid_constant__ CUtensorMap map) {
   constexpr int T = yt(N);
   if constexpr (TMA) col_pipeline_tma<N, fft_rows<N>() * TW, false, 0, T>(op, twg, ntiles, &map, nullptr);
@@ -2439,36 +2471,39 @@ constexpr bool tma_shape() {
   return N >= 1024 && TW <= 8 && TW % 2 == 0;
 }
 
-template <int N>
-static cudaError_t launch_col(float2* data, int axis, bool inv, const float2* tw,
-                              cudaStream_t s, Multi m) {
+// DENSE as in OpCol (in or out is then a dense half spectrum, axis 1)
+template <int N, bool INV, int DENSE>
+static cudaError_t launch_col(const float2* in, float2* out, int axis, const float2* tw, cudaStream_t s, Multi m) {
   constexpr int TW = ytw(N);
-  constexpr size_t sm = col_smem_tw(N, TW);
   const int64_t ntiles = col_tiles<N, TW>() * m.nb;
   const ColGeo<N, TW> geo = axis == 1 ? geo_y<N, TW>(m) : geo_z<N, TW>(m);
   CUtensorMap map{};
-  const bool tma = tma_shape<N, TW>() && !m.shift && spectrum_map(map, data, N, TW, axis != 1);
-  auto go = [&](auto inv_c, auto tma_c) {
-    constexpr bool INV = decltype(inv_c)::value, TMA = decltype(tma_c)::value;
-    constexpr size_t smk = TMA ? tma_smem<N, fft_rows<N>() * TW, 0>() : sm;
-    auto k = k_col<N, TW, INV, TMA>;
+  auto go = [&](auto tma_c) {
+    constexpr bool TMA = decltype(tma_c)::value;
+    constexpr size_t smk = TMA ? tma_smem<N, fft_rows<N>() * TW, 0>() : col_smem_tw(N, TW);
+    auto k = k_col<N, TW, INV, TMA, DENSE>;
     unsigned grid;
     cudaError_t e = prep(k, smk, ntiles, grid, yt(N));
     if (e != cudaSuccess) return e;
-    k<<<grid, yt(N), smk, s>>>(OpCol<N, TW, INV>{geo, data, data}, tw, ntiles, map);
+    k<<<grid, yt(N), smk, s>>>(OpCol<N, TW, INV, DENSE>{geo, in, out}, tw, ntiles, map);
     return cudaGetLastError();
   };
-  using T = std::true_type;
-  using F = std::false_type;
-  if constexpr (tma_shape<N, TW>()) {
-    if (tma) return inv ? go(T{}, T{}) : go(F{}, T{});
+  if constexpr (tma_shape<N, TW>() && DENSE != 2) {
+    if (!m.shift && spectrum_map(map, in, N, TW, axis != 1)) return go(std::true_type{});
   }
-  return inv ? go(T{}, F{}) : go(F{}, F{});
+  return go(std::false_type{});
 }
 
 cudaError_t fft_col(int Nv, float2* data, int axis, bool inv, const float2* tw, cudaStream_t s,
                     Multi m) {
-  COLA_SWITCH_N(Nv, return launch_col<N>(data, axis, inv, tw, s, m));
+  COLA_SWITCH_N(Nv, return inv ? launch_col<N, true, 0>(data, data, axis, tw, s, m)
+                               : launch_col<N, false, 0>(data, data, axis, tw, s, m));
+  return cudaSuccess;
+}
+
+cudaError_t fft_y_dense(int Nv, float2* data, float2* dense, bool inv, const float2* tw, cudaStream_t s) {
+  COLA_SWITCH_N(Nv, return inv ? launch_col<N, true, 2>(dense, data, 1, tw, s, Multi{})
+                               : launch_col<N, false, 1>(data, dense, 1, tw, s, Multi{}));
   return cudaSuccess;
 }
 
