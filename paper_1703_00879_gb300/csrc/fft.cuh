@@ -42,6 +42,12 @@ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return __fmul2_rn(a, make_float2(s, s)); }
 // multiply by +i
 __device__ __forceinline__ float2 cmul_i(float2 a) { return make_float2(-a.y, a.x); }
+// i f a, each product rounded on its own.  cscale(cmul_i(a), f) may fuse with the additions
+// of a transform that follows; this gives the value that a product stored in a pass of its
+// own has (the LPT fields depend on it bit for bit where they are kept in 16 bits).
+__device__ __forceinline__ float2 cmul_if(float2 a, float f) {
+  return make_float2(__fmul_rn(-f, a.y), __fmul_rn(f, a.x));
+}
 // multiply by -i (forward) or +i (inverse)
 template <bool INV>
 __device__ __forceinline__ float2 rot_q(float2 a) {
@@ -537,8 +543,7 @@ __device__ __forceinline__ void fft_tile_inv_deriv(float2* __restrict__ buf, flo
         const float2 x = buf[n * PITCH + c];
         const float f = n == L / 2 ? 0.f : kfs * (float)(n < L / 2 ? n : n - L);
         v[i][pos_of<R1>(n1)] = x;
-        // rounded products: left to the compiler they may fuse with the first butterflies
-        d[pos_of<R1>(n1)] = make_float2(__fmul_rn(-f, x.y), __fmul_rn(f, x.x));
+        d[pos_of<R1>(n1)] = cmul_if(x, f);
       }
       dftR<R1, true>(d);
       dftR<R1, true>(v[i]);

@@ -2119,8 +2119,7 @@ struct PlaneLoad {
   float kfs;
   __device__ __forceinline__ float2 in(float2 v, int n) const {
     if (!DY) return v;
-    const float f = (n == N / 2) ? 0.f : kfs * (float)freq_index(n, N);
-    return cscale(cmul_i(v), f);
+    return cmul_if(v, (n == N / 2) ? 0.f : kfs * (float)freq_index(n, N));
   }
   __device__ __forceinline__ float2 operator()(const float2* buf, int n, int c, int at) const {
     float2 v = in(buf[at], n);
