@@ -11,6 +11,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "cola_internal.h"
 
@@ -125,24 +126,39 @@ __device__ __forceinline__ void cic_deposit_merged(float* __restrict__ rho, int 
   row_add(rho + (z1 + c.i1[1]) * Nm, c.i0[0], c.i1[0], w[6], w[7]);
 }
 
-__device__ __forceinline__ float cic_interp(const float* __restrict__ F, int Nm, const Cic& c) {
+// Parameter type of an array that the launch just before may write, and a load from it.  DEP: the
+// kernel was launched dependently (launch_pdl) and is resident while that launch still runs, so
+// the array is not constant for the kernel's lifetime: it is read by ordinary loads after
+// pdl_wait(), through a pointer that is not __restrict__ (either would let the compiler read it
+// early or through the read-only path, which is not kept coherent).
+template <bool DEP>
+using InPtr = std::conditional_t<DEP, const float*, const float* __restrict__>;
+template <bool DEP, class T>
+__device__ __forceinline__ T ld_in(const T* p) {
+  if constexpr (DEP) return *p;
+  else return __ldg(p);
+}
+
+template <bool DEP = false>
+__device__ __forceinline__ float cic_interp(const float* F, int Nm, const Cic& c) {
   const float wx0 = 1.f - c.f[0], wx1 = c.f[0];
   const float wy0 = 1.f - c.f[1], wy1 = c.f[1];
   const float wz0 = 1.f - c.f[2], wz1 = c.f[2];
   const int64_t z0 = (int64_t)c.i0[2] * Nm, z1 = (int64_t)c.i1[2] * Nm;
   const int64_t r00 = (z0 + c.i0[1]) * Nm, r01 = (z0 + c.i1[1]) * Nm;
   const int64_t r10 = (z1 + c.i0[1]) * Nm, r11 = (z1 + c.i1[1]) * Nm;
-  const float a00 = wx0 * __ldg(F + r00 + c.i0[0]) + wx1 * __ldg(F + r00 + c.i1[0]);
-  const float a01 = wx0 * __ldg(F + r01 + c.i0[0]) + wx1 * __ldg(F + r01 + c.i1[0]);
-  const float a10 = wx0 * __ldg(F + r10 + c.i0[0]) + wx1 * __ldg(F + r10 + c.i1[0]);
-  const float a11 = wx0 * __ldg(F + r11 + c.i0[0]) + wx1 * __ldg(F + r11 + c.i1[0]);
+  const float a00 = wx0 * ld_in<DEP>(F + r00 + c.i0[0]) + wx1 * ld_in<DEP>(F + r00 + c.i1[0]);
+  const float a01 = wx0 * ld_in<DEP>(F + r01 + c.i0[0]) + wx1 * ld_in<DEP>(F + r01 + c.i1[0]);
+  const float a10 = wx0 * ld_in<DEP>(F + r10 + c.i0[0]) + wx1 * ld_in<DEP>(F + r10 + c.i1[0]);
+  const float a11 = wx0 * ld_in<DEP>(F + r11 + c.i0[0]) + wx1 * ld_in<DEP>(F + r11 + c.i1[0]);
   return wz0 * (wy0 * a00 + wy1 * a01) + wz1 * (wy0 * a10 + wy1 * a11);
 }
 
 // (F_x, F_y) at the particle from the interleaved pair mesh Fxy (one float2 per
 // cell): the same weights and operation order as cic_interp per component, one
 // 8-byte load per corner instead of two 4-byte loads.
-__device__ __forceinline__ float2 cic_interp2(const float2* __restrict__ F, int Nm, const Cic& c) {
+template <bool DEP = false>
+__device__ __forceinline__ float2 cic_interp2(const float2* F, int Nm, const Cic& c) {
   const float wx0 = 1.f - c.f[0], wx1 = c.f[0];
   const float wy0 = 1.f - c.f[1], wy1 = c.f[1];
   const float wz0 = 1.f - c.f[2], wz1 = c.f[2];
@@ -150,7 +166,7 @@ __device__ __forceinline__ float2 cic_interp2(const float2* __restrict__ F, int 
   const int64_t r00 = (z0 + c.i0[1]) * Nm, r01 = (z0 + c.i1[1]) * Nm;
   const int64_t r10 = (z1 + c.i0[1]) * Nm, r11 = (z1 + c.i1[1]) * Nm;
   auto row = [&](int64_t r) {
-    const float2 a = __ldg(F + r + c.i0[0]), b = __ldg(F + r + c.i1[0]);
+    const float2 a = ld_in<DEP>(F + r + c.i0[0]), b = ld_in<DEP>(F + r + c.i1[0]);
     return make_float2(wx0 * a.x + wx1 * b.x, wx0 * a.y + wx1 * b.y);
   };
   const float2 a00 = row(r00), a01 = row(r01), a10 = row(r10), a11 = row(r11);
@@ -215,14 +231,15 @@ __device__ __forceinline__ int64_t patch16x2(const PartParams& pp, int64_t i) {
 
 // Sec. 2 drift in the LPT frame: delta_v += acc dtk (closing the previous
 // half kick), s += delta_v dtd + dPsi_LPT(q); then CIC deposit of x = q + s.
+// DEP: launched dependently, after the LPT pass that writes dp (InPtr).
+template <bool DEP>
 __global__ void __launch_bounds__(NTP) k_drift_deposit(
     PartParams pp, float* __restrict__ sx, float* __restrict__ sy, float* __restrict__ sz,
     float* __restrict__ vx, float* __restrict__ vy, float* __restrict__ vz,
     const float* __restrict__ ax, const float* __restrict__ ay, const float* __restrict__ az,
-    const float* __restrict__ dpx, const float* __restrict__ dpy,
-    const float* __restrict__ dpz, float* __restrict__ rho, StepDt dt, int64_t P, Multi m,
+    InPtr<DEP> dpx, InPtr<DEP> dpy, InPtr<DEP> dpz, float* __restrict__ rho, StepDt dt, int64_t P, Multi m,
     LptMix mix) {
-  pdl_wait();
+  if constexpr (DEP) pdl_wait();
   const int64_t p = (int64_t)blockIdx.x * NTP + threadIdx.x;
   const bool valid = p < P;
   const int64_t by = shift_of(m, blockIdx.y);
@@ -289,15 +306,16 @@ __global__ void __launch_bounds__(NTP) k_drift_deposit(
 // (displacement load -> cell index -> 24 mesh loads) of different particles overlap.
 constexpr int PPT = 2;
 
-template <bool XY>
+// DEP: launched dependently, after the force pass that writes F (InPtr).
+template <bool XY, bool DEP>
 __global__ void __launch_bounds__(NTP) k_gather_kick(
     PartParams pp, const float* __restrict__ sx, const float* __restrict__ sy,
     const float* __restrict__ sz, float* __restrict__ vx, float* __restrict__ vy,
     float* __restrict__ vz, float* __restrict__ ax, float* __restrict__ ay,
     float* __restrict__ az, const float* __restrict__ Ax, const float* __restrict__ Ay,
-    const float* __restrict__ Az, const float* __restrict__ F0, const float* __restrict__ F1,
-    const float* __restrict__ Fz, StepDt dt, int64_t P, Multi m, LptMix mix) {
-  pdl_wait();
+    const float* __restrict__ Az, InPtr<DEP> F0, InPtr<DEP> F1, InPtr<DEP> Fz, StepDt dt, int64_t P, Multi m,
+    LptMix mix) {
+  if constexpr (DEP) pdl_wait();
   const int64_t p0 = (int64_t)blockIdx.x * NTP * PPT + threadIdx.x;
   const int64_t by = shift_of(m, blockIdx.y);
   sx = moved(sx, by);
@@ -339,14 +357,14 @@ __global__ void __launch_bounds__(NTP) k_gather_kick(
       lattice(pp, p, ix, iy, iz);
       const Cic c = cic_setup(pp, ix, iy, iz, px[u], py[u], pz[u]);
       if constexpr (XY) {  // (F_x, F_y) pairs in F0
-        const float2 gxy = cic_interp2(reinterpret_cast<const float2*>(F0), pp.Nm, c);
+        const float2 gxy = cic_interp2<DEP>(reinterpret_cast<const float2*>(F0), pp.Nm, c);
         gx[u] = gxy.x;
         gy[u] = gxy.y;
       } else {
-        gx[u] = cic_interp(F0, pp.Nm, c);
-        gy[u] = cic_interp(F1, pp.Nm, c);
+        gx[u] = cic_interp<DEP>(F0, pp.Nm, c);
+        gy[u] = cic_interp<DEP>(F1, pp.Nm, c);
       }
-      gz[u] = cic_interp(Fz, pp.Nm, c);
+      gz[u] = cic_interp<DEP>(Fz, pp.Nm, c);
     }
   }
   pdl_go();
@@ -401,15 +419,15 @@ __global__ void __launch_bounds__(NTP) k_gather_kick(
 // table, so the pass reads the six fields once for both (72 bytes per particle instead
 // of the 156 of the two kernels).  256^3 particles / 256^3 mesh, LCDM: 630 us against 443
 // for the drift + deposit and 371 for the gather + kick.
-template <int Q, int MINB, bool XY, bool MIX>
+// DEP: launched dependently, after the LPT pass that writes dp (InPtr).
+template <int Q, int MINB, bool XY, bool MIX, bool DEP>
 __global__ void __launch_bounds__(NTP, MINB) k_kick_drift_deposit(
     PartParams pp, float* __restrict__ sx, float* __restrict__ sy, float* __restrict__ sz,
     float* __restrict__ vx, float* __restrict__ vy, float* __restrict__ vz,
     const float* __restrict__ Ax, const float* __restrict__ Ay, const float* __restrict__ Az,
-    const float* __restrict__ dpx, const float* __restrict__ dpy, const float* __restrict__ dpz,
-    const float* __restrict__ F0, const float* __restrict__ F1, const float* __restrict__ Fz,
+    InPtr<DEP> dpx, InPtr<DEP> dpy, InPtr<DEP> dpz, InPtr<DEP> F0, InPtr<DEP> F1, InPtr<DEP> Fz,
     float* __restrict__ rho, const SimHeader* __restrict__ hdr, int64_t P, Multi m, LptMix mix) {
-  pdl_wait();
+  if constexpr (DEP) pdl_wait();
   const int64_t p0 = (int64_t)blockIdx.x * NTP * Q + threadIdx.x;
   const int64_t by = shift_of(m, blockIdx.y);
   sx = moved(sx, by);
@@ -455,14 +473,14 @@ __global__ void __launch_bounds__(NTP, MINB) k_kick_drift_deposit(
       lattice(pp, p, ix, iy, iz);
       const Cic c = cic_setup(pp, ix, iy, iz, px[u], py[u], pz[u]);
       if constexpr (XY) {  // (F_x, F_y) pairs in F0
-        const float2 gxy = cic_interp2(reinterpret_cast<const float2*>(F0), pp.Nm, c);
+        const float2 gxy = cic_interp2<DEP>(reinterpret_cast<const float2*>(F0), pp.Nm, c);
         gx[u] = gxy.x;
         gy[u] = gxy.y;
       } else {
-        gx[u] = cic_interp(F0, pp.Nm, c);
-        gy[u] = cic_interp(F1, pp.Nm, c);
+        gx[u] = cic_interp<DEP>(F0, pp.Nm, c);
+        gy[u] = cic_interp<DEP>(F1, pp.Nm, c);
       }
-      gz[u] = cic_interp(Fz, pp.Nm, c);
+      gz[u] = cic_interp<DEP>(Fz, pp.Nm, c);
     }
   }
   pdl_go();
@@ -1265,8 +1283,9 @@ cudaError_t part_drift_deposit(const PartParams& pp, float* sx, float* sy, float
         pp, sx, sy, sz, vx, vy, vz, ax, ay, az, dpx, dpy, dpz, rho, dt, m, mix, g_dep_box);
     return cudaGetLastError();
   }
-  return launch_pdl(P <= (1 << 18) && m.nb == 1, k_drift_deposit, dim3(blocks_for(P), m.nb), NTP, 0, s, pp, sx, sy, sz, vx, vy, vz, ax, ay, az,
-                    dpx, dpy, dpz, rho, dt, P, m, mix);
+  const bool dep = P <= (1 << 18) && m.nb == 1;
+  return launch_pdl(dep, dep ? k_drift_deposit<true> : k_drift_deposit<false>, dim3(blocks_for(P), m.nb), NTP, 0, s,
+                    pp, sx, sy, sz, vx, vy, vz, ax, ay, az, dpx, dpy, dpz, rho, dt, P, m, mix);
 }
 
 cudaError_t part_gather_kick(const PartParams& pp, const float* sx, const float* sy,
@@ -1282,9 +1301,11 @@ cudaError_t part_gather_kick(const PartParams& pp, const float* sx, const float*
         pp, sx, sy, sz, vx, vy, vz, ax, ay, az, Ax, Ay, Az, F0, F1, Fz, dt, m, mix, g_gk_box);
     return cudaGetLastError();
   }
-  auto k = pairs ? k_gather_kick<true> : k_gather_kick<false>;
-  return launch_pdl(P <= (1 << 18) && m.nb == 1, k, dim3((unsigned)((P + NTP * PPT - 1) / (NTP * PPT)), m.nb), NTP, 0, s, pp, sx, sy, sz, vx, vy, vz,
-                    ax, ay, az, Ax, Ay, Az, F0, F1, Fz, dt, P, m, mix);
+  const bool dep = P <= (1 << 18) && m.nb == 1;
+  auto k = dep ? (pairs ? k_gather_kick<true, true> : k_gather_kick<false, true>)
+               : (pairs ? k_gather_kick<true, false> : k_gather_kick<false, false>);
+  return launch_pdl(dep, k, dim3((unsigned)((P + NTP * PPT - 1) / (NTP * PPT)), m.nb), NTP, 0, s, pp, sx, sy, sz, vx,
+                    vy, vz, ax, ay, az, Ax, Ay, Az, F0, F1, Fz, dt, P, m, mix);
 }
 
 cudaError_t split_pairs(const float2* fxy, float* x, float* y, int64_t n, cudaStream_t s) {
@@ -1303,10 +1324,14 @@ cudaError_t part_kick_drift_deposit(const PartParams& pp, float* sx, float* sy, 
   // two particles per thread at four CTAs per SM (64 registers); measured on the 512^3 / 1024^3
   // run (ms per launch): 8.9 against 9.5 at 76 registers, 10.4 at 119, 9.4 with one particle
   constexpr int Q = 2;
-  auto k = mix.on ? (pairs ? k_kick_drift_deposit<Q, 4, true, true> : k_kick_drift_deposit<Q, 4, false, true>)
-                  : (pairs ? k_kick_drift_deposit<Q, 4, true, false> : k_kick_drift_deposit<Q, 4, false, false>);
-  return launch_pdl(P <= (1 << 18) && m.nb == 1, k, dim3((unsigned)((P + NTP * Q - 1) / (NTP * Q)), m.nb), NTP, 0, s, pp, sx, sy, sz, vx, vy, vz, Ax,
-                    Ay, Az, dpx, dpy, dpz, F0, F1, Fz, rho, hdr, P, m, mix);
+  auto launch = [&](auto dep) {
+    constexpr bool D = decltype(dep)::value;
+    auto k = mix.on ? (pairs ? k_kick_drift_deposit<Q, 4, true, true, D> : k_kick_drift_deposit<Q, 4, false, true, D>)
+                    : (pairs ? k_kick_drift_deposit<Q, 4, true, false, D> : k_kick_drift_deposit<Q, 4, false, false, D>);
+    return launch_pdl(D, k, dim3((unsigned)((P + NTP * Q - 1) / (NTP * Q)), m.nb), NTP, 0, s, pp, sx, sy, sz, vx, vy,
+                      vz, Ax, Ay, Az, dpx, dpy, dpz, F0, F1, Fz, rho, hdr, P, m, mix);
+  };
+  return P <= (1 << 18) && m.nb == 1 ? launch(std::true_type{}) : launch(std::false_type{});
 }
 
 cudaError_t part_snapshot(const PartParams& pp, const float* sx, const float* sy, const float* sz,

@@ -18,7 +18,7 @@ from workloads import LCDM_MODEL, Run
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("N", [128, 256, 512])
+@pytest.mark.parametrize("N", [32, 64, 128, 256, 512])
 def test_y_derivative_products_are_rounded_once(N):
     import paper_1703_00879_gb300 as pkg
     run = Run(Np=N, Nmesh=N, Lbox=1.7 * N, nsteps=4, model=LCDM_MODEL)
