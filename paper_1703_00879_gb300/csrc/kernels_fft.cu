@@ -1262,7 +1262,9 @@ __global__ void __launch_bounds__(NT, 1) k_lpt_z8(ColGeo<N, 8> geo, const void* 
 // Against two- and four-array tiles of 256 threads (k_lpt_z, k_lpt_z8): 142 -> 104 us at
 // 256^3, 718 -> 488 us over 256 lattices of 64^3.  A launch of few tiles (one lattice of 64^3
 // or 128^3) is bound by the length of one tile's chain instead and keeps k_lpt_z (10.5 and
-// 24.8 us against 11.1 and 26.8).
+// 24.8 us against 11.1 and 26.8).  Both forms give the same bits, so a lattice's fields
+// do not depend on how many others share its launch: a product that k_lpt_z leaves in shared
+// memory is rounded on its own here too (cmul_if).
 template <int N>
 struct LptZr {
   static constexpr int TW = ztw(N), T = 128, BUF = fft_rows<N>() * TW;
@@ -1344,7 +1346,7 @@ __global__ void __launch_bounds__(128, 4) k_lpt_zr(ColGeo<N, LptZr<N>::TW> geo, 
           for (int n1 = 0; n1 < R1; ++n1) {
             const int n = R2 * n1 + n2;
             const float kz = (n == N / 2) ? 0.f : lp.kf * (float)freq_index(n, N);
-            v[pos_of<R1>(n1)] = deriv ? cscale(cmul_i(src[i][n1]), kz) : src[i][n1];
+            v[pos_of<R1>(n1)] = deriv ? cmul_if(src[i][n1], kz) : src[i][n1];
           }
           dftR<R1, true>(v);
           float2* y = X + n2 * (R1 + 1) * TW + c;
