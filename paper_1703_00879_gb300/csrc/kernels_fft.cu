@@ -139,16 +139,22 @@ struct KernelInfo {
 std::mutex g_kinfo_mu;
 std::vector<KernelInfo> g_kinfo;
 
-// Sets the shared-memory limit of a kernel once and caches its resident CTAs per SM.
+// Raises the shared-memory limit of a kernel where a launch needs more than those before, and
+// caches its resident CTAs per SM for each size.  The limit is never lowered: launches of
+// every size seen so far rely on it.
 template <class K>
 cudaError_t resident_ctas(K kernel, size_t smem, int& per_sm, int threads) {
   std::lock_guard<std::mutex> lk(g_kinfo_mu);
+  size_t limit = 48 * 1024;
   for (const KernelInfo& k : g_kinfo)
-    if (k.fn == (const void*)kernel && k.smem == smem) {
-      per_sm = k.per_sm;
-      return cudaSuccess;
+    if (k.fn == (const void*)kernel) {
+      if (k.smem == smem) {
+        per_sm = k.per_sm;
+        return cudaSuccess;
+      }
+      limit = std::max(limit, k.smem);
     }
-  if (smem > 48 * 1024) {
+  if (smem > limit) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
