@@ -139,6 +139,17 @@ struct KernelInfo {
 std::mutex g_kinfo_mu;
 std::vector<KernelInfo> g_kinfo;
 
+// Largest dynamic shared memory a CTA may be given on this device.
+size_t smem_most() {
+  static const size_t most = [] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return n > 0 ? (size_t)n : (size_t)48 * 1024;
+  }();
+  return most;
+}
+
 // Raises the shared-memory limit of a kernel where a launch needs more than those before, and
 // caches its resident CTAs per SM for each size.  The limit is never lowered: launches of
 // every size seen so far rely on it.
@@ -2651,15 +2662,17 @@ static cudaError_t launch_lpt_t(const void* p1, const void* p2, float2* o0, floa
                                 cudaStream_t s, Multi m, float* zero_dst, int64_t zero_floats,
                                 bool* zeroed) {
   constexpr int TW = col_tw(N, 4);
-  // one simulation at N >= 512 (one CTA per SM either way): the table row also
-  // goes to shared memory
-  const int tab_smem = (N >= 512 && !m.shift) ? 1 : 0;
   // the zero fill rides along where the pass runs one CTA per SM (N >= 512: room for the
   // 16 KB zero region) on 16-byte aligned memory
   const bool zf = zero_dst && zero_floats > 0 && N >= 512 && (zero_floats % 4) == 0 &&
                   (reinterpret_cast<uintptr_t>(zero_dst) & 15) == 0;
   using Op = OpLptZ<N, TW, PREC>;
-  const size_t sm = col_smem<N, 4>() + (tab_smem ? (size_t)lp.nk * sizeof(float4) : 0) + (zf ? Op::kZero : 0);
+  // one simulation at N >= 512 (one CTA per SM either way): the table row also goes to shared
+  // memory if it fits there (about 4500 nodes); a longer one is read from global memory
+  size_t sm = col_smem<N, 4>() + (zf ? Op::kZero : 0);
+  const size_t row = (size_t)lp.nk * sizeof(float4);
+  const int tab_smem = N >= 512 && !m.shift && sm + row <= smem_most() ? 1 : 0;
+  if (tab_smem) sm += row;
   const int64_t ntiles = col_tiles<N, TW>() * m.nb;
   auto k = k_lpt_z<N, TW, PREC>;
   unsigned grid;
