@@ -124,26 +124,34 @@ __device__ __forceinline__ void resolve(ForceParams& fp, int64_t by) {
 }
 
 
-// Programmatic dependent launches.  The kernels of a step up to 128 points follow one
-// another at a few microseconds each, a good part of it the launch latency between
-// dependent kernels; launched with launch_pdl, a kernel's CTAs become resident while the one
-// before drains and load their twiddles meanwhile.  Such a kernel calls pdl_wait() before it
-// touches anything an earlier kernel writes (twiddle tables are never written by one): it
-// returns once every earlier kernel of the stream has completed and its writes are
-// visible.  pdl_go() lets the next kernel of the stream become resident once every CTA has
-// called it (or ended): it is called when a CTA's input has landed or its last tile begins,
-// not earlier, since waiting CTAs take shared memory and L1 from the running ones.  Both do
-// nothing in a kernel launched the ordinary way.
+// Programmatic dependent launches.  The kernels of a small step follow one another at a few
+// microseconds each, a good part of it the launch latency between dependent kernels; launched
+// with launch_pdl(true, ...), a kernel's CTAs become resident while the one before drains and
+// load their twiddles meanwhile.  Such a kernel calls pdl_wait() before it touches anything an
+// earlier kernel writes (twiddle tables are never written by one): it returns once every
+// earlier kernel of the stream has completed and its writes are visible.  pdl_go() lets the
+// next kernel of the stream, if that is launched dependently, become resident once every CTA
+// has called it (or ended): it is called when a CTA's input has landed or its last tile
+// begins, not earlier, since waiting CTAs take shared memory and L1 from the running ones.
+// In a kernel launched the ordinary way pdl_wait() does nothing; pdl_go() has its effect there
+// too, on the step counter after a particle pass of any size.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-//
-// `small` (one simulation on lattices up to 64^3 and meshes up to 128^3, whose kernels run 3 to
-// 25 us) selects it: the whole 32^3 f(R) run of ten steps 513 -> 315 us, eight steps at 64^3 /
-// 128^3 1036 -> 1000 us.  Larger launches are launched the ordinary way: a 256-member batch pass
-// measured 64.9 ms that way and 66.6 ms with it, 512^3 / 1024^3 139.4 and 140.1 ms.
+// Which launches of one simulation are dependent: each kernel by the side of the arrays it works on,
+// transform passes and plane passes up to 128 points, particle passes up to 64^3 particles; the
+// step counter always.  Ten steps of the 32^3 f(R) run 513 -> 309 us, eight steps at 64^3 / 128^3
+// 1036 -> 1005 us.  Lattice and mesh of different sizes, us per nDGP step, so / only where
+// both are small: 128^3 / 128^3 197 / 205, 128^3 / 256^3 534 / 539, 32^3 / 256^3 402 / 408, 256^3 /
+// 128^3 1113 / 1117.  Beyond these sizes, and over several simulations, the waiting CTAs cost
+// more than they hide: a 256-member batch pass 64.9 ms without and 66.6 with them, 512^3 / 1024^3
+// 139.4 and 140.1.  The step counter of a large run hides its launch behind the particle pass: five
+// steps at 256^3 on the scale-independent path 5.00 ms so and 5.08 without pdl_go there.
+constexpr int kDepTransform = 128, kDepParticles = 64;
+inline bool dependent_launch(const Multi& m, int side, int most) { return m.nb == 1 && side <= most; }
+
 template <class... P, class... A>
-cudaError_t launch_pdl(bool small, void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... a) {
+cudaError_t launch_pdl(bool dep, void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... a) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
@@ -153,7 +161,7 @@ cudaError_t launch_pdl(bool small, void (*k)(P...), dim3 grid, unsigned threads,
   c.dynamicSmemBytes = smem;
   c.stream = s;
   c.attrs = &at;
-  c.numAttrs = small ? 1 : 0;
+  c.numAttrs = dep ? 1 : 0;
   return cudaLaunchKernelEx(&c, k, P(a)...);
 }
 

@@ -2387,7 +2387,7 @@ static cudaError_t launch_xc2r_pair(const float2* a, const float2* b, float* xy,
     return cudaErrorInvalidValue;
   } else {
     constexpr RowShape SH = pair_shape(N);
-  constexpr int TWX = SH.rows, T = SH.threads;
+    constexpr int TWX = SH.rows, T = SH.threads;
     const size_t sm = RowCfg<N, TWX>::smem;
     const int64_t tps = (int64_t)N * N / (TWX / 2);
     auto k = k_xc2r_pair<N, TWX, T, SH.ctas>;
@@ -2569,8 +2569,8 @@ static cudaError_t launch_zsf(const float2* in, float2* dk_out, float2* w_out,
     unsigned grid;
     cudaError_t e = prep(k, smk, ntiles, grid, T);
     if (e != cudaSuccess) return e;
-    return launch_pdl(N <= 128 && m.nb == 1, k, dim3(grid), T, smk, s, OpZScreenField<N, TW, MODEL, T>{geo_z<N, TW>(m), in, dk_out, w_out, fp}, tw, ntiles,
-                            map);
+    return launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(grid), T, smk, s,
+                      OpZScreenField<N, TW, MODEL, T>{geo_z<N, TW>(m), in, dk_out, w_out, fp}, tw, ntiles, map);
   };
   auto pick = [&](auto tma_c) {
     if (fp.model == 1) return go(std::integral_constant<int, 1>{}, tma_c);
@@ -2637,8 +2637,8 @@ static cudaError_t launch_zforce_t(const float2* in, const float2* dk, float2* p
     unsigned grid;
     cudaError_t e = prep(k, smk, ntiles, grid, T);
     if (e != cudaSuccess) return e;
-    return launch_pdl(N <= 128 && m.nb == 1, k, dim3(grid), T, smk, s, OpZForce<N, TW, SCR, T>{geo_z<N, TW>(m), in, dk, phi, phiz, fp}, tw, ntiles, map,
-                            dmap);
+    return launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(grid), T, smk, s,
+                      OpZForce<N, TW, SCR, T>{geo_z<N, TW>(m), in, dk, phi, phiz, fp}, tw, ntiles, map, dmap);
   };
   if constexpr (tma_shape<N, TW>()) {
     if (tma) return go(std::true_type{});
@@ -2685,7 +2685,7 @@ static cudaError_t launch_lpt_t(const void* p1, const void* p2, float2* o0, floa
     const int64_t tps = col_tiles<N, TW>();
     op.zchunk = ((op.zbytes + tps - 1) / tps + 15) / 16 * 16;
   }
-  e = launch_pdl(N <= 128 && m.nb == 1, k, dim3(grid), NT, sm, s, op, tw, ntiles);
+  e = launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(grid), NT, sm, s, op, tw, ntiles);
   if (e == cudaSuccess && zeroed) *zeroed = zf;
   return e;
 }
@@ -2712,8 +2712,8 @@ static cudaError_t launch_lptr(const void* p1, const void* p2, float2* o0, float
   unsigned grid;
   cudaError_t e = prep(k, sm, ntiles, grid, T);
   if (e != cudaSuccess) return e;
-  return launch_pdl(N <= 128 && m.nb == 1, k, dim3(grid), T, sm, s, geo_z<N, TW>(m), static_cast<const float2*>(p1), static_cast<const float2*>(p2), o0, o1, o2, o3,
-                        lp, tw, ntiles);
+  return launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(grid), T, sm, s, geo_z<N, TW>(m),
+                    static_cast<const float2*>(p1), static_cast<const float2*>(p2), o0, o1, o2, o3, lp, tw, ntiles);
 }
 template <int N>
 static cudaError_t launch_lpt(const void* p1, const void* p2, float2* o0, float2* o1, float2* o2,
@@ -2757,7 +2757,7 @@ static cudaError_t launch_plane_r2c(const float* in, float2* out, float scale, f
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
-    return launch_pdl(N <= 128 && m.nb == 1, k, dim3(N, m.nb), NT, sm, s, in, out, scale, offset, tw, m);
+    return launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(N, m.nb), NT, sm, s, in, out, scale, offset, tw, m);
   }
 }
 
@@ -2778,7 +2778,7 @@ static cudaError_t launch_plane_grad(const PlaneJobs& jobs, const float2* tw, cu
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
-    return launch_pdl(N <= 128 && m.nb == 1, k, dim3(jobs.n * N, m.nb), NT, sm, s, jobs, tw, m);
+    return launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(jobs.n * N, m.nb), NT, sm, s, jobs, tw, m);
   }
 }
 
@@ -2828,7 +2828,7 @@ static cudaError_t launch_plane_screen(const float2* w_in, const float* rho, flo
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
-    return launch_pdl(N <= 128 && m.nb == 1, k, dim3(N, m.nb), NT, sm, s, w_in, rho, s_out, fp, tw, m);
+    return launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(N, m.nb), NT, sm, s, w_in, rho, s_out, fp, tw, m);
   }
 }
 
