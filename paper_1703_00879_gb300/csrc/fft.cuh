@@ -239,8 +239,7 @@ __host__ __device__ constexpr int fft_rows() {
 // Hooks (defaults: the tile itself): step 1 reads element n of column c as
 // ld(buf, n, c, at) and step 2 writes X[n] as st(X[n], n, c, at), at = n PITCH
 // + c, so a k-space operation fuses into the first load or the last store
-// (reading or writing another array at the same offset); st.ready() runs in
-// every thread before the barrier between the steps.  A store hook with
+// (reading or writing another array at the same offset).  A store hook with
 // kSmem = false writes the outputs itself (e.g. straight to HBM) and the tile
 // is left holding the intermediate.
 struct TileLoad {
@@ -249,7 +248,6 @@ struct TileLoad {
 struct TileStore {
   static constexpr bool kSmem = true;
   __device__ __forceinline__ float2 operator()(float2 v, int, int, int) const { return v; }
-  __device__ __forceinline__ void ready() const {}
 };
 
 template <int L, int TW, int PITCH, int NT, bool INV, int TWS = 1, class Load = TileLoad,
@@ -294,7 +292,6 @@ __device__ __forceinline__ void fft_tile(float2* __restrict__ buf, const float2*
       }
     }
   }
-  st.ready();
   __syncthreads();
   {
     float2 y[P2][R2];
@@ -447,8 +444,7 @@ __device__ __forceinline__ void col_inv2(const float2* __restrict__ buf, Store s
 }
 
 // Forward transform of the tile's TW columns, x = mid(X[n], n, c, at) on every value,
-// inverse transform of x to st.  mid.ready() runs in every thread before the barrier
-// ahead of mid.  The caller synchronises before the call and before it reuses the tile.
+// inverse transform of x to st.  The caller synchronises before the call and before it reuses the tile.
 template <int L, int TW, int PITCH, int NT, class Mid, class Store>
 __device__ __forceinline__ void fft_tile_fwd_inv(float2* __restrict__ buf, const float2* __restrict__ tw, Mid mid,
                                                  Store st) {
@@ -456,7 +452,6 @@ __device__ __forceinline__ void fft_tile_fwd_inv(float2* __restrict__ buf, const
   constexpr int U = TW * R1, P = (U + NT - 1) / NT;
   static_assert(PITCH % 4 == 0, "column tiles: row pitch a multiple of 4");
   col_step1<R1, R2, TW, PITCH, NT, false>(buf, tw, TileLoad{});
-  mid.ready();
   __syncthreads();
   float2 v[P][R2];
 #pragma unroll
@@ -482,8 +477,8 @@ __device__ __forceinline__ void fft_tile_fwd_inv(float2* __restrict__ buf, const
 }
 
 // The same with two inverse transforms, of x = mid(X) to st and of grad(x, n) to st2, one
-// after the other; x stays in registers in between.  after() runs in every thread once
-// all of mid's reads are done.
+// after the other; x stays in registers in between.  mid.ready() runs in every thread before
+// the barrier ahead of mid, after() once all of mid's reads are done.
 template <int L, int TW, int PITCH, int NT, class Mid, class Grad, class After, class Store>
 __device__ __forceinline__ void fft_tile_fwd_inv2(float2* __restrict__ buf, const float2* __restrict__ tw, Mid mid,
                                                   Grad grad, After after, Store st, Store st2) {
@@ -605,8 +600,7 @@ struct NoPre {
 // 1.17 -> 1.01.
 // Each warp owns TW 32 / NT consecutive rows (RowMap), so the steps are ordered by
 // warp barriers alone and the warps of a CTA drift apart: while one computes another
-// loads.  PAIR32: for L = 16 x 32 with one row per warp, step 2 runs on lane pairs
-// (dft32_pair).  The caller makes the warp's rows visible to it before the call and
+// loads.  The caller makes the warp's rows visible to it before the call and
 // synchronises the warp before it reuses them.
 // Store hook of fft_rowtile's last step: output k of row c as st(X[k], c, k);
 // with kSmem = false the hook writes the output itself and the tile keeps the
@@ -672,52 +666,36 @@ __device__ __forceinline__ void row_step1(float2* __restrict__ buf, const float2
   __syncwarp();
 }
 
-// Lane pairs for the radix-32 step of L = 16 x 32 rows: one row per warp.
+// PAIR32 (the forward and the chained row transforms): for L = 16 x 32 with one row per warp the
+// radix-32 step runs on lane pairs (dft32_pair).
 template <int L, int TW, int NT, bool PAIR32>
 __host__ __device__ constexpr bool row_pairs() {
   return PAIR32 && Split<L>::R1 == 16 && Split<L>::R2 == 32 && TW * 32 == NT;
 }
 
-template <int L, int TW, int CW, int NT, bool INV, class Pre = NoPre, bool PAIR32 = false,
-          class Store = RowStore>
+template <int L, int TW, int CW, int NT, bool INV, class Pre = NoPre, class Store = RowStore>
 __device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const float2* __restrict__ w1,
                                             Pre pre = Pre(), Store st = Store()) {
   constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;
   row_step1<L, TW, CW, NT, INV, Pre>(buf, w1, pre);
-  if constexpr (row_pairs<L, TW, NT, PAIR32>()) {
-    const int lane = threadIdx.x & 31, half = lane >> 4, c = threadIdx.x >> 5, k1 = lane & 15;
-    float2 y[16];
-    const float2* yr = buf + c * CW + k1 + 16 * half * (R1 + 1);
+  using Map = RowMap<TW, NT, R1>;
+  const Map mp;
+  float2 y[Map::P][R2];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) y[j] = yr[j * (R1 + 1)];
-    dft32_pair<INV>(y, half);
-    if constexpr (Store::kSmem) __syncwarp();
+  for (int i = 0; i < Map::P; ++i) {
+    const float2* yr = buf + mp.c(i) * CW + mp.q(i);
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const int n = k1 + R1 * (2 * k + half);
-      const float2 o = st(y[k], c, n);
-      if constexpr (Store::kSmem) buf[c * CW + n] = o;
-    }
-  } else {
-    using Map = RowMap<TW, NT, R1>;
-    const Map mp;
-    float2 y[Map::P][R2];
+    for (int n2 = 0; n2 < R2; ++n2) y[i][pos_of<R2>(n2)] = yr[n2 * (R1 + 1)];
+    dftR<R2, INV>(y[i]);
+  }
+  if constexpr (Store::kSmem) __syncwarp();
 #pragma unroll
-    for (int i = 0; i < Map::P; ++i) {
-      const float2* yr = buf + mp.c(i) * CW + mp.q(i);
+  for (int i = 0; i < Map::P; ++i) {
+    const int c = mp.c(i), k1 = mp.q(i);
 #pragma unroll
-      for (int n2 = 0; n2 < R2; ++n2) y[i][pos_of<R2>(n2)] = yr[n2 * (R1 + 1)];
-      dftR<R2, INV>(y[i]);
-    }
-    if constexpr (Store::kSmem) __syncwarp();
-#pragma unroll
-    for (int i = 0; i < Map::P; ++i) {
-      const int c = mp.c(i), k1 = mp.q(i);
-#pragma unroll
-      for (int k2 = 0; k2 < R2; ++k2) {
-        const float2 o = st(y[i][k2], c, k1 + R1 * k2);
-        if constexpr (Store::kSmem) buf[c * CW + k1 + R1 * k2] = o;
-      }
+    for (int k2 = 0; k2 < R2; ++k2) {
+      const float2 o = st(y[i][k2], c, k1 + R1 * k2);
+      if constexpr (Store::kSmem) buf[c * CW + k1 + R1 * k2] = o;
     }
   }
 }
@@ -733,7 +711,7 @@ __device__ __forceinline__ void fft_rowtile(float2* __restrict__ buf, const floa
 // there costs 8 shared-memory wavefronts per point and warp, this 3 (two
 // shuffles, one broadcast twiddle read), and one barrier less: x r2c 1.61 ->
 // 1.30 ms and screening x 3.45 -> 3.14 ms at 1024^3, x r2c plane pass 1.21 ->
-// 1.06 ms over 256 meshes of 128^3.  PAIR32 as in fft_rowtile.
+// 1.06 ms over 256 meshes of 128^3.
 template <int L, int TW, int CW, int NT, bool PAIR32, class Store>
 __device__ __forceinline__ void row_r2c_step2(float2* __restrict__ buf, const float2* __restrict__ twr, Store st) {
   constexpr int R1 = Split<L>::R1, R2 = Split<L>::R2;

@@ -326,7 +326,6 @@ struct ColOut {
     if (c < live) g[(n / HQ) * ra + (n % HQ) * rb + hcol(c)] = v;
     return v;
   }
-  __device__ __forceinline__ void ready() const {}
 };
 
 // Column geometry: tile t -> (simulation b, outer index o, column block c0);
@@ -652,7 +651,6 @@ struct DenseOut {
     if (c < live) g[n * (N / 2 + 1) + c] = v;
     return v;
   }
-  __device__ __forceinline__ void ready() const {}
 };
 template <int N, int TW, int T>
 __device__ __forceinline__ void col_issue_dense(float2* buf, const float2* __restrict__ g, int live) {
@@ -871,7 +869,6 @@ struct OpZScreenField {
       }
       return cscale(v, m);
     }
-    __device__ __forceinline__ void ready() const {}
   };
   ColGeo<N, TW> geo;
   const float2* in;
@@ -1134,17 +1131,15 @@ __global__ void __launch_bounds__(NT, blocks_for_smem(col_smem_c(N, 4), N)) k_lp
   if (op.zdst && threadIdx.x == 0) bulk_store_drain();  // the zero fill completes with the kernel
 }
 
-// The LPT z pass with 8-column tiles (N = 256, 512), where four 4-column
+// The LPT z pass for 16-bit seeds with 8-column tiles (N = 256, 512), where four 4-column
 // output arrays would otherwise fill shared memory: an 8-column tile reads and
-// writes whole 64-byte chunks of the interleaved layout (4-column
-// tiles move 32-byte halves of them).  Shared memory: two input buffers
-// (phi1 in columns 0..7, phi2 in 8..15; double-buffered) and one work buffer
-// that first holds (d, i kz d) and then (A, i kz A), each pair inverse
+// writes whole chunks of the interleaved layout (4-column tiles move halves of
+// them).  Shared memory: two input buffers of raw seeds (phi1 words 0..7, phi2 words
+// 8..15 of each 32-word row; double-buffered) and one work buffer that first holds
+// (d, i kz d) and then (A, i kz A), formed from the dequantised seeds, each pair inverse
 // transformed as one 16-column tile whose outputs leave for HBM from the last
-// step's registers.  The table row is read through L1.  16-bit seeds are
-// staged raw (phi1 words 0..7, phi2 words 8..15 of each 32-word row) and
-// dequantised as the work pairs are formed.
-template <int N, int PREC>
+// step's registers.  The table row is read through L1.
+template <int N>
 struct LptZ8 {
   static constexpr int TW = 8, TP = 16, ROWS = fft_rows<N>(), BUF = ROWS * TP;
   static constexpr size_t smem = (N + 3 * (size_t)BUF) * sizeof(float2);
@@ -1162,7 +1157,6 @@ struct PairColOut {
     if (cc < live) (b ? gb : ga)[(n / HQ) * ra + (n % HQ) * rb + hcol(cc)] = v;
     return v;
   }
-  __device__ __forceinline__ void ready() const {}
 };
 
 // 16-bit seeds of one field, raw, into words f*8 .. f*8+7 of each 32-word staged row.
@@ -1183,12 +1177,13 @@ __device__ __forceinline__ void col_issue_raw8(uint32_t* sb, int f, const uint32
 }
 
 template <int N, int PREC>
-__global__ void __launch_bounds__(NT, 1) k_lpt_z8(ColGeo<N, 8> geo, const void* __restrict__ phi1,
-                                                   const void* __restrict__ phi2, float2* __restrict__ o0,
+__global__ void __launch_bounds__(NT, 1) k_lpt_z8(ColGeo<N, 8> geo, const uint32_t* __restrict__ phi1,
+                                                   const uint32_t* __restrict__ phi2, float2* __restrict__ o0,
                                                    float2* __restrict__ o1, float2* __restrict__ o2,
                                                    float2* __restrict__ o3, LptParams lp0,
                                                    const float2* __restrict__ twg, int64_t ntiles) {
-  using C = LptZ8<N, PREC>;
+  static_assert(PREC == 1 || PREC == 2, "16-bit seeds");
+  using C = LptZ8<N>;
   extern __shared__ __align__(128) float2 sm[];
   float2* tw = sm;
   float2* const S0 = sm + N;
@@ -1199,14 +1194,9 @@ __global__ void __launch_bounds__(NT, 1) k_lpt_z8(ColGeo<N, 8> geo, const void* 
     int o, c0;
     int64_t base, by;
     geo.tile(t, o, c0, base, by);
-    if constexpr (PREC == 0) {
-      col_issue<N, 8, 16>(buf, 0, moved(static_cast<const float2*>(phi1), by), base, geo.ra, geo.rb, c0);
-      col_issue<N, 8, 16>(buf, 1, moved(static_cast<const float2*>(phi2), by), base, geo.ra, geo.rb, c0);
-    } else {
-      uint32_t* sb = reinterpret_cast<uint32_t*>(buf);
-      col_issue_raw8<N>(sb, 0, moved(static_cast<const uint32_t*>(phi1), by), base, geo.ra, geo.rb, c0);
-      col_issue_raw8<N>(sb, 1, moved(static_cast<const uint32_t*>(phi2), by), base, geo.ra, geo.rb, c0);
-    }
+    uint32_t* sb = reinterpret_cast<uint32_t*>(buf);
+    col_issue_raw8<N>(sb, 0, moved(phi1, by), base, geo.ra, geo.rb, c0);
+    col_issue_raw8<N>(sb, 1, moved(phi2, by), base, geo.ra, geo.rb, c0);
   };
   if (!geo.m.shift) resolve(lp0, 0);  // one simulation: once per launch
   int64_t t = blockIdx.x;
@@ -1225,7 +1215,7 @@ __global__ void __launch_bounds__(NT, 1) k_lpt_z8(ColGeo<N, 8> geo, const void* 
     LptParams lp = lp0;
     resolve(lp, by);
     const float4* __restrict__ tab = lp.row;
-    const float2* sb = cur ? S1 : S0;
+    const uint32_t* sb = reinterpret_cast<const uint32_t*>(cur ? S1 : S0);
     const TileLane<N, 8> ln(c0, iy);
     const float kf2 = lp.kf * lp.kf;
     const int c = ln.c;
@@ -1245,15 +1235,8 @@ __global__ void __launch_bounds__(NT, 1) k_lpt_z8(ColGeo<N, 8> geo, const void* 
           const float4 t0 = __ldg(tab + i0), t1 = __ldg(tab + i0 + 1);
           const float a = pass == 0 ? t0.x * (1.f - f) + t1.x * f : t0.z * (1.f - f) + t1.z * f;
           const float b = pass == 0 ? t0.y * (1.f - f) + t1.y * f : t0.w * (1.f - f) + t1.w * f;
-          float2 p1, p2;
-          if constexpr (PREC == 0) {
-            p1 = sb[n * 16 + c];
-            p2 = sb[n * 16 + 8 + c];
-          } else {
-            const uint32_t* rb = reinterpret_cast<const uint32_t*>(sb);
-            p1 = dequant<PREC>(rb[n * 32 + c], lp.scale[0]);
-            p2 = dequant<PREC>(rb[n * 32 + 8 + c], lp.scale[1]);
-          }
+          const float2 p1 = dequant<PREC>(sb[n * 32 + c], lp.scale[0]);
+          const float2 p2 = dequant<PREC>(sb[n * 32 + 8 + c], lp.scale[1]);
           v = cscale(cadd(cscale(p1, a), cscale(p2, b)), lp.norm);
         }
         const float kz = (n == N / 2) ? 0.f : lp.kf * (float)freq_index(n, N);
@@ -1276,7 +1259,7 @@ __global__ void __launch_bounds__(NT, 1) k_lpt_z8(ColGeo<N, 8> geo, const void* 
 // registers; the four outputs d, i kz d, A, i kz A are then transformed one after the other
 // through one tile buffer.  Three buffers rotate: the two seed tiles, whose room is free once
 // they are in registers, and one more, so that the next tile's seeds land meanwhile.
-// Against two- and four-array tiles of 256 threads (k_lpt_z, k_lpt_z8): 142 -> 104 us at
+// Against two- and four-array tiles of 256 threads: 142 -> 104 us at
 // 256^3, 718 -> 488 us over 256 lattices of 64^3.  A launch of few tiles (one lattice of 64^3
 // or 128^3) is bound by the length of one tile's chain instead and keeps k_lpt_z (10.5 and
 // 24.8 us against 11.1 and 26.8).  Both forms give the same bits, so a lattice's fields
@@ -1818,7 +1801,7 @@ __global__ void __launch_bounds__(T, CTAS) k_xc2r(const __grid_constant__ RowJob
     if constexpr (OUT == 0) {
       float* out = moved(static_cast<float*>(jobs.out[j.job]), j.by);
       const RealRowOut<M> o{reinterpret_cast<float2*>(out + real_row_q(j.row0, N) * N)};
-      fft_rowtile<M, TWX, C::CW, T, true, Pre, false, RealRowOut<M>>(buf, tw + M, pre, o);
+      fft_rowtile<M, TWX, C::CW, T, true, Pre, RealRowOut<M>>(buf, tw + M, pre, o);
     } else {
       const SimHeader* h = moved(jobs.hdr, j.by);
       if (j.q != run_q) {  // the same for every thread of the CTA
@@ -1832,7 +1815,7 @@ __global__ void __launch_bounds__(T, CTAS) k_xc2r(const __grid_constant__ RowJob
       float tile_max = 0.f;
       const RealRowOut16<M, OUT> o{out + real_row_q(j.row0, N) * M,
                                    1.f / h->lq_scale[j.job], &tile_max};
-      fft_rowtile<M, TWX, C::CW, T, true, Pre, false, RealRowOut16<M, OUT>>(buf, tw + M, pre, o);
+      fft_rowtile<M, TWX, C::CW, T, true, Pre, RealRowOut16<M, OUT>>(buf, tw + M, pre, o);
       run_max = fmaxf(run_max, tile_max);
     }
     cur ^= 1;
@@ -1917,7 +1900,7 @@ __global__ void __launch_bounds__(T, CTAS) k_xc2r_pair(
     float2* buf = cur ? st1 : st0;
     float2* o = moved(out, by);
     const PairRowOut<N, R1> st{o + real_row_q(q0, N) * N};
-    fft_rowtile<M, TWX, C::CW, T, true, C2rCombine2<N, C::CW>, false, PairRowOut<N, R1>>(
+    fft_rowtile<M, TWX, C::CW, T, true, C2rCombine2<N, C::CW>, PairRowOut<N, R1>>(
         buf, tw + M, C2rCombine2<N, C::CW>{buf, tw, kfs, 0.f}, st);
     cur ^= 1;
   }
@@ -2159,7 +2142,6 @@ struct PlaneUnpack {
     buf[at + N / 2] = make_float2(v.y, 0.f);
     return make_float2(v.x, 0.f);
   }
-  __device__ __forceinline__ void ready() const {}
 };
 
 // y inverse of every column of plane a, in place (DY: of i kfs f_y times them).
@@ -2169,6 +2151,9 @@ struct PlaneUnpack {
 // and screening spectra are such; caller-given potentials (the LPT planes) need not be.
 // Force plane pass 3.41 -> 2.99 ms, screening plane pass 863 -> 838 us over 256 meshes of
 // 128^3 (the derivative on load instead of in a pass of its own also in the LPT planes, 957 -> 908).
+// Where |X_M| is far below |X_0| (a potential: by about M^2) the joined column's rounding is
+// relative to X_0, so column M's own relative error grows by their ratio.  The field's does not: its
+// x transform adds the two columns in its first step, with a rounding of that size.
 template <int N, bool HERM, bool DY>
 __device__ __forceinline__ void plane_yinv(float2* a, const float2* tw, float kfs) {
   using C = PlaneCfg<N>;
@@ -2191,7 +2176,7 @@ __device__ __forceinline__ void plane_yinv(float2* a, const float2* tw, float kf
 template <int N>
 __device__ __forceinline__ void plane_xc2r(float2* a, const float2* tw, float kfs, float* g) {
   using C = PlaneCfg<N>;
-  fft_rowtile<C::M, N, C::CW, NT, true, C2rCombine<N, C::CW>, false, PlaneRowOut<C::M>>(
+  fft_rowtile<C::M, N, C::CW, NT, true, C2rCombine<N, C::CW>, PlaneRowOut<C::M>>(
       a, tw + N, C2rCombine<N, C::CW>{a, tw, kfs}, PlaneRowOut<C::M>{reinterpret_cast<float2*>(g)});
 }
 
@@ -2693,13 +2678,14 @@ static cudaError_t launch_lpt_t(const void* p1, const void* p2, float2* o0, floa
 template <int N, int PREC>
 static cudaError_t launch_lpt8(const void* p1, const void* p2, float2* o0, float2* o1, float2* o2, float2* o3,
                                const LptParams& lp, const float2* tw, cudaStream_t s, Multi m) {
-  const size_t sm = LptZ8<N, PREC>::smem;
+  const size_t sm = LptZ8<N>::smem;
   const int64_t ntiles = col_tiles<N, 8>() * m.nb;
   auto k = k_lpt_z8<N, PREC>;
   unsigned grid;
   cudaError_t e = prep(k, sm, ntiles, grid);
   if (e != cudaSuccess) return e;
-  k<<<grid, NT, sm, s>>>(geo_z<N, 8>(m), p1, p2, o0, o1, o2, o3, lp, tw, ntiles);
+  k<<<grid, NT, sm, s>>>(geo_z<N, 8>(m), static_cast<const uint32_t*>(p1), static_cast<const uint32_t*>(p2), o0, o1,
+                         o2, o3, lp, tw, ntiles);
   return cudaGetLastError();
 }
 template <int N>
@@ -2719,8 +2705,8 @@ template <int N>
 static cudaError_t launch_lpt(const void* p1, const void* p2, float2* o0, float2* o1, float2* o2,
                               float2* o3, const LptParams& lp, const float2* tw,
                               cudaStream_t s, Multi m, float* zd, int64_t zn, bool* zeroed) {
-  // measured on GB300 (ms per launch, 4-column -> 8-column tiles): N = 256 FP32 0.154 -> 0.144,
-  // FP16 0.180 -> 0.143; N = 512 FP32 1.40 -> 1.46 (kept on 4 columns), FP16 1.55 -> 1.44
+  // 16-bit seeds, ms per launch with 4-column tiles (k_lpt_z) -> 8-column tiles: N = 256 0.180 ->
+  // 0.143, N = 512 1.55 -> 1.44 (FP32 seeds at 512 the other way, 1.40 -> 1.46)
   if constexpr (N == 256 || N == 512) {
     if (lp.seed_prec == 1) return launch_lpt8<N, 1>(p1, p2, o0, o1, o2, o3, lp, tw, s, m);
     if (lp.seed_prec == 2) return launch_lpt8<N, 2>(p1, p2, o0, o1, o2, o3, lp, tw, s, m);

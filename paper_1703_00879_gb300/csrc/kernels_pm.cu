@@ -410,9 +410,11 @@ __global__ void __launch_bounds__(NTP) k_gather_kick(
 // acc = g(x) - A_n(q) and delta_v += acc dtk2_n, then the closing half kick of
 // step n + 1, delta_v += acc dtk1_{n+1}, the drift s += delta_v dtd_{n+1} +
 // dPsi_{n+1}(q) and the CIC deposit of the new x.  The arithmetic and its order
-// are those of k_gather_kick followed by k_drift_deposit, so the particle state
-// is the same bit for bit; acc is not stored (the next gather forms it again)
-// and delta_v and s are read and written once instead of twice.  hdr->step = n.
+// are those of k_gather_kick followed by k_drift_deposit, so from the same force the
+// particle state is the same bit for bit (MIX: up to the rounding of the two-term
+// combinations, whose products the compiler may fuse differently); acc is not stored
+// (the next gather forms it again) and delta_v and s are read and written once instead
+// of twice.  hdr->step = n.
 // Particles as in the gather (16 x 2 lattice patches per warp, PPT per thread).
 // MIX (the scale-independent path): A and dp hold Psi1 (one set of arrays) and mix.q2
 // Psi2; A_n and dPsi_{n+1} are formed from them with rows 1 + n and 2 + n of the growth
