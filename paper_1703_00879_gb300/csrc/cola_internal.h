@@ -147,8 +147,18 @@ __device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_d
 // more than they hide: a 256-member batch pass 64.9 ms without and 66.6 with them, 512^3 / 1024^3
 // 139.4 and 140.1.  The step counter of a large run hides its launch behind the particle pass: five
 // steps at 256^3 on the scale-independent path 5.00 ms so and 5.08 without pdl_go there.
-constexpr int kDepTransform = 128, kDepParticles = 64;
-inline bool dependent_launch(const Multi& m, int side, int most) { return m.nb == 1 && side <= most; }
+//
+// In a CUDA graph the launch gaps are short, and only the shortest kernels gain: launches that are
+// being captured (a Batch whose runs are launched one by one) are dependent up to 32 points.
+// Twelve 64^3 / 128^3 runs on one chain, us for one step of each: 1238 before there were
+// dependent launches, 1418 with them, 1090 without; 24 runs of 32^3 / 32^3 782, 709, 748.
+constexpr int kDepTransform = 128, kDepParticles = 64, kDepCaptured = 32;
+inline bool dependent_launch(const Multi& m, int side, int most, cudaStream_t s) {
+  if (m.nb != 1 || side > most) return false;
+  if (side <= kDepCaptured) return true;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+}
 
 template <class... P, class... A>
 cudaError_t launch_pdl(bool dep, void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... a) {

@@ -2554,7 +2554,7 @@ static cudaError_t launch_zsf(const float2* in, float2* dk_out, float2* w_out,
     unsigned grid;
     cudaError_t e = prep(k, smk, ntiles, grid, T);
     if (e != cudaSuccess) return e;
-    return launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(grid), T, smk, s,
+    return launch_pdl(dependent_launch(m, N, kDepTransform, s), k, dim3(grid), T, smk, s,
                       OpZScreenField<N, TW, MODEL, T>{geo_z<N, TW>(m), in, dk_out, w_out, fp}, tw, ntiles, map);
   };
   auto pick = [&](auto tma_c) {
@@ -2622,7 +2622,7 @@ static cudaError_t launch_zforce_t(const float2* in, const float2* dk, float2* p
     unsigned grid;
     cudaError_t e = prep(k, smk, ntiles, grid, T);
     if (e != cudaSuccess) return e;
-    return launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(grid), T, smk, s,
+    return launch_pdl(dependent_launch(m, N, kDepTransform, s), k, dim3(grid), T, smk, s,
                       OpZForce<N, TW, SCR, T>{geo_z<N, TW>(m), in, dk, phi, phiz, fp}, tw, ntiles, map, dmap);
   };
   if constexpr (tma_shape<N, TW>()) {
@@ -2670,7 +2670,7 @@ static cudaError_t launch_lpt_t(const void* p1, const void* p2, float2* o0, floa
     const int64_t tps = col_tiles<N, TW>();
     op.zchunk = ((op.zbytes + tps - 1) / tps + 15) / 16 * 16;
   }
-  e = launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(grid), NT, sm, s, op, tw, ntiles);
+  e = launch_pdl(dependent_launch(m, N, kDepTransform, s), k, dim3(grid), NT, sm, s, op, tw, ntiles);
   if (e == cudaSuccess && zeroed) *zeroed = zf;
   return e;
 }
@@ -2698,7 +2698,7 @@ static cudaError_t launch_lptr(const void* p1, const void* p2, float2* o0, float
   unsigned grid;
   cudaError_t e = prep(k, sm, ntiles, grid, T);
   if (e != cudaSuccess) return e;
-  return launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(grid), T, sm, s, geo_z<N, TW>(m),
+  return launch_pdl(dependent_launch(m, N, kDepTransform, s), k, dim3(grid), T, sm, s, geo_z<N, TW>(m),
                     static_cast<const float2*>(p1), static_cast<const float2*>(p2), o0, o1, o2, o3, lp, tw, ntiles);
 }
 template <int N>
@@ -2743,7 +2743,7 @@ static cudaError_t launch_plane_r2c(const float* in, float2* out, float scale, f
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
-    return launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(N, m.nb), NT, sm, s, in, out, scale, offset, tw, m);
+    return launch_pdl(dependent_launch(m, N, kDepTransform, s), k, dim3(N, m.nb), NT, sm, s, in, out, scale, offset, tw, m);
   }
 }
 
@@ -2764,7 +2764,7 @@ static cudaError_t launch_plane_grad(const PlaneJobs& jobs, const float2* tw, cu
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
-    return launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(jobs.n * N, m.nb), NT, sm, s, jobs, tw, m);
+    return launch_pdl(dependent_launch(m, N, kDepTransform, s), k, dim3(jobs.n * N, m.nb), NT, sm, s, jobs, tw, m);
   }
 }
 
@@ -2814,7 +2814,7 @@ static cudaError_t launch_plane_screen(const float2* w_in, const float* rho, flo
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
-    return launch_pdl(dependent_launch(m, N, kDepTransform), k, dim3(N, m.nb), NT, sm, s, w_in, rho, s_out, fp, tw, m);
+    return launch_pdl(dependent_launch(m, N, kDepTransform, s), k, dim3(N, m.nb), NT, sm, s, w_in, rho, s_out, fp, tw, m);
   }
 }
 

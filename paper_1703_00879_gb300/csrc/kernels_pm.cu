@@ -1285,7 +1285,7 @@ cudaError_t part_drift_deposit(const PartParams& pp, float* sx, float* sy, float
         pp, sx, sy, sz, vx, vy, vz, ax, ay, az, dpx, dpy, dpz, rho, dt, m, mix, g_dep_box);
     return cudaGetLastError();
   }
-  const bool dep = dependent_launch(m, pp.Np, kDepParticles);
+  const bool dep = dependent_launch(m, pp.Np, kDepParticles, s);
   return launch_pdl(dep, dep ? k_drift_deposit<true> : k_drift_deposit<false>, dim3(blocks_for(P), m.nb), NTP, 0, s,
                     pp, sx, sy, sz, vx, vy, vz, ax, ay, az, dpx, dpy, dpz, rho, dt, P, m, mix);
 }
@@ -1303,7 +1303,7 @@ cudaError_t part_gather_kick(const PartParams& pp, const float* sx, const float*
         pp, sx, sy, sz, vx, vy, vz, ax, ay, az, Ax, Ay, Az, F0, F1, Fz, dt, m, mix, g_gk_box);
     return cudaGetLastError();
   }
-  const bool dep = dependent_launch(m, pp.Np, kDepParticles);
+  const bool dep = dependent_launch(m, pp.Np, kDepParticles, s);
   auto k = dep ? (pairs ? k_gather_kick<true, true> : k_gather_kick<false, true>)
                : (pairs ? k_gather_kick<true, false> : k_gather_kick<false, false>);
   return launch_pdl(dep, k, dim3((unsigned)((P + NTP * PPT - 1) / (NTP * PPT)), m.nb), NTP, 0, s, pp, sx, sy, sz, vx,
@@ -1333,7 +1333,7 @@ cudaError_t part_kick_drift_deposit(const PartParams& pp, float* sx, float* sy, 
     return launch_pdl(D, k, dim3((unsigned)((P + NTP * Q - 1) / (NTP * Q)), m.nb), NTP, 0, s, pp, sx, sy, sz, vx, vy,
                       vz, Ax, Ay, Az, dpx, dpy, dpz, F0, F1, Fz, rho, hdr, P, m, mix);
   };
-  return dependent_launch(m, pp.Np, kDepParticles) ? launch(std::true_type{}) : launch(std::false_type{});
+  return dependent_launch(m, pp.Np, kDepParticles, s) ? launch(std::true_type{}) : launch(std::false_type{});
 }
 
 cudaError_t part_snapshot(const PartParams& pp, const float* sx, const float* sy, const float* sz,
