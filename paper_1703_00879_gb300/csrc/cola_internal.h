@@ -160,19 +160,32 @@ inline bool dependent_launch(const Multi& m, int side, int most, cudaStream_t s)
   return cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
 }
 
+// keep_l1: the kernel's CTAs go to SMs that give all of the unified memory to L1.
 template <class... P, class... A>
-cudaError_t launch_pdl(bool dep, void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... a) {
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch_with(bool dep, bool keep_l1, void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
+                        A... a) {
+  cudaLaunchAttribute at[2]{};
+  int n = 0;
+  if (dep) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (keep_l1) {
+    at[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at[n++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxL1;
+  }
   cudaLaunchConfig_t c{};
   c.gridDim = grid;
   c.blockDim = dim3(threads);
   c.dynamicSmemBytes = smem;
   c.stream = s;
-  c.attrs = &at;
-  c.numAttrs = dep ? 1 : 0;
+  c.attrs = at;
+  c.numAttrs = n;
   return cudaLaunchKernelEx(&c, k, P(a)...);
+}
+template <class... P, class... A>
+cudaError_t launch_pdl(bool dep, void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... a) {
+  return launch_with(dep, false, k, grid, threads, smem, s, a...);
 }
 
 // Parameters of the per-k LPT reweight (Sec. 4.1): table of float4 per log-k node.

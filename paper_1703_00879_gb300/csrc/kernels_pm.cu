@@ -1273,6 +1273,16 @@ void set_particle_plan(int deposit_box, int gather_box) {
   g_gk_box = std::max(0, std::min(gather_box, kMaxGatherBox)) & ~3;
 }
 
+// The particle kernels use no shared memory and live on L1 (the mesh rows and lattice rows that
+// neighbouring threads share).  The four small CTAs per SM of the z passes leave little of it,
+// and a particle kernel whose CTAs join them, of another run's chain or of the launch before, ran
+// with what was left.  Asking for all of it keeps the two apart.  Twelve 64^3 / 128^3 runs on
+// eight chains, us for one step of each: 950 with the larger z CTAs, 1120 with the small ones, 860
+// so; eight steps of one such run 1015 -> 846 us.  On smaller meshes most of a force component
+// fits what is left and the change of an SM's split costs more: ten steps at 32^3 / 32^3 310 us
+// against 322, steps at 64^3 / 64^3 58.0 against 59.2 us.
+inline bool keep_l1(int Nm) { return Nm >= 128; }
+
 cudaError_t part_drift_deposit(const PartParams& pp, float* sx, float* sy, float* sz, float* vx,
                                float* vy, float* vz, const float* ax, const float* ay,
                                const float* az, const float* dpx, const float* dpy,
@@ -1286,7 +1296,7 @@ cudaError_t part_drift_deposit(const PartParams& pp, float* sx, float* sy, float
     return cudaGetLastError();
   }
   const bool dep = dependent_launch(m, pp.Np, kDepParticles, s);
-  return launch_pdl(dep, dep ? k_drift_deposit<true> : k_drift_deposit<false>, dim3(blocks_for(P), m.nb), NTP, 0, s,
+  return launch_with(dep, keep_l1(pp.Nm), dep ? k_drift_deposit<true> : k_drift_deposit<false>, dim3(blocks_for(P), m.nb), NTP, 0, s,
                     pp, sx, sy, sz, vx, vy, vz, ax, ay, az, dpx, dpy, dpz, rho, dt, P, m, mix);
 }
 
@@ -1306,7 +1316,7 @@ cudaError_t part_gather_kick(const PartParams& pp, const float* sx, const float*
   const bool dep = dependent_launch(m, pp.Np, kDepParticles, s);
   auto k = dep ? (pairs ? k_gather_kick<true, true> : k_gather_kick<false, true>)
                : (pairs ? k_gather_kick<true, false> : k_gather_kick<false, false>);
-  return launch_pdl(dep, k, dim3((unsigned)((P + NTP * PPT - 1) / (NTP * PPT)), m.nb), NTP, 0, s, pp, sx, sy, sz, vx,
+  return launch_with(dep, keep_l1(pp.Nm), k, dim3((unsigned)((P + NTP * PPT - 1) / (NTP * PPT)), m.nb), NTP, 0, s, pp, sx, sy, sz, vx,
                     vy, vz, ax, ay, az, Ax, Ay, Az, F0, F1, Fz, dt, P, m, mix);
 }
 
@@ -1330,7 +1340,7 @@ cudaError_t part_kick_drift_deposit(const PartParams& pp, float* sx, float* sy, 
     constexpr bool D = decltype(dep)::value;
     auto k = mix.on ? (pairs ? k_kick_drift_deposit<Q, 4, true, true, D> : k_kick_drift_deposit<Q, 4, false, true, D>)
                     : (pairs ? k_kick_drift_deposit<Q, 4, true, false, D> : k_kick_drift_deposit<Q, 4, false, false, D>);
-    return launch_pdl(D, k, dim3((unsigned)((P + NTP * Q - 1) / (NTP * Q)), m.nb), NTP, 0, s, pp, sx, sy, sz, vx, vy,
+    return launch_with(D, keep_l1(pp.Nm), k, dim3((unsigned)((P + NTP * Q - 1) / (NTP * Q)), m.nb), NTP, 0, s, pp, sx, sy, sz, vx, vy,
                       vz, Ax, Ay, Az, dpx, dpy, dpz, F0, F1, Fz, rho, hdr, P, m, mix);
   };
   return dependent_launch(m, pp.Np, kDepParticles, s) ? launch(std::true_type{}) : launch(std::false_type{});

@@ -53,7 +53,7 @@ def test_every_dependent_launch_has_a_kernel_that_waits():
     launched = set()
     for f in CSRC.glob("*.cu"):
         text = re.sub(r"//[^\n]*", "", f.read_text())
-        for m in re.finditer(r"launch_pdl\(", text):
+        for m in re.finditer(r"launch_(?:pdl|with)\(", text):
             head = text[max(0, text.rfind("\ncudaError_t", 0, m.start()), text.rfind("\nstatic cudaError_t", 0, m.start())):text.index(";", m.end())]
             launched |= set(re.findall(r"\bk_\w+", head)) - {"k_drift_deposit_box", "k_gather_kick_box"}
     assert launched and launched == set(KERNELS)
