@@ -1043,9 +1043,12 @@ __global__ void __launch_bounds__(NTP) k_pos_deposit(int Nm, float cellscale,
 // (the power as a float pair: the sum and the exact rounding error of each
 // addition, recovered from the value the atomic returns), and the launch's bins
 // in double at the end: |k| with a relative error ~1e-15.  The bin logic is a serial chain
-// per mode, so the values of PKU modes are loaded before it: bound by the latency of those
-// loads, P(k) and snapshot of 256^3 / 512^3 3.21 -> 3.02 ms with 4 at a time (6: 3.02, 12: 3.04).
-constexpr int PKU = 4;  // modes loaded ahead (below)
+// per mode, so the values of U modes are loaded before it.  U = 4 where the latency of those loads
+// bounds the pass, one mesh of 256 points and more: P(k) and snapshot of 256^3 / 512^3 3.21 ->
+// 3.02 ms (6: 3.02, 12: 3.04).  Many meshes at once hide it, and a longer body only costs
+// instructions: 128 meshes of 128^3 3.33 ms with U = 1, 3.36, 3.39, 3.42 with 2, 3, 4; 64 of 64^3
+// 320 us with 1 and 2, 330, 337; 16 of 256^3 3.29 ms with 1, 2.87, 2.92, 2.95.
+template <int U>
 __global__ void __launch_bounds__(NTP) k_pk_bin(const float2* __restrict__ dk, int N,
                                                 int64_t P, int nbins,
                                                 double* __restrict__ acc, double norm, Multi m,
@@ -1100,13 +1103,13 @@ __global__ void __launch_bounds__(NTP) k_pk_bin(const float2* __restrict__ dk, i
     };
     const int x0 = lane * K, x1 = min(x0 + K, H);
     bool more = true;
-    for (int xb = x0; xb < x1 && more; xb += PKU) {
-      float2 vv[PKU];  // the loads of PKU modes before the serial bin logic
+    for (int xb = x0; xb < x1 && more; xb += U) {
+      float2 vv[U];  // the loads of U modes before the serial bin logic
 #pragma unroll
-      for (int j = 0; j < PKU; ++j)
+      for (int j = 0; j < U; ++j)
         if (xb + j < x1) vv[j] = dk[hidx(iz, iy, xb + j, N, P)];
 #pragma unroll
-      for (int j = 0; j < PKU; ++j) {
+      for (int j = 0; j < U; ++j) {
         const int ix = xb + j;
         if (ix >= x1 || !more) continue;
         const int q = ix * ix + c;  // |n|^2 < 2^24 for N <= 4096
@@ -1447,14 +1450,17 @@ cudaError_t pk_bin(int N, const float2* dk, int nbins, double* acc, double norm,
   if (N > 4096 || sm > 200 * 1024) return cudaErrorInvalidValue;  // |n|^2 in 24 bits
   static bool attr = false;
   if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(k_pk_bin, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
+    for (auto k : {k_pk_bin<1>, k_pk_bin<2>, k_pk_bin<4>}) {
+      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      if (e != cudaSuccess) return e;
+    }
     attr = true;
   }
   const int64_t rows = (int64_t)N * N, wpb = NTP / 32;
   unsigned grid = (unsigned)std::min<int64_t>((rows + wpb - 1) / wpb, 152 * 8);
   if (m.nb > 1) grid = std::max<unsigned>(1, grid / (unsigned)std::min(m.nb, 8));
-  k_pk_bin<<<dim3(grid, m.nb), NTP, sm, s>>>(dk, N, half_pitch(N), nbins, acc, norm, m, acc_stride);
+  auto k = N <= 128 ? k_pk_bin<1> : m.nb > 1 ? k_pk_bin<2> : k_pk_bin<4>;
+  k<<<dim3(grid, m.nb), NTP, sm, s>>>(dk, N, half_pitch(N), nbins, acc, norm, m, acc_stride);
   return cudaGetLastError();
 }
 
