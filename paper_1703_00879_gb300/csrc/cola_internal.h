@@ -141,12 +141,13 @@ __device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_d
 // Which launches of one simulation are dependent: each kernel by the side of the arrays it works on,
 // transform passes and plane passes up to 128 points, particle passes up to 64^3 particles; the
 // step counter always.  Ten steps of the 32^3 f(R) run 513 -> 309 us, eight steps at 64^3 / 128^3
-// 1036 -> 1005 us.  Lattice and mesh of different sizes, us per nDGP step, so / only where
-// both are small: 128^3 / 128^3 197 / 205, 128^3 / 256^3 534 / 539, 32^3 / 256^3 402 / 408, 256^3 /
-// 128^3 1113 / 1117.  Beyond these sizes, and over several simulations, the waiting CTAs cost
-// more than they hide: a 256-member batch pass 64.9 ms without and 66.6 with them, 512^3 / 1024^3
-// 139.4 and 140.1.  The step counter of a large run hides its launch behind the particle pass: five
-// steps at 256^3 on the scale-independent path 5.00 ms so and 5.08 without pdl_go there.
+// 1036 -> 1005 us (845 with keep_l1, beside part_drift_deposit).  Lattice and mesh of different
+// sizes, us per nDGP step, by this rule / with dependent launches only where both are small:
+// 128^3 / 128^3 197 / 205, 128^3 / 256^3 534 / 539, 32^3 / 256^3 402 / 408, 256^3 / 128^3 1113 / 1117.
+// Beyond these sizes, and over several simulations, the waiting CTAs cost more than they hide: a
+// 256-member batch pass 64.9 ms without and 66.6 with them, 512^3 / 1024^3 139.4 and 140.1.  The
+// step counter of a large run hides its launch behind the particle pass: five steps at 256^3 on the
+// scale-independent path 5.00 ms so and 5.08 without pdl_go there.
 //
 // In a CUDA graph the launch gaps are short, and only the shortest kernels gain: launches that are
 // being captured (a Batch whose runs are launched one by one) are dependent up to 32 points.
